@@ -4,7 +4,7 @@
 // Every triangle carries the 16 points of the 4x4 Gauss-Legendre product rule
 // on the collapsed parent triangle (xi = (1 - eta) s, Jacobian (1 - eta) 2A_k);
 // they are point sources of strength 8 pi mu w q(xi, eta) summed by the
-// ordinary local-sum kernel.  For a target node z, the triangles having z as a
+// ordinary local-sum kernel (FP64 plans; ggem_elem32.cu holds the FP32 form).  For a target node z, the triangles having z as a
 // vertex need the polar rule instead (Sec. 3.4.1): the local-sum kernel skips
 // their regular points, and the correction kernel adds the same 4x4 rule in
 // polar coordinates (rho, theta) about z, with n-tilde = n_tri phi1 +
@@ -28,11 +28,10 @@ template <> __device__ __forceinline__ float e_rsqrt<float>(float x) { return rs
 template <> __device__ __forceinline__ double e_rsqrt<double>(double x) { return rsqrt(x); }
 
 // quadrature-point generation: one thread per (triangle, point)
-template <typename T>
 __global__ void k_qp_gen(int m, const double* __restrict__ x, const int* __restrict__ tri,
                          const double* __restrict__ tri_area, QuadRule rule,
                          double* __restrict__ xq, int4* __restrict__ qv,
-                         v4_t<T>* __restrict__ qw) {
+                         double4_32a* __restrict__ qw) {
     int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= m * 16) return;
     int k = e >> 4, a = e & 3, c = (e >> 2) & 3;
@@ -43,64 +42,32 @@ __global__ void k_qp_gen(int m, const double* __restrict__ x, const int* __restr
     for (int d = 0; d < 3; ++d)
         xq[3 * e + d] = p1 * x[3 * i1 + d] + p2 * x[3 * i2 + d] + p3 * x[3 * i3 + d];
     qv[e] = make_int4(i1, i2, i3, 0);
-    v4_t<T> w;
-    w.x = (T)(p1 * wt); w.y = (T)(p2 * wt); w.z = (T)(p3 * wt); w.w = (T)0;
+    double4_32a w;
+    w.x = p1 * wt; w.y = p2 * wt; w.z = p3 * wt; w.w = 0.0;
     qw[e] = w;
 }
 
 // strengths of the sorted quadrature points: g = scale * sum_v (phi_v w) q_v,
-// from the vertex indices and weights already in point order (qv, qw), into
-// interleaved v4 (g); in T throughout (q is the nodal density in T, so FP32
-// plans spend no FP64 instruction here -- GB300 runs FP64 at 1/64 of the FP32
-// rate)
-template <typename T>
-__device__ __forceinline__ void qp_strength_of(int s, const int4* __restrict__ qv,
-                                               const v4_t<T>* __restrict__ qw,
-                                               const T* __restrict__ q, T scale, T& rx, T& ry,
-                                               T& rz) {
-    const int4 v = qv[s];
-    const v4_t<T> w = qw[s];
-    const T a = scale * w.x, b = scale * w.y, c = scale * w.z;
-    rx = a * q[3 * v.x] + b * q[3 * v.y] + c * q[3 * v.z];
-    ry = a * q[3 * v.x + 1] + b * q[3 * v.y + 1] + c * q[3 * v.z + 1];
-    rz = a * q[3 * v.x + 2] + b * q[3 * v.y + 2] + c * q[3 * v.z + 2];
-}
-
-template <typename T>
-__global__ void k_qp_strength(int n, const int4* __restrict__ qv, const v4_t<T>* __restrict__ qw,
-                              const T* __restrict__ q, T scale, v4_t<T>* __restrict__ g) {
+// from the vertex indices and weights already in point order (qv, qw)
+__global__ void k_qp_strength(int n, const int4* __restrict__ qv,
+                              const double4_32a* __restrict__ qw, const double* __restrict__ q,
+                              double scale, double4_32a* __restrict__ g) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
-    v4_t<T> r;
-    qp_strength_of<T>(s, qv, qw, q, scale, r.x, r.y, r.z);
-    r.w = (T)0;
+    const int4 v = qv[s];
+    const double4_32a w = qw[s];
+    const double a = scale * w.x, b = scale * w.y, c = scale * w.z;
+    double4_32a r;
+    r.x = a * q[3 * v.x] + b * q[3 * v.y] + c * q[3 * v.z];
+    r.y = a * q[3 * v.x + 1] + b * q[3 * v.y + 1] + c * q[3 * v.z + 1];
+    r.z = a * q[3 * v.x + 2] + b * q[3 * v.y + 2] + c * q[3 * v.z + 2];
+    r.w = 0.0;
     g[s] = r;
 }
 
-// The same for the FP32 element rule, straight into the packed point layout:
-// one thread per pair of slots h (slots 2h, 2h + 1; inv maps a slot to its
-// sorted point, -1 for a dummy, whose strength stays zero), writing gx, gy, gz
-// of both as three 8-byte pairs at floats 6, 8, 10 of the pair's 12
-__global__ void k_qp_strength_pack(long npairs, const int* __restrict__ inv,
-                                   const int4* __restrict__ qv, const float4* __restrict__ qw,
-                                   const float* __restrict__ q, float scale,
-                                   float* __restrict__ pack) {
-    const long h = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (h >= npairs) return;
-    const int s0 = inv[2 * h], s1 = inv[2 * h + 1];
-    float x0 = 0.f, y0 = 0.f, z0 = 0.f, x1 = 0.f, y1 = 0.f, z1 = 0.f;
-    if (s0 >= 0) qp_strength_of<float>(s0, qv, qw, q, scale, x0, y0, z0);
-    if (s1 >= 0) qp_strength_of<float>(s1, qv, qw, q, scale, x1, y1, z1);
-    float2* o = reinterpret_cast<float2*>(pack + 12 * h + 6);
-    o[0] = make_float2(x0, x1);
-    o[1] = make_float2(y0, y1);
-    o[2] = make_float2(z0, z1);
-}
-
 // out[s] = in[perm[s]] (the quadrature weights into point order)
-template <typename T>
-__global__ void k_gather_v4(int n, const int* __restrict__ perm, const v4_t<T>* __restrict__ in,
-                            v4_t<T>* __restrict__ out) {
+__global__ void k_gather_v4(int n, const int* __restrict__ perm,
+                            const double4_32a* __restrict__ in, double4_32a* __restrict__ out) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n) out[s] = in[perm[s]];
 }
@@ -252,14 +219,9 @@ QuadRule make_quad_rule() {
     return r;
 }
 
-template <typename T>
-cudaError_t elem_setup(int m, const double* x, const int* tri, const double* tri_area,
-                       const QuadRule& rule, double* xq, int4* qv, v4_t<T>* qw, int nnodes,
-                       int* adj_cnt, int* adj_start, int* adj_cur, int* adj,
-                       cudaStream_t st) {
+cudaError_t tri_adjacency(int m, const int* tri, int nnodes, int* adj_cnt, int* adj_start,
+                          int* adj_cur, int* adj, cudaStream_t st) {
     if (m <= 0) return cudaSuccess;
-    if (xq)      // quadrature points (element rule only); the adjacency always
-        k_qp_gen<T><<<(m * 16 + 255) / 256, 256, 0, st>>>(m, x, tri, tri_area, rule, xq, qv, qw);
     cudaMemsetAsync(adj_cnt, 0, nnodes * sizeof(int), st);
     cudaMemsetAsync(adj_cur, 0, nnodes * sizeof(int), st);
     k_adj_count<<<(m + 255) / 256, 256, 0, st>>>(m, tri, adj_cnt);
@@ -268,37 +230,25 @@ cudaError_t elem_setup(int m, const double* x, const int* tri, const double* tri
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t qp_sort_weights(int nq, const int* perm, v4_t<T>* qw, v4_t<T>* tmp, cudaStream_t st) {
+cudaError_t qp_points(int m, const double* x, const int* tri, const double* tri_area,
+                      const QuadRule& rule, double* xq, int4* qv, double4_32a* qw,
+                      cudaStream_t st) {
+    if (m > 0)
+        k_qp_gen<<<(m * 16 + 255) / 256, 256, 0, st>>>(m, x, tri, tri_area, rule, xq, qv, qw);
+    return cudaGetLastError();
+}
+
+cudaError_t qp_sort_weights(int nq, const int* perm, double4_32a* qw, double4_32a* tmp,
+                            cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
-    k_gather_v4<T><<<(nq + 255) / 256, 256, 0, st>>>(nq, perm, qw, tmp);
-    return cudaMemcpyAsync(qw, tmp, (size_t)nq * sizeof(v4_t<T>), cudaMemcpyDeviceToDevice, st);
+    k_gather_v4<<<(nq + 255) / 256, 256, 0, st>>>(nq, perm, qw, tmp);
+    return cudaMemcpyAsync(qw, tmp, (size_t)nq * sizeof(double4_32a), cudaMemcpyDeviceToDevice,
+                           st);
 }
 
-__global__ void k_density_f32(long n, const double* __restrict__ q, float* __restrict__ out) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) out[e] = (float)q[e];
-}
-
-template <typename T>
-cudaError_t qp_strengths(int nq, const int4* qv, const v4_t<T>* qw, int nnodes, const double* q,
-                         T* qT, double scale, v4_t<T>* g, T* pack, const int* inv, long nslots,
-                         cudaStream_t st) {
-    if constexpr (sizeof(T) == 8) {
-        (void)qT;
-        (void)pack;
-        (void)inv;
-        (void)nslots;
-        if (nq > 0) k_qp_strength<T><<<(nq + 255) / 256, 256, 0, st>>>(nq, qv, qw, q, scale, g);
-    } else {
-        if (!qT || !pack || !inv) return cudaErrorInvalidValue;
-        const long ne = 3L * nnodes;
-        if (ne > 0) k_density_f32<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(ne, q, qT);
-        const long npairs = nslots / 2;
-        if (npairs > 0)
-            k_qp_strength_pack<<<(unsigned)((npairs + 255) / 256), 256, 0, st>>>(
-                npairs, inv, qv, qw, qT, (float)scale, pack);
-    }
+cudaError_t qp_strengths(int nq, const int4* qv, const double4_32a* qw, const double* q,
+                         double scale, double4_32a* g, cudaStream_t st) {
+    if (nq > 0) k_qp_strength<<<(nq + 255) / 256, 256, 0, st>>>(nq, qv, qw, q, scale, g);
     return cudaGetLastError();
 }
 
@@ -315,13 +265,6 @@ cudaError_t elem_correct(int n, int layer, const GridGeom& geo, const double* x,
 }
 
 #define GGEM_INST_ELEM(T)                                                                     \
-    template cudaError_t elem_setup<T>(int, const double*, const int*, const double*,          \
-                                       const QuadRule&, double*, int4*, v4_t<T>*, int, int*,    \
-                                       int*, int*, int*, cudaStream_t);                         \
-    template cudaError_t qp_sort_weights<T>(int, const int*, v4_t<T>*, v4_t<T>*, cudaStream_t); \
-    template cudaError_t qp_strengths<T>(int, const int4*, const v4_t<T>*, int, const double*, \
-                                         T*, double, v4_t<T>*, T*, const int*, long,           \
-                                         cudaStream_t);                                        \
     template cudaError_t elem_correct<T>(int, int, const GridGeom&, const double*, const int*, \
                                          const double*, const double*, const int*, const int*,  \
                                          const T*, const QuadRule&, T*, int, cudaStream_t);

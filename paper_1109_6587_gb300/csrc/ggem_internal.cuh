@@ -75,6 +75,38 @@ template <typename T> struct SortedSources {
     int n;
 };
 
+// locate a point: cell coordinates and offsets from the cell corner
+__device__ __forceinline__ void locate(const GridGeom& geo, const CellGrid& cg, double x,
+                                       double y, double z, int& cx, int& cy, int& cz,
+                                       double& ox, double& oy, double& oz) {
+    double xw = x - geo.Lx * floor(x / geo.Lx);
+    double zw = z - geo.Lz * floor(z / geo.Lz);
+    double yr = y - cg.y0;
+    cx = min(max((int)(xw / cg.hx), 0), cg.ncx - 1);
+    cz = min(max((int)(zw / cg.hz), 0), cg.ncz - 1);
+    cy = min(max((int)floor(yr / cg.hy), 0), cg.ncy - 1);
+    ox = xw - cx * cg.hx;
+    oy = yr - cy * cg.hy;
+    oz = zw - cz * cg.hz;
+}
+
+// FP32 element rule: point lists per quadrature rule of the triangles, binned
+// by centroid (ggem_elem32.cu).  Cells at least r_cut / kElemReach wide.
+constexpr int kElemLists = 2, kElemReach = 3;
+struct ElemLists32 {
+    int* tri_start = nullptr;             // [ncell + 1] sorted triangles of each cell
+    int4* tv = nullptr;                   // [m] sorted triangles: vertices, 2A (float bits)
+    double* shift = nullptr;              // [m][3] point position -> offset from the cell corner
+    int* sstart[kElemLists] = {};         // [ncell + 1] first 64-point step of each cell
+    int4* map[kElemLists] = {};           // per step: its cell's triangles, first point
+    int nsteps[kElemLists] = {};
+    float4* pack = nullptr;               // [steps][3][32]: the lists one after the other
+    int4* vert = nullptr;                 // [4 steps of list 0] vertices of each 16-slot group
+    int* nstart = nullptr;                // [ncell + 1] neighbour list of each target cell
+    int4* nbr = nullptr;                  // its entries
+    double far = 0.0;                     // distance of a cell from which it uses list 1
+};
+
 // 4x4 Gauss-Legendre product rule on [0,1]^2 and the polar-rule angles
 struct QuadRule {
     double t[4], w[4];                // nodes and weights on [0,1]
@@ -156,7 +188,7 @@ struct ggem_plan {
     int4* d_sdi = nullptr;             // spreading descriptors of free sources
     void* d_sdf = nullptr;
 
-    // element quadrature (16 points per triangle)
+    // element quadrature (16 points per triangle; FP64 plans but for the rule, n_qp, near_edge)
     ggem::QuadRule rule;
     int cap_qp = 0, n_qp = 0;
     double* d_qx = nullptr;            // [cap_qp][3] point positions
@@ -233,11 +265,16 @@ struct ggem_plan {
     bool ff = false;                   // element-rule local sum in double-float arithmetic
     void* d_qp_ff = nullptr;           // [cap_qp][2] float4: sorted point offsets, hi / lo
     void* d_qg_ff = nullptr;           // [cap_qp][2] float4: sorted point strengths, hi / lo
-    float* d_qp_pack = nullptr;        // [6 soa_ld] FP32 plans: packed point offsets and strengths
-    size_t soa_ld = 0;                 // slots of the packed layout: padded size + 64, a multiple of 64
-    long qp_np = 0;                    // slots in use (the padded size, even)
-    int* d_qp_pstart = nullptr;        // [ncell + 1] FP32 plans: padded cell starts
-    int* d_qp_inv = nullptr;           // [soa_ld] padded slot -> sorted point, -1 for dummies
+    // FP32 element rule: point lists of the triangles
+    ggem::ElemLists32 el;
+    size_t nbr_cap = 0;                // entries that el.nbr holds
+    size_t step_cap = 0;               // steps that el.pack holds,
+    size_t step_cap_l[ggem::kElemLists] = {};  // and el.map (el.vert: list 0)
+    double* d_et_cen = nullptr;        // triangles: centroids, cell / perm (unordered, ordered) / offsets
+    int* d_et_cell = nullptr;
+    int* d_et_perm = nullptr;
+    int* d_et_perm2 = nullptr;
+    float4* d_et_pos = nullptr;
     float* d_q32 = nullptr;            // [cap][3] FP32 plans: the density in FP32
     int* d_orec = nullptr;             // [4 cap][2] overlap records: particle pair
     double* d_orecd = nullptr;         // [4 cap] overlap records: node gap
@@ -316,36 +353,41 @@ cudaError_t local_sum(const GridGeom& geo, const CellGrid& cg, const SortedSourc
                       const double* nrm_tgt, int out_mode, T* out, int out_stride,
                       cudaStream_t st);
 
-// element rule: local sum over sorted quadrature points at the sorted mesh
-// nodes tgt (output in caller order), skipping points of triangles that
-// contain the target (only tested when closer than `near`); layer 0
-// velocity, 1 double layer
-// aux_pos / aux_g: FP32, the structure-of-arrays planes of the sorted points
-// (x, y, z, stride aux_ld; required); FP64, float-pair copies selecting the
-// double-float kernel (nullptr: native FP64)
-template <typename T>
-cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg, const SortedSources<T>& src,
-                           const int4* qvs, double near, const SortedSources<T>& tgt,
-                           const double* nrm_tgt, int layer, T* out, int out_stride,
-                           cudaStream_t st, const void* aux_pos = nullptr,
-                           const void* aux_g = nullptr, size_t aux_ld = 0,
-                           const int* aux_inv = nullptr);
-// FP32 element rule, padded and packed layout of the sorted points (each cell
-// from a multiple of 64, whole 64-point steps, dummies of zero strength far
-// away; 12 floats per slot pair: x0 x1 y0 y1 z0 z1 gx0 gx1 gy0 gy1 gz0 gz1):
-// padded counts and starts (pcnt: ncell scratch, pstart: ncell + 1), then the
-// np slots of pack (np even; dummies at 1e4, strengths zero), the positions
-// (scaled by alpha sqrt(log2 e), the local-sum kernel's units), and the map
-// slot -> sorted point (inv, -1 for dummies)
-cudaError_t pad_layout_counts(int ncell, const int* start, int* pcnt, int* pstart,
-                              cudaStream_t st);
-cudaError_t pad_layout_fill(int n, size_t np, const int* cell, const int* start,
-                            const int* pstart, const float4* pos, double alpha, float* pack,
-                            int* inv, cudaStream_t st);
-// FP32 element rule: sub-sort the sorted points within each cell (4 x 4 x 4
-// sub-cells in Morton order; tmp_* of n entries as scratch)
-cudaError_t cell_subsort(const CellGrid& cg, int n, int ncell, const int* start, float4* pos,
-                         int* perm, float4* tmp_pos, int* tmp_perm, cudaStream_t st);
+// FP64 element rule: local sum over sorted quadrature points at the sorted
+// mesh nodes tgt (output in caller order), skipping points of triangles that
+// contain the target (only tested when closer than `near`); layer 0 velocity,
+// 1 double layer.  ff_pos / ff_g: float-pair copies of the points selecting
+// the double-float kernel (nullptr: native FP64)
+cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg,
+                           const SortedSources<double>& src, const int4* qvs, double near,
+                           const SortedSources<double>& tgt, const double* nrm_tgt, int layer,
+                           double* out, int out_stride, cudaStream_t st,
+                           const void* ff_pos = nullptr, const void* ff_g = nullptr);
+// FP32 element rule (ggem_elem32.cu).  At mesh_set: triangle centroids cen
+// (binned by build_cells into tri_start / pos / perm), then the order within
+// the cells (perm_out; fills tv, shift), the steps per cell (scratch: ncell
+// ints; fills sstart), and, with the lists allocated, their points.  Per
+// evaluation: the strengths (q32: the density in FP32), then the sum at the
+// sorted mesh nodes (near: no triangle around a target has a longer edge).
+cudaError_t elem32_centroids(int m, const double* x, const int* tri, double* cen,
+                             cudaStream_t st);
+cudaError_t elem32_order(const GridGeom& geo, const CellGrid& cg, int m, const ElemLists32& L,
+                         const float4* pos, const int* perm, int* perm_out, const double* cen,
+                         const int* tri, const double* tri_area, cudaStream_t st);
+cudaError_t elem32_steps(const ElemLists32& L, int ncell, int* scratch, cudaStream_t st);
+// neighbour lists of the cells with targets (tgt_start): counts (scratch: ncell
+// ints; fills nstart), or with `fill` the entries
+cudaError_t elem32_neighbours(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
+                              const int* tgt_start, int* scratch, bool fill, cudaStream_t st);
+cudaError_t elem32_fill(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
+                        const QuadRule& rule, const double* x, cudaStream_t st);
+cudaError_t elem32_strengths(const ElemLists32& L, const QuadRule& rule, int nnodes,
+                             const double* q, float* q32, double scale, cudaStream_t st);
+cudaError_t elem32_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
+                       double near, const SortedSources<float>& tgt, const double* nrm, int layer,
+                       float* out, int out_stride, cudaStream_t st);
+// distance of a cell from which the FP32 element rule uses list 1
+double elem32_far_distance(double near_edge);
 // float-pair copy of n double4 (x, y, z, w) values: out[2 i] = hi, out[2 i + 1] = lo
 cudaError_t to_float_pairs(int n, const void* in, void* out, cudaStream_t st);
 cudaError_t gather_int4(int n, const int* perm, const int4* in, int4* out, cudaStream_t st);
@@ -354,22 +396,21 @@ cudaError_t gather_int4(int n, const int* perm, const int4* in, int4* out, cudaS
 cudaError_t scan_counts(int n, const int* count, int* start, cudaStream_t st);
 
 QuadRule make_quad_rule();
-// quadrature points of m triangles and the node -> triangle adjacency
-template <typename T>
-cudaError_t elem_setup(int m, const double* x, const int* tri, const double* tri_area,
-                       const QuadRule& rule, double* xq, int4* qv, v4_t<T>* qw, int nnodes,
-                       int* adj_cnt, int* adj_start, int* adj_cur, int* adj, cudaStream_t st);
-// quadrature weights qw into point order, qw[s] <- qw[perm[s]] (tmp: nq v4 T)
-template <typename T>
-cudaError_t qp_sort_weights(int nq, const int* perm, v4_t<T>* qw, v4_t<T>* tmp, cudaStream_t st);
+// node -> triangle adjacency of m triangles
+cudaError_t tri_adjacency(int m, const int* tri, int nnodes, int* adj_cnt, int* adj_start,
+                          int* adj_cur, int* adj, cudaStream_t st);
+// FP64 element rule: quadrature points of m triangles, their vertices and
+// weights
+cudaError_t qp_points(int m, const double* x, const int* tri, const double* tri_area,
+                      const QuadRule& rule, double* xq, int4* qv, double4_32a* qw,
+                      cudaStream_t st);
+// quadrature weights qw into point order, qw[s] <- qw[perm[s]] (tmp: nq)
+cudaError_t qp_sort_weights(int nq, const int* perm, double4_32a* qw, double4_32a* tmp,
+                            cudaStream_t st);
 // sorted point strengths g = scale sum_v (phi_v w) q_v from the sorted vertex
-// indices and weights, in T: FP64 plans into g (v4); FP32 plans copy the
-// nnodes x 3 density q into qT, then fill the strengths of the nslots slots of
-// the packed layout (pad_layout_fill; inv: slot -> sorted point)
-template <typename T>
-cudaError_t qp_strengths(int nq, const int4* qv, const v4_t<T>* qw, int nnodes, const double* q,
-                         T* qT, double scale, v4_t<T>* g, T* pack, const int* inv, long nslots,
-                         cudaStream_t st);
+// indices and weights
+cudaError_t qp_strengths(int nq, const int4* qv, const double4_32a* qw, const double* q,
+                         double scale, double4_32a* g, cudaStream_t st);
 // polar-rule correction of the local part at the mesh nodes (layer 0 single, 1 double);
 // q: the nodal density in T
 template <typename T>

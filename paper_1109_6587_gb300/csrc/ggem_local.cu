@@ -8,8 +8,6 @@
 // +-R cells carries the image; as r_cut < L/2 (Sec. 3.2.2, alpha L > 8), at
 // most one image of a source lies within r_cut even where a small grid
 // visits a cell twice.
-#include <type_traits>
-
 #include "ggem_internal.cuh"
 #include "ggem_erfcx.cuh"
 #include "ggem_ff.cuh"
@@ -25,21 +23,6 @@ template <> __device__ __forceinline__ float d_rsqrt<float>(float x) {
     return y;
 }
 template <> __device__ __forceinline__ double d_rsqrt<double>(double x) { return rsqrt(x); }
-
-// locate a point: cell coordinates and offsets from the cell corner
-__device__ __forceinline__ void locate(const GridGeom& geo, const CellGrid& cg, double x,
-                                       double y, double z, int& cx, int& cy, int& cz,
-                                       double& ox, double& oy, double& oz) {
-    double xw = x - geo.Lx * floor(x / geo.Lx);
-    double zw = z - geo.Lz * floor(z / geo.Lz);
-    double yr = y - cg.y0;
-    cx = min(max((int)(xw / cg.hx), 0), cg.ncx - 1);
-    cz = min(max((int)(zw / cg.hz), 0), cg.ncz - 1);
-    cy = min(max((int)floor(yr / cg.hy), 0), cg.ncy - 1);
-    ox = xw - cx * cg.hx;
-    oy = yr - cy * cg.hy;
-    oz = zw - cz * cg.hz;
-}
 
 __global__ void k_cell_count(GridGeom geo, CellGrid cg, int n, const double* __restrict__ x,
                              int* __restrict__ count, int* __restrict__ cell_of) {
@@ -158,9 +141,6 @@ cudaError_t gather_strengths(int n, const int* perm, const double* q, const doub
 template <typename T> struct LocalConst {
     T al, al2, rc2, c1, c2, c3, c4, fU, fS, hx, hy, hz;
     T ke;   // -alpha^2 log2(e): exp(-alpha^2 r^2) = 2^(ke r^2)
-    // FP32 element rule (scaled coordinates, set by local_sum_elem): the
-    // coordinate scale s, the reciprocal's slope P alpha / s, and -6 s^3
-    T sc = (T)1, pt = (T)0, c6 = (T)-6;
 };
 
 template <typename T> LocalConst<T> local_const(const GridGeom& geo, const CellGrid& cg) {
@@ -190,7 +170,6 @@ template <typename T> struct LocalArgs {
     const double* nrm;       // OUT_DBL: [n][3] target normals (caller order)
     T* out;
     int out_stride;
-    const int* qinv = nullptr;   // FP32 element rule: padded slot -> sorted point (-1: dummy)
 };
 
 // Locate targets once (one thread each, FP64): cell index and offsets from
@@ -294,72 +273,6 @@ __device__ __forceinline__ void pair_terms(const LocalConst<T>& k, T dx, T dy, T
     }
 }
 
-// Two candidate pairs at once, FP32 (element rule): the arithmetic of
-// pair_terms on paired lanes (add/mul/fma .f32x2), so one issued instruction
-// serves two pairs; rsqrt and exp2 stay scalar.  Every multiply-add is an
-// explicit FMA.
-struct PairAcc2 {
-    f2 ux = {0ull}, uy = {0ull}, uz = {0ull};
-    f2 sn = {0ull};     // double layer: sum of E x.g (times the target normal at the end)
-};
-
-__device__ __forceinline__ float rsqrt_ftz(float x) {
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float ex2_ftz(float x) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// In the FP32 element rule the coordinates are scaled by s = alpha sqrt(log2 e)
-// (local_sum_elem), so exp(-alpha^2 r^2) = 2^(-r_s^2) takes no multiply; the
-// displacements, r and 1/r below are in scaled units, and the constants
-// (c1 / s, c2 s^2, -6 s^3, the output factor s or 1 / s) make every term the
-// unscaled one.
-template <int MODE>
-__device__ __forceinline__ void pair_terms2(const LocalConst<float>& k, f2 dx, f2 dy, f2 dz,
-                                            f2 r2, f2 gx, f2 gy, f2 gz, f2 nx, f2 ny, f2 nz,
-                                            PairAcc2& a) {
-    float lo, hi;
-    f2_split(r2, lo, hi);
-    const f2 ir = f2_make(rsqrt_ftz(lo), rsqrt_ftz(hi));
-    const f2 ex = f2_make(ex2_ftz(-lo), ex2_ftz(-hi));               // exp(-alpha^2 r^2)
-    const f2 r = r2 * ir;
-    f2_split(fma2(r, f2_splat(k.pt), f2_splat(1.0f)), lo, hi);
-    const f2 t = f2_make(rcp_ftz(lo), rcp_ftz(hi));                 // 1/(1 + P alpha r)
-    const f2 ec = ex * erfcx_t2(t);                                  // erfc(alpha r)
-    const f2 xg = fma2(dz, gz, fma2(dy, gy, dx * gx));
-    if (MODE & OUT_U) {
-        // A = ec/r - c1 ex,  B = (ec/r^3 + c1 ex/r^2) xg
-        const f2 eir = ec * ir;
-        const f2 A = fma2(f2_splat(-k.c1), ex, eir);
-        const f2 B = (ir * ir) * fma2(f2_splat(k.c1), ex, eir) * xg;
-        a.ux = fma2(B, dx, fma2(A, gx, a.ux));
-        a.uy = fma2(B, dy, fma2(A, gy, a.uy));
-        a.uz = fma2(B, dz, fma2(A, gz, a.uz));
-    }
-    if (MODE & OUT_DBL) {
-        // D = -6 ec/r^5 - c2 ex/r^4 - c3 ex/r^2 = ir2 (ir2 (-6 ec ir - c2 ex) - c3 ex),
-        // E = c4 ex; the update D xg xn d + E (d gn + g xn + n xg) regrouped as
-        // d (D xg xn + E gn) + g (E xn) + n (E xg), the last term's scalar E xg
-        // summed over the pairs and multiplied by the (fixed) target normal once
-        const f2 ir2 = ir * ir;
-        const f2 t = fma2(f2_splat(k.c6), ec * ir, f2_splat(-k.c2) * ex);
-        const f2 D = ir2 * fma2(ir2, t, f2_splat(-k.c3) * ex);
-        const f2 E = f2_splat(k.c4) * ex;
-        const f2 xn = fma2(dz, nz, fma2(dy, ny, dx * nx));
-        const f2 gn = fma2(gz, nz, fma2(gy, ny, gx * nx));
-        const f2 cd = fma2(D * xg, xn, E * gn), cg = E * xn;
-        a.sn = fma2(E, xg, a.sn);
-        a.ux = fma2(dx, cd, fma2(gx, cg, a.ux));
-        a.uy = fma2(dy, cd, fma2(gy, cg, a.uy));
-        a.uz = fma2(dz, cd, fma2(gz, cg, a.uz));
-    }
-}
-
 // scaled output of one target in caller order
 template <typename T, int MODE>
 __device__ __forceinline__ void store_target(const LocalConst<T>& k, const PairAcc<T>& a, T* o) {
@@ -449,60 +362,6 @@ __device__ __forceinline__ int cull_cells(const LocalArgs<T>& a, int lane, T ox,
     return nc;
 }
 
-// The same culling in batches: rounds of 32 neighbour offsets from *round
-// on, stopping before a round could overflow `cap` entries; *round is left at
-// the first round not culled (nb rounds = done).  Bit 15 of s_off marks the
-// cells within near2 of the target (the only ones that can hold points of
-// the triangles around it).
-template <typename T, int R>
-__device__ __forceinline__ int cull_cells_batch(const LocalArgs<T>& a, int lane, T ox, T oy,
-                                                T oz, int cx, int cy, int cz, int* s_cst,
-                                                int* s_cnt, unsigned short* s_off, int& round,
-                                                int cap) {
-    const CellGrid& cg = a.cg;
-    const unsigned lt = (1u << lane) - 1u;
-    const T reach2 = a.k.rc2 * (T)1.0001;
-    constexpr int side = 2 * R + 1, nb = side * side * side, nr = (nb + 31) / 32;
-    int nc = 0;
-    for (; round < nr && nc + 32 <= cap; ++round) {
-        const int oi = round * 32 + lane;
-        bool keep = false, nearc = false;
-        int st = 0, cnt = 0;
-        if (oi < nb) {
-            const int ix = oi % side - R, iy = (oi / side) % side - R, iz = oi / (side * side) - R;
-            const int cyy = cy + iy;
-            if (cyy >= 0 && cyy < cg.ncy) {
-                const T gx = ix > 0 ? (T)ix * a.k.hx - ox : (ix < 0 ? ox - (T)(ix + 1) * a.k.hx : (T)0);
-                const T gy = iy > 0 ? (T)iy * a.k.hy - oy : (iy < 0 ? oy - (T)(iy + 1) * a.k.hy : (T)0);
-                const T gz = iz > 0 ? (T)iz * a.k.hz - oz : (iz < 0 ? oz - (T)(iz + 1) * a.k.hz : (T)0);
-                const T d2 = gx * gx + gy * gy + gz * gz;
-                nearc = d2 <= a.near2 * (T)1.0001;
-                if (d2 <= reach2) {
-                    int cxx = cx + ix, czz = cz + iz;
-                    cxx += (cxx < 0) ? cg.ncx : 0;
-                    cxx -= (cxx >= cg.ncx) ? cg.ncx : 0;
-                    czz += (czz < 0) ? cg.ncz : 0;
-                    czz -= (czz >= cg.ncz) ? cg.ncz : 0;
-                    const int c = (czz * cg.ncy + cyy) * cg.ncx + cxx;
-                    st = a.src.cell_start[c];
-                    cnt = a.src.cell_start[c + 1] - st;
-                    keep = cnt > 0;
-                }
-            }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (keep) {
-            const int slot = nc + __popc(m & lt);
-            s_cst[slot] = st;
-            s_cnt[slot] = cnt;
-            s_off[slot] = (unsigned short)(oi | (nearc ? 0x8000 : 0));
-        }
-        nc += __popc(m);
-    }
-    __syncwarp();
-    return nc;
-}
-
 // u_i = sum G^l_ij g_j ; sigma_ik = sum T^l_ijk g_j ; v_i = n_k sigma_ik
 // (unscaled in the loop; the caller-facing factors are applied at the end).
 //
@@ -518,7 +377,7 @@ constexpr int kNb = 7 * 7 * 7;   // neighbour cell offsets for the largest reach
 // ELEM: sources are element quadrature points and targets are mesh nodes
 // (caller index t); points of triangles having the target as a vertex are
 // skipped (their integral is done by the polar rule, Sec. 3.4.1).  Used in
-// FP64; the FP32 element rule runs in k_local_elem32 below.
+// FP64; the FP32 element rule has a kernel of its own (k_local_elem32).
 template <typename T, int KIND, int MODE, bool ELEM, int REACH>
 __global__ void __launch_bounds__(LW * 32) k_local(LocalArgs<T> a) {
     __shared__ int s_cst[LW][kNb];            // this target's cells: first source,
@@ -633,164 +492,6 @@ __global__ void __launch_bounds__(LW * 32) k_local(LocalArgs<T> a) {
         return;
     }
     store_target<T, MODE>(a.k, acc, a.out + (size_t)oidx * a.out_stride);
-}
-
-// ------------------------------------------------- FP32 element rule
-// The element-rule local sum in FP32 reads ~700 quadrature points per cell
-// and finds about 80 % of them within r_cut, so no hit queue: every lane
-// takes two adjacent candidates of each 64-point step through a cell and
-// evaluates both with paired FP32 arithmetic.  The points are read from a
-// packed copy, 48 bytes per pair of adjacent points (x0 x1 y0 y1 | z0 z1 gx0
-// gx1 | gy0 gy1 gz0 gz1), so a lane's two candidates arrive with three 16-byte
-// loads, every coordinate already paired; the layout is padded: each cell
-// starts on a multiple of 64 points and fills whole steps with dummies of zero
-// strength far away, so a step needs no bounds test.
-// Candidates beyond r_cut are evaluated unmasked: their terms carry
-// exp(-alpha^2 r^2) <= e^-16 (and erfc(alpha r) <= 1.6e-8), below the FP32
-// rounding of the sum, and a step with no candidate within r_cut is skipped.
-// Points of the triangles around the target (left to the singular
-// correction) can only lie in the cells the culling marks near; only there
-// is each candidate within near2 checked and, if excluded, given zero strength.
-constexpr int LWE = 4;        // warps (targets) per block; 10 blocks per SM (48 registers)
-constexpr int kCap = 128;     // culled cells per batch (a target may need several batches)
-constexpr int kChunk = 64;    // candidates per warp step
-
-template <int MODE, int REACH>
-__global__ void __launch_bounds__(LWE * 32, 10) k_local_elem32(LocalArgs<float> a,
-                                                          const float4* __restrict__ pk) {
-    __shared__ int s_cst[LWE][kCap];
-    __shared__ int s_cnt[LWE][kCap];
-    __shared__ unsigned short s_off[LWE][kCap];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = blockIdx.x * LWE + wid;
-    if (t >= a.n_tgt) return;                     // warp-uniform
-    int cx, cy, cz, oidx;
-    float ox, oy, oz;
-    load_target<float, TK_POINTS>(a, t, ox, oy, oz, cx, cy, cz, oidx);
-    ox *= a.k.sc;                                 // scaled coordinates (set by local_sum_elem)
-    oy *= a.k.sc;
-    oz *= a.k.sc;
-    constexpr int R = REACH, side = 2 * R + 1;
-    float nx = 0.f, ny = 0.f, nz = 0.f;
-    if (MODE & OUT_DBL) {
-        nx = (float)a.nrm[3 * oidx]; ny = (float)a.nrm[3 * oidx + 1]; nz = (float)a.nrm[3 * oidx + 2];
-    }
-    const f2 nx2 = f2_splat(nx), ny2 = f2_splat(ny), nz2 = f2_splat(nz);
-    const float rc2 = a.k.rc2;
-    PairAcc2 acc;
-    for (int round = 0; round < (side * side * side + 31) / 32;) {
-    const int nc = cull_cells_batch<float, R>(a, lane, ox, oy, oz, cx, cy, cz, s_cst[wid],
-                                              s_cnt[wid], s_off[wid], round, kCap);
-    for (int ci = 0; ci < nc; ++ci) {
-        const int st = s_cst[wid][ci], end = st + s_cnt[wid][ci];
-        const int oi = s_off[wid][ci] & 0x7fff;
-        const bool nearc = s_off[wid][ci] >> 15;
-        // target position in the frame of this source cell's corner
-        const f2 tx = f2_splat(ox - (float)(oi % side - R) * a.k.hx);
-        const f2 ty = f2_splat(oy - (float)((oi / side) % side - R) * a.k.hy);
-        const f2 tz = f2_splat(oz - (float)(oi / (side * side) - R) * a.k.hz);
-        // one 64-point step; NEAR: check for points of the target's own triangles
-        auto step = [&](int i0, auto near_tag) {
-            constexpr bool NEAR = decltype(near_tag)::value;
-            const int i = i0 + 2 * lane;          // even: candidates i and i + 1
-            const int h = i >> 1;
-            // positions and strengths in one go (the strengths before the test,
-            // so their latency overlaps the distance arithmetic)
-            const float4 pa = pk[3 * h], pb = pk[3 * h + 1], pc = pk[3 * h + 2];
-            const f2 dx = tx - f2_make(pa.x, pa.y), dy = ty - f2_make(pa.z, pa.w),
-                     dz = tz - f2_make(pb.x, pb.y);
-            const f2 r2 = fma2(dz, dz, fma2(dy, dy, dx * dx));
-            float r0, r1;
-            float2 wx = make_float2(pb.z, pb.w), wy = make_float2(pc.x, pc.y),
-                   wz = make_float2(pc.z, pc.w);
-            f2_split(r2, r0, r1);
-            if (!__any_sync(0xffffffffu, r0 < rc2 || r1 < rc2)) return;
-            if (NEAR) {
-                if (r0 < a.near2) {
-                    const int s = a.qinv[i];
-                    if (s >= 0) {
-                        const int4 v = a.qvs[s];
-                        if (v.x == oidx || v.y == oidx || v.z == oidx) wx.x = wy.x = wz.x = 0.f;
-                    }
-                }
-                if (r1 < a.near2) {
-                    const int s = a.qinv[i + 1];
-                    if (s >= 0) {
-                        const int4 v = a.qvs[s];
-                        if (v.x == oidx || v.y == oidx || v.z == oidx) wx.y = wy.y = wz.y = 0.f;
-                    }
-                }
-            }
-            pair_terms2<MODE>(a.k, dx, dy, dz, r2, f2_make(wx.x, wx.y), f2_make(wy.x, wy.y),
-                              f2_make(wz.x, wz.y), nx2, ny2, nz2, acc);
-        };
-        if (nearc) {
-            for (int i0 = st; i0 < end; i0 += kChunk) step(i0, std::true_type{});
-        } else {
-            for (int i0 = st; i0 < end; i0 += kChunk) step(i0, std::false_type{});
-        }
-    }
-    __syncwarp();
-    }
-    float ux = f2_sum(acc.ux), uy = f2_sum(acc.uy), uz = f2_sum(acc.uz);
-    if (MODE & OUT_DBL) {
-        const float sn = f2_sum(acc.sn);
-        ux = fmaf(nx, sn, ux);
-        uy = fmaf(ny, sn, uy);
-        uz = fmaf(nz, sn, uz);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ux += __shfl_xor_sync(0xffffffffu, ux, o);
-        uy += __shfl_xor_sync(0xffffffffu, uy, o);
-        uz += __shfl_xor_sync(0xffffffffu, uz, o);
-    }
-    if (lane == 0) {
-        float* o = a.out + (size_t)oidx * a.out_stride;
-        o[0] = a.k.fU * ux;
-        o[1] = a.k.fU * uy;
-        o[2] = a.k.fU * uz;
-    }
-}
-
-// Order of the sorted points within each cell: 4 x 4 x 4 sub-cells in Morton
-// order, so that consecutive points (the 64-point steps of the FP32 element
-// rule) lie close together.  One block per cell; a counting sort by the 6-bit
-// key into pos_out / perm_out.
-__device__ __forceinline__ int subcell_key(float4 p, float ihx, float ihy, float ihz) {
-    const int ix = min(3, max(0, (int)(p.x * ihx))), iy = min(3, max(0, (int)(p.y * ihy))),
-              iz = min(3, max(0, (int)(p.z * ihz)));
-    return (ix & 1) | ((iy & 1) << 1) | ((iz & 1) << 2) | ((ix & 2) << 2) | ((iy & 2) << 3) |
-           ((iz & 2) << 4);
-}
-
-__global__ void k_cell_subsort(const int* __restrict__ start, const float4* __restrict__ pos,
-                               const int* __restrict__ perm, float ihx, float ihy, float ihz,
-                               float4* __restrict__ pos_out, int* __restrict__ perm_out) {
-    __shared__ int cnt[64];
-    const int c = blockIdx.x;
-    const int st = start[c], n = start[c + 1] - st;
-    if (n == 0) return;                          // block-uniform
-    if (threadIdx.x < 64) cnt[threadIdx.x] = 0;
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x)
-        atomicAdd(&cnt[subcell_key(pos[st + i], ihx, ihy, ihz)], 1);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int k = 0; k < 64; ++k) {
-            const int v = cnt[k];
-            cnt[k] = run;
-            run += v;
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float4 p = pos[st + i];
-        const int slot = st + atomicAdd(&cnt[subcell_key(p, ihx, ihy, ihz)], 1);
-        pos_out[slot] = p;
-        perm_out[slot] = perm[st + i];
-    }
 }
 
 // ----------------------------------- element rule, FP64-accurate in float pairs
@@ -1012,155 +713,41 @@ static void launch_kind(const LocalArgs<T>& a, int mode, cudaStream_t st) {
     else launch_kind<T, KIND, 2>(a, mode, st);
 }
 
-// Within-cell sub-sort of sorted points (pos, perm); tmp_* of n entries as scratch.
-cudaError_t cell_subsort(const CellGrid& cg, int n, int ncell, const int* start, float4* pos,
-                         int* perm, float4* tmp_pos, int* tmp_perm, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    k_cell_subsort<<<ncell, 256, 0, st>>>(start, pos, perm, (float)(4.0 / cg.hx),
-                                          (float)(4.0 / cg.hy), (float)(4.0 / cg.hz), tmp_pos,
-                                          tmp_perm);
-    cudaMemcpyAsync(pos, tmp_pos, (size_t)n * sizeof(float4), cudaMemcpyDeviceToDevice, st);
-    cudaMemcpyAsync(perm, tmp_perm, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, st);
-    return cudaGetLastError();
-}
-
-// Padded, packed layout of the sorted points for the FP32 element rule: each
-// cell's points start on a multiple of 64 and fill whole 64-point steps; slot
-// pair h holds 12 floats x0 x1 y0 y1 z0 z1 gx0 gx1 gy0 gy1 gz0 gz1 (slots 2h,
-// 2h + 1); the slots after a cell's last point hold dummies (offset 1e4 from
-// the cell corner, strength zero), whose terms are exactly zero.
-__global__ void k_pad_counts(int ncell, const int* __restrict__ start, int* __restrict__ pcnt) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < ncell) pcnt[c] = (start[c + 1] - start[c] + 63) & ~63;
-}
-
-__global__ void k_pad_fill(size_t npairs, float4* __restrict__ pack) {
-    const size_t h = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (h >= npairs) return;
-    pack[3 * h] = make_float4(1e4f, 1e4f, 1e4f, 1e4f);
-    pack[3 * h + 1] = make_float4(1e4f, 1e4f, 0.f, 0.f);
-    pack[3 * h + 2] = make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
-__global__ void k_pad_scatter(int n, const int* __restrict__ cell, const int* __restrict__ start,
-                              const int* __restrict__ pstart, const float4* __restrict__ pos,
-                              float sc, float* __restrict__ pack, int* __restrict__ inv) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const int c = cell[s];
-    const int p = pstart[c] + (s - start[c]);
-    const float4 v = pos[s];
-    float* o = pack + 12 * (size_t)(p >> 1) + (p & 1);
-    o[0] = v.x * sc;
-    o[2] = v.y * sc;
-    o[4] = v.z * sc;
-    inv[p] = s;
-}
-
-cudaError_t pad_layout_counts(int ncell, const int* start, int* pcnt, int* pstart,
-                              cudaStream_t st) {
-    if (ncell <= 0) return cudaSuccess;
-    k_pad_counts<<<(ncell + 255) / 256, 256, 0, st>>>(ncell, start, pcnt);
-    return scan_counts(ncell, pcnt, pstart, st);
-}
-
-float elem32_scale(double alpha) { return (float)(alpha * 1.2011224087864498); }
-
-cudaError_t pad_layout_fill(int n, size_t np, const int* cell, const int* start,
-                            const int* pstart, const float4* pos, double alpha, float* pack,
-                            int* inv, cudaStream_t st) {
-    if (np > 0) {
-        const size_t npairs = np / 2;
-        k_pad_fill<<<(unsigned)((npairs + 255) / 256), 256, 0, st>>>(npairs, (float4*)pack);
-        cudaMemsetAsync(inv, 0xff, np * sizeof(int), st);
-    }
-    if (n > 0)
-        k_pad_scatter<<<(n + 255) / 256, 256, 0, st>>>(n, cell, start, pstart, pos,
-                                                      elem32_scale(alpha), pack, inv);
-    return cudaGetLastError();
-}
-
 cudaError_t to_float_pairs(int n, const void* in, void* out, cudaStream_t st) {
     if (n > 0)
         k_to_float_pairs<<<(n + 255) / 256, 256, 0, st>>>(n, (const double*)in, (float4*)out);
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg, const SortedSources<T>& src,
-                           const int4* qvs, double near, const SortedSources<T>& tgt,
-                           const double* nrm_tgt, int layer, T* out, int out_stride,
-                           cudaStream_t st, const void* aux_pos, const void* aux_g,
-                           size_t aux_ld, const int* aux_inv) {
+cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg,
+                           const SortedSources<double>& src, const int4* qvs, double near,
+                           const SortedSources<double>& tgt, const double* nrm_tgt, int layer,
+                           double* out, int out_stride, cudaStream_t st, const void* ff_pos,
+                           const void* ff_g) {
     if (tgt.n <= 0) return cudaSuccess;
     // targets: the mesh nodes in cell order, so the warps of a block mostly
     // scan the same candidate cells (L1 reuse); output in caller order
-    LocalArgs<T> a{geo, cg, local_const<T>(geo, cg), src, qvs, (T)(near * near), tgt.n,
-                   tgt.cell, tgt.pos, tgt.perm, nrm_tgt, out, out_stride};
-    if constexpr (sizeof(T) == 4) {
-        (void)aux_g;
-        (void)aux_ld;
-        if (!aux_pos || !aux_inv) return cudaErrorInvalidValue;
-        a.qinv = aux_inv;
-        // scaled coordinates: lengths times s = alpha sqrt(log2 e), the
-        // packed points scaled likewise at mesh_set (pad_layout_fill)
-        {
-            const double sc = (double)elem32_scale(geo.alpha);
-            LocalConst<float>& k = a.k;
-            k.sc = (float)sc;
-            k.hx = (float)(cg.hx * sc);
-            k.hy = (float)(cg.hy * sc);
-            k.hz = (float)(cg.hz * sc);
-            k.rc2 = (float)(geo.rcut * geo.rcut * sc * sc);
-            a.near2 = (float)(near * near * sc * sc);
-            k.pt = (float)(GGEM_ERFCX_P * geo.alpha / sc);
-            k.c1 = (float)(2.0 * geo.alpha / 1.7724538509055160273 / sc);
-            k.c2 = (float)(12.0 * geo.alpha / 1.7724538509055160273 * sc * sc);
-            k.c6 = (float)(-6.0 * sc * sc * sc);
-            k.fU = (float)(layer == 0 ? sc : 1.0 / sc) * k.fU;
-        }
-        const float4* pk = (const float4*)aux_pos;
-        dim3 b(LWE * 32), g((tgt.n + LWE - 1) / LWE);
-        // ~6 KB of shared memory per block, 10 blocks per SM: ask for a small
-        // shared-memory carveout (25 %: the 64 KB configuration) so that the
-        // rest of the SM's 256 KB serves as L1
-        // for the candidates the warps of a block re-read (a preference; cheap
-        // per launch)
-        const void* kf = layer == 0 ? (cg.reach == 3 ? (const void*)k_local_elem32<OUT_U, 3>
-                                                     : (const void*)k_local_elem32<OUT_U, 2>)
-                                    : (cg.reach == 3 ? (const void*)k_local_elem32<OUT_DBL, 3>
-                                                     : (const void*)k_local_elem32<OUT_DBL, 2>);
-        cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
+    LocalArgs<double> a{geo, cg, local_const<double>(geo, cg), src, qvs, near * near, tgt.n,
+                        tgt.cell, tgt.pos, tgt.perm, nrm_tgt, out, out_stride};
+    dim3 b(LW * 32), g((tgt.n + LW - 1) / LW);
+    if (ff_pos && ff_g) {
+        const float4* fp = (const float4*)ff_pos;
+        const float4* fg = (const float4*)ff_g;
         if (cg.reach == 3) {
-            if (layer == 0) k_local_elem32<OUT_U, 3><<<g, b, 0, st>>>(a, pk);
-            else k_local_elem32<OUT_DBL, 3><<<g, b, 0, st>>>(a, pk);
+            if (layer == 0) k_local_elem_ff<OUT_U, 3><<<g, b, 0, st>>>(a, fp, fg);
+            else k_local_elem_ff<OUT_DBL, 3><<<g, b, 0, st>>>(a, fp, fg);
         } else {
-            if (layer == 0) k_local_elem32<OUT_U, 2><<<g, b, 0, st>>>(a, pk);
-            else k_local_elem32<OUT_DBL, 2><<<g, b, 0, st>>>(a, pk);
+            if (layer == 0) k_local_elem_ff<OUT_U, 2><<<g, b, 0, st>>>(a, fp, fg);
+            else k_local_elem_ff<OUT_DBL, 2><<<g, b, 0, st>>>(a, fp, fg);
         }
         return cudaGetLastError();
     }
-    dim3 b(LW * 32), g((tgt.n + LW - 1) / LW);
-    if constexpr (sizeof(T) == 8) {
-        if (aux_pos && aux_g) {
-            const float4* fp = (const float4*)aux_pos;
-            const float4* fg = (const float4*)aux_g;
-            if (cg.reach == 3) {
-                if (layer == 0) k_local_elem_ff<OUT_U, 3><<<g, b, 0, st>>>(a, fp, fg);
-                else k_local_elem_ff<OUT_DBL, 3><<<g, b, 0, st>>>(a, fp, fg);
-            } else {
-                if (layer == 0) k_local_elem_ff<OUT_U, 2><<<g, b, 0, st>>>(a, fp, fg);
-                else k_local_elem_ff<OUT_DBL, 2><<<g, b, 0, st>>>(a, fp, fg);
-            }
-            return cudaGetLastError();
-        }
-    }
     if (cg.reach == 3) {
-        if (layer == 0) k_local<T, TK_POINTS, OUT_U, true, 3><<<g, b, 0, st>>>(a);
-        else k_local<T, TK_POINTS, OUT_DBL, true, 3><<<g, b, 0, st>>>(a);
+        if (layer == 0) k_local<double, TK_POINTS, OUT_U, true, 3><<<g, b, 0, st>>>(a);
+        else k_local<double, TK_POINTS, OUT_DBL, true, 3><<<g, b, 0, st>>>(a);
     } else {
-        if (layer == 0) k_local<T, TK_POINTS, OUT_U, true, 2><<<g, b, 0, st>>>(a);
-        else k_local<T, TK_POINTS, OUT_DBL, true, 2><<<g, b, 0, st>>>(a);
+        if (layer == 0) k_local<double, TK_POINTS, OUT_U, true, 2><<<g, b, 0, st>>>(a);
+        else k_local<double, TK_POINTS, OUT_DBL, true, 2><<<g, b, 0, st>>>(a);
     }
     return cudaGetLastError();
 }
@@ -1189,12 +776,7 @@ cudaError_t local_sum(const GridGeom& geo, const CellGrid& cg, const SortedSourc
                                       const v4_t<T>*, const double*, int, T*, int,             \
                                       cudaStream_t);                                           \
     template cudaError_t locate_targets<T>(const GridGeom&, const CellGrid&, int, int,        \
-                                           const double*, int*, v4_t<T>*, cudaStream_t);       \
-    template cudaError_t local_sum_elem<T>(const GridGeom&, const CellGrid&,                  \
-                                           const SortedSources<T>&, const int4*, double,        \
-                                           const SortedSources<T>&, const double*, int, T*, int, \
-                                           cudaStream_t, const void*, const void*, size_t, \
-                                           const int*);
+                                           const double*, int*, v4_t<T>*, cudaStream_t);
 GGEM_INST_LOCAL(float)
 GGEM_INST_LOCAL(double)
 

@@ -315,10 +315,11 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
     stage(P, ST_GATHER, elem ? 2 : 1, [&] {
         GG_CUDA(gather_strengths<T>(n, P->d_mesh_perm, q, P->d_area, 8.0 * kPi * geo.mu,
                                     (v4_t<T>*)P->d_sg, st));
-        if (elem)
-            GG_CUDA(qp_strengths<T>(P->n_qp, P->d_qv_sorted, (const v4_t<T>*)P->d_qw, n, q,
-                                    (T*)P->d_q32, 8.0 * kPi * geo.mu, (v4_t<T>*)P->d_qg,
-                                    (T*)P->d_qp_pack, P->d_qp_inv, P->qp_np, st));
+        if (elem && !P->fp64)
+            GG_CUDA(elem32_strengths(P->el, P->rule, n, q, P->d_q32, 8.0 * kPi * geo.mu, st));
+        if (elem && P->fp64)
+            GG_CUDA(qp_strengths(P->n_qp, P->d_qv_sorted, (const double4_32a*)P->d_qw, q,
+                                 8.0 * kPi * geo.mu, (double4_32a*)P->d_qg, st));
         if (elem && P->ff) GG_CUDA(to_float_pairs(P->n_qp, P->d_qg, P->d_qg_ff, st));
     });
     SortedSources<T> src = sources_of<T>(P, true);
@@ -351,18 +352,21 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
     } else {
         // local part by the element rule: all quadrature points, then the polar
         // rule on the triangles that touch each node (Sec. 3.4.1, 3.5.2)
-        SortedSources<T> qs;
-        qs.pos = (v4_t<T>*)P->d_qp_pos;
-        qs.g = (v4_t<T>*)P->d_qg;
-        qs.cell = P->d_qp_cell;
-        qs.perm = P->d_qp_perm;
-        qs.cell_start = P->fp64 ? P->d_qp_start : P->d_qp_pstart;   // FP32: padded layout
-        qs.n = P->n_qp;
         stage(P, ST_LOCAL, 1, [&] {
-            GG_CUDA(local_sum_elem<T>(geo, P->cg, qs, P->d_qv_sorted, 1.01 * P->near_edge, src,
-                                      P->d_nrm, layer, loc, 3, ls,
-                                      P->fp64 ? P->d_qp_ff : (void*)P->d_qp_pack,
-                                      P->fp64 ? P->d_qg_ff : nullptr, P->soa_ld, P->d_qp_inv));
+            if constexpr (sizeof(T) == 4) {
+                GG_CUDA(elem32_sum(geo, P->cg, P->el, 1.01 * P->near_edge, src, P->d_nrm, layer,
+                                   loc, 3, ls));
+            } else {
+                SortedSources<double> qs;
+                qs.pos = (double4_32a*)P->d_qp_pos;
+                qs.g = (double4_32a*)P->d_qg;
+                qs.cell = P->d_qp_cell;
+                qs.perm = P->d_qp_perm;
+                qs.cell_start = P->d_qp_start;
+                qs.n = P->n_qp;
+                GG_CUDA(local_sum_elem(geo, P->cg, qs, P->d_qv_sorted, 1.01 * P->near_edge, src,
+                                       P->d_nrm, layer, loc, 3, ls, P->d_qp_ff, P->d_qg_ff));
+            }
         });
         stage(P, ST_ELEM, 1, [&] {
             GG_CUDA(elem_correct<T>(n, layer, geo, P->d_x, P->d_tri, P->d_tri_nrm, P->d_nrm,
@@ -697,24 +701,33 @@ void plan_build(ggem_plan_t* P, const ggem_params& prm) {
         size_t cq = (size_t)16 * prm.max_tris;
         GG_CHECK(cq < (size_t)1 << 31, GGEM_ERR_CAPACITY, "too many quadrature points");
         P->cap_qp = (int)cq;
-        dalloc(P, &P->d_qx, cq * 3);
-        dalloc(P, &P->d_qv, cq);
-        dalloc(P, &P->d_qv_sorted, cq);
-        GG_CUDA(cudaMalloc(&P->d_qw, cq * v4 + 32));
-        dalloc(P, &P->d_qp_cell, cq);
-        dalloc(P, &P->d_qp_perm, cq);
-        dalloc(P, &P->d_qp_start, (size_t)P->ncell + 1);
-        GG_CUDA(cudaMalloc(&P->d_qp_pos, cq * v4 + 32));
-        GG_CUDA(cudaMalloc(&P->d_qg, cq * v4 + 32));
-        if (P->ff) {                       // float-pair copies: [point][hi, lo] float4
-            GG_CUDA(cudaMalloc(&P->d_qp_ff, cq * 2 * sizeof(float4) + 32));
-            GG_CUDA(cudaMalloc(&P->d_qg_ff, cq * 2 * sizeof(float4) + 32));
-        }
-        if (!P->fp64) {                    // padded planes; grown at mesh_set if needed
-            P->soa_ld = (cq + cq / 8 + 64 + 63) / 64 * 64;
-            dalloc(P, &P->d_qp_pack, 6 * P->soa_ld);
-            dalloc(P, &P->d_qp_inv, P->soa_ld);
-            dalloc(P, &P->d_qp_pstart, (size_t)P->ncell + 1);
+        if (P->fp64) {
+            dalloc(P, &P->d_qx, cq * 3);
+            dalloc(P, &P->d_qv, cq);
+            dalloc(P, &P->d_qv_sorted, cq);
+            GG_CUDA(cudaMalloc(&P->d_qw, cq * v4 + 32));
+            dalloc(P, &P->d_qp_cell, cq);
+            dalloc(P, &P->d_qp_perm, cq);
+            dalloc(P, &P->d_qp_start, (size_t)P->ncell + 1);
+            GG_CUDA(cudaMalloc(&P->d_qp_pos, cq * v4 + 32));
+            GG_CUDA(cudaMalloc(&P->d_qg, cq * v4 + 32));
+            if (P->ff) {                   // float-pair copies: [point][hi, lo] float4
+                GG_CUDA(cudaMalloc(&P->d_qp_ff, cq * 2 * sizeof(float4) + 32));
+                GG_CUDA(cudaMalloc(&P->d_qg_ff, cq * 2 * sizeof(float4) + 32));
+            }
+        } else {
+            // the plan's cells (r_cut / 3); the lists are sized by mesh_set
+            const size_t nce = P->ncell, mt = prm.max_tris;
+            dalloc(P, &P->d_et_cen, 3 * mt);
+            dalloc(P, &P->d_et_cell, mt);
+            dalloc(P, &P->d_et_perm, mt);
+            dalloc(P, &P->d_et_perm2, mt);
+            dalloc(P, &P->d_et_pos, mt);
+            dalloc(P, &P->el.tri_start, nce + 1);
+            dalloc(P, &P->el.tv, mt);
+            dalloc(P, &P->el.shift, 3 * mt);
+            for (int l = 0; l < kElemLists; ++l) dalloc(P, &P->el.sstart[l], nce + 1);
+            dalloc(P, &P->el.nstart, nce + 1);
             dalloc(P, &P->d_q32, (size_t)3 * cap);
         }
     }
@@ -759,15 +772,77 @@ void plan_free(ggem_plan_t* P) {
                     P->d_pnodes, P->d_rc, P->d_rscale, P->d_mref, P->d_cx0, P->d_cdf,
                     P->d_cuinf, P->d_cfinf, P->d_cb, P->d_ckap, P->d_clam, P->d_cw, P->d_cq,
                     P->d_cmin, P->d_tstart, P->d_tlist, P->d_cvol, P->d_orec, P->d_orecd,
-                    P->d_ocount, P->d_odisp, P->d_qp_ff, P->d_qg_ff, P->d_qp_pack,
+                    P->d_ocount, P->d_odisp, P->d_qp_ff, P->d_qg_ff,
                     P->d_spec, P->d_spec_twx, P->d_spec_twz, P->d_spec_dx,
                     P->d_spec_dz, P->d_spec_mid, P->d_spec_ct, P->d_mlp_tc,
-                    P->d_mlp_tcs, P->d_qp_pstart, P->d_qp_inv, P->d_q32};
+                    P->d_mlp_tcs, P->d_q32, P->d_et_cen, P->d_et_cell,
+                    P->d_et_perm, P->d_et_perm2, P->d_et_pos, P->el.tri_start, P->el.tv,
+                    P->el.shift, P->el.sstart[0], P->el.sstart[1], P->el.map[0], P->el.map[1],
+                    P->el.pack, P->el.vert, P->el.nstart, P->el.nbr};
     for (void* p : ptrs) dfree(p);
     precond_free(P);
     dfree(P->d_pc_Zb);
     if (P->h_sh) cudaFreeHost(P->h_sh);
     if (P->twin) ggem_plan_destroy(P->twin);
+}
+
+// FP32 element rule: the triangles (by centroid) into the cells, then the
+// neighbour lists of the mesh nodes' cells and the point lists, grown where the mesh needs more steps than they
+// hold.  List 1 is built where cells beyond its distance are common: at 0.85
+// r_cut and more the few percent of points it would save cost as much again in
+// strengths.
+void elem32_mesh(ggem_plan_t* P, int m) {
+    cudaStream_t st = P->st;
+    ElemLists32& L = P->el;
+    GG_CUDA(elem32_centroids(m, P->d_x, P->d_tri, P->d_et_cen, st));
+    GG_CUDA(build_cells<float>(P->geo, P->cg, m, P->d_et_cen, P->d_cell_count, L.tri_start,
+                               P->d_cursor, P->d_et_cell, P->d_et_perm, P->d_et_pos, st));
+    GG_CUDA(elem32_order(P->geo, P->cg, m, L, P->d_et_pos, P->d_et_perm, P->d_et_perm2,
+                         P->d_et_cen, P->d_tri, P->d_tri_area, st));
+    GG_CUDA(elem32_steps(L, P->ncell, P->d_cell_count, st));
+    GG_CUDA(elem32_neighbours(P->geo, P->cg, L, P->d_mesh_start, P->d_cell_count, false, st));
+    int nnbr = 0;
+    GG_CUDA(cudaMemcpyAsync(&nnbr, L.nstart + P->ncell, sizeof(int), cudaMemcpyDeviceToHost,
+                            st));
+    for (int l = 0; l < kElemLists; ++l)
+        GG_CUDA(cudaMemcpyAsync(&L.nsteps[l], L.sstart[l] + P->ncell, sizeof(int),
+                                cudaMemcpyDeviceToHost, st));
+    GG_CUDA(cudaStreamSynchronize(st));
+    L.far = elem32_far_distance(P->near_edge);
+    if (!(L.far < 0.85 * P->geo.rcut)) L.nsteps[1] = 0;
+    size_t total = 0;
+    for (int l = 0; l < kElemLists; ++l) {
+        const size_t ns = L.nsteps[l];
+        total += ns;
+        if (ns > P->step_cap_l[l]) {
+            dfree(L.map[l]);
+            L.map[l] = nullptr;
+            if (l == 0) {
+                dfree(L.vert);
+                L.vert = nullptr;
+            }
+            P->step_cap_l[l] = 0;
+            dalloc(P, &L.map[l], ns + ns / 8);
+            if (l == 0) dalloc(P, &L.vert, 4 * (ns + ns / 8));
+            P->step_cap_l[l] = ns + ns / 8;
+        }
+    }
+    if (total > P->step_cap) {
+        dfree(L.pack);
+        L.pack = nullptr;
+        P->step_cap = 0;
+        dalloc(P, &L.pack, 96 * (total + total / 8));
+        P->step_cap = total + total / 8;
+    }
+    if ((size_t)nnbr > P->nbr_cap) {
+        dfree(L.nbr);
+        L.nbr = nullptr;
+        P->nbr_cap = 0;
+        dalloc(P, &L.nbr, (size_t)nnbr + nnbr / 8);
+        P->nbr_cap = (size_t)nnbr + nnbr / 8;
+    }
+    GG_CUDA(elem32_neighbours(P->geo, P->cg, L, P->d_mesh_start, nullptr, true, st));
+    GG_CUDA(elem32_fill(P->geo, P->cg, L, P->rule, P->d_x, st));
 }
 
 }  // namespace
@@ -890,21 +965,9 @@ ggem_status ggem_mesh_set(ggem_plan_t* P, int n_nodes, const double* x, int n_tr
         }
         const bool elem = P->prm.quadrature == GGEM_ELEMENT && n_tris > 0;
         if (n_tris > 0) {
-            // node -> triangle adjacency (element correction, ring features) and,
-            // in element-rule plans, the quadrature points
-            if (elem)
-                GG_CHECK(P->d_qx && P->d_qv && P->d_qw, GGEM_ERR_INVALID_ARG,
-                         "element buffers missing");
-            if (P->fp64)
-                GG_CUDA(elem_setup<double>(n_tris, P->d_x, P->d_tri, P->d_tri_area, P->rule,
-                                           elem ? P->d_qx : nullptr, P->d_qv,
-                                           (double4_32a*)P->d_qw, n_nodes, P->d_adj_cnt,
-                                           P->d_adj_start, P->d_adj_cur, P->d_adj, st));
-            else
-                GG_CUDA(elem_setup<float>(n_tris, P->d_x, P->d_tri, P->d_tri_area, P->rule,
-                                          elem ? P->d_qx : nullptr, P->d_qv, (float4*)P->d_qw,
-                                          n_nodes, P->d_adj_cnt, P->d_adj_start, P->d_adj_cur,
-                                          P->d_adj, st));
+            // node -> triangle adjacency (element correction, ring features)
+            GG_CUDA(tri_adjacency(n_tris, P->d_tri, n_nodes, P->d_adj_cnt, P->d_adj_start,
+                                  P->d_adj_cur, P->d_adj, st));
         }
         P->n_qp = 0;
         if (elem) {
@@ -916,48 +979,19 @@ ggem_status ggem_mesh_set(ggem_plan_t* P, int n_nodes, const double* x, int n_tr
             GG_CUDA(cudaStreamSynchronize(st));
             int nq = 16 * n_tris;
             if (P->fp64) {
+                GG_CUDA(qp_points(n_tris, P->d_x, P->d_tri, P->d_tri_area, P->rule, P->d_qx,
+                                  P->d_qv, (double4_32a*)P->d_qw, st));
                 GG_CUDA(build_cells<double>(P->geo, P->cg, nq, P->d_qx, P->d_cell_count,
                                             P->d_qp_start, P->d_cursor, P->d_qp_cell,
                                             P->d_qp_perm, (double4_32a*)P->d_qp_pos, st));
                 if (P->ff) GG_CUDA(to_float_pairs(nq, P->d_qp_pos, P->d_qp_ff, st));
+                GG_CUDA(gather_int4(nq, P->d_qp_perm, P->d_qv, P->d_qv_sorted, st));
+                // weights into point order too (scratch: the strength buffer)
+                GG_CUDA(qp_sort_weights(nq, P->d_qp_perm, (double4_32a*)P->d_qw,
+                                        (double4_32a*)P->d_qg, st));
             } else {
-                GG_CUDA(build_cells<float>(P->geo, P->cg, nq, P->d_qx, P->d_cell_count,
-                                           P->d_qp_start, P->d_cursor, P->d_qp_cell,
-                                           P->d_qp_perm, (float4*)P->d_qp_pos, st));
-                // within-cell order (scratch: the strength buffer and the cursors,
-                // both free until the first evaluation)
-                GG_CUDA(cell_subsort(P->cg, nq, P->ncell, P->d_qp_start, (float4*)P->d_qp_pos,
-                                     P->d_qp_perm, (float4*)P->d_qg, P->d_cursor, st));
-                // padded layout: whole 64-point steps per cell (the cursors as
-                // scratch for the padded counts); the planes grow if it needs more
-                GG_CUDA(pad_layout_counts(P->ncell, P->d_qp_start, P->d_cursor, P->d_qp_pstart,
-                                          st));
-                int np = 0;
-                GG_CUDA(cudaMemcpyAsync(&np, P->d_qp_pstart + P->ncell, sizeof(int),
-                                        cudaMemcpyDeviceToHost, st));
-                GG_CUDA(cudaStreamSynchronize(st));
-                if ((size_t)np + 64 > P->soa_ld) {
-                    dfree(P->d_qp_pack);
-                    dfree(P->d_qp_inv);
-                    P->d_qp_pack = nullptr;
-                    P->d_qp_inv = nullptr;
-                    P->soa_ld = ((size_t)np + (size_t)np / 8 + 64 + 63) / 64 * 64;
-                    dalloc(P, &P->d_qp_pack, 6 * P->soa_ld);
-                    dalloc(P, &P->d_qp_inv, P->soa_ld);
-                }
-                GG_CUDA(pad_layout_fill(nq, P->soa_ld, P->d_qp_cell, P->d_qp_start,
-                                        P->d_qp_pstart, (const float4*)P->d_qp_pos,
-                                        P->geo.alpha, P->d_qp_pack, P->d_qp_inv, st));
-                P->qp_np = np;
+                elem32_mesh(P, n_tris);
             }
-            GG_CUDA(gather_int4(nq, P->d_qp_perm, P->d_qv, P->d_qv_sorted, st));
-            // weights into point order too (scratch: the strength buffer)
-            if (P->fp64)
-                GG_CUDA(qp_sort_weights<double>(nq, P->d_qp_perm, (double4_32a*)P->d_qw,
-                                                (double4_32a*)P->d_qg, st));
-            else
-                GG_CUDA(qp_sort_weights<float>(nq, P->d_qp_perm, (float4*)P->d_qw,
-                                               (float4*)P->d_qg, st));
             P->n_qp = nq;
         }
         P->n_nodes = n_nodes;
