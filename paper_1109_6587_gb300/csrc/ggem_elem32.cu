@@ -193,8 +193,8 @@ __global__ void k_neighbours(CellGrid cg, float hx, float hy, float hz, float re
                     e.y = ss0[c + 1] - e.x;
                     keep = e.y > 0;
                     if (FILL && keep) {
-                        e.z = base1 + ss1[c];
-                        e.w = oi | ((ss1[c + 1] - ss1[c]) << 10);
+                        e.z = ss1 ? base1 + ss1[c] : 0;
+                        e.w = oi | (ss1 ? (ss1[c + 1] - ss1[c]) << 10 : 0);
                     }
                 }
             }
@@ -585,19 +585,21 @@ cudaError_t elem32_steps(const ElemLists32& L, int ncell, int* scratch, cudaStre
 }
 
 cudaError_t elem32_neighbours(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
-                              const int* tgt_start, int* scratch, bool fill, cudaStream_t st) {
+                              const int* tgt_start, const int* src_start, int* scratch,
+                              bool fill, cudaStream_t st) {
     const int ncell = cg.ncx * cg.ncy * cg.ncz;
     const float reach2 = (float)(geo.rcut * geo.rcut * 1.0002);
+    const int* ss0 = src_start ? src_start : L.sstart[0];
+    const int* ss1 = src_start ? nullptr : L.sstart[1];
     const unsigned nb = (unsigned)((ncell + 7) / 8);
     if (fill) {
         k_neighbours<true><<<nb, 256, 0, st>>>(cg, (float)cg.hx, (float)cg.hy, (float)cg.hz, reach2,
-                                              tgt_start, L.sstart[0], L.sstart[1], L.nsteps[0],
-                                              L.nstart, nullptr, L.nbr);
+                                              tgt_start, ss0, ss1, L.nsteps[0], L.nstart, nullptr,
+                                              L.nbr);
         return cudaGetLastError();
     }
     k_neighbours<false><<<nb, 256, 0, st>>>(cg, (float)cg.hx, (float)cg.hy, (float)cg.hz, reach2,
-                                           tgt_start, L.sstart[0], L.sstart[1], 0, nullptr,
-                                           scratch, nullptr);
+                                           tgt_start, ss0, ss1, 0, nullptr, scratch, nullptr);
     return scan_counts(ncell, scratch, L.nstart, st);
 }
 

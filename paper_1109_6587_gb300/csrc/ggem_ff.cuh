@@ -1,12 +1,16 @@
 // Double-float arithmetic: a value is the unevaluated sum hi + lo of two
-// floats with |lo| <= ulp(hi)/2, about 48 significant bits.  GB300 issues
-// FP64 at 1/64 of its FP32 rate, so FP64-accurate pair sums run faster in
-// float pairs than in doubles.  Built on Knuth's two-sum and the exact product
-// of a fused multiply-add (a*b - fl(a*b) = fma(a, b, -fl(a*b))); the addition
-// and multiplication follow the published double-double algorithms of Dekker
-// (1971) and Hida, Li and Bailey (2001), applied to float pairs.  Additions use
-// the short ("sloppy") form: the error is about 2^-44 of the larger operand,
-// which the pair sums tolerate (FP64 parity is checked at 1e-10).
+// floats, about 48 significant bits.  GB300 issues FP64 at 1/64 of its FP32
+// rate, so FP64-accurate pair sums run faster in float pairs than in doubles.
+// Built on Knuth's two-sum and the exact product of a fused multiply-add
+// (a*b - fl(a*b) = fma(a, b, -fl(a*b))), after Dekker (1971) and Hida, Li and
+// Bailey (2001).  Sums and products are left unnormalised -- lo up to a few
+// 2^-23 of the largest term, not half an ulp of hi -- as every operation takes
+// its operands' lo parts to first order anyway; the dropped lo * lo products
+// and the rounding of the lo parts are about 2^-46 of the largest term.  The
+// rounded products are __fmul_rn: a plain multiply could be contracted with the
+// addition that follows it, whose error term then counts twice.  The
+// renormalising steps (3 operations each) are kept where a value is compared,
+// accumulated over many pairs or fed to the reciprocal square root.
 #pragma once
 
 struct ff {
@@ -19,7 +23,6 @@ __device__ __forceinline__ ff ff_from_double(double x) {
     return {h, __double2float_rn(x - (double)h)};
 }
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
-__device__ __forceinline__ ff ff_of(float a) { return {a, 0.f}; }
 
 // s + e = a + b exactly (Knuth)
 __device__ __forceinline__ ff two_sum(float a, float b) {
@@ -32,70 +35,48 @@ __device__ __forceinline__ ff fast_two_sum(float a, float b) {
     const float s = a + b;
     return {s, b - (s - a)};
 }
-// p + e = a * b exactly
-__device__ __forceinline__ ff two_prod(float a, float b) {
-    const float p = a * b;
-    return {p, fmaf(a, b, -p)};
+__device__ __forceinline__ ff ff_norm(ff a) { return fast_two_sum(a.hi, a.lo); }
+__device__ __forceinline__ ff ff_mul(ff a, ff b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    return {p, fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, fmaf(a.hi, b.hi, -p)))};
+}
+__device__ __forceinline__ ff ff_sqr(ff a) {
+    const float p = __fmul_rn(a.hi, a.hi);
+    return {p, fmaf(a.hi, a.lo + a.lo, fmaf(a.hi, a.hi, -p))};
 }
 __device__ __forceinline__ ff ff_add(ff a, ff b) {
-    ff s = two_sum(a.hi, b.hi);
-    s.lo += a.lo + b.lo;
-    return fast_two_sum(s.hi, s.lo);
+    const ff s = two_sum(a.hi, b.hi);
+    return {s.hi, (a.lo + b.lo) + s.lo};
 }
-__device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ ff ff_sub(ff a, ff b) { return ff_add(a, ff_neg(b)); }
-__device__ __forceinline__ ff ff_add_f(ff a, float b) {
-    ff s = two_sum(a.hi, b);
-    s.lo += a.lo;
-    return fast_two_sum(s.hi, s.lo);
+__device__ __forceinline__ ff ff_sub(ff a, ff b) { return ff_add(a, {-b.hi, -b.lo}); }
+// a + b + c of products
+__device__ __forceinline__ ff ff_sum3(ff a, ff b, ff c) {
+    const ff s = two_sum(a.hi, b.hi), t = two_sum(s.hi, c.hi);
+    return {t.hi, ((a.lo + b.lo) + (c.lo + s.lo)) + t.lo};
 }
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-    ff p = two_prod(a.hi, b.hi);
-    p.lo = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, p.lo));
-    return fast_two_sum(p.hi, p.lo);
+__device__ __forceinline__ ff ff_dot(const ff* a, const ff* b) {
+    return ff_sum3(ff_mul(a[0], b[0]), ff_mul(a[1], b[1]), ff_mul(a[2], b[2]));
 }
-__device__ __forceinline__ ff ff_mul_f(ff a, float b) {
-    ff p = two_prod(a.hi, b);
-    p.lo = fmaf(a.lo, b, p.lo);
-    return fast_two_sum(p.hi, p.lo);
-}
-// a < b
-__device__ __forceinline__ bool ff_lt(ff a, ff b) {
-    return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo);
-}
+// acc += p, acc normalised
+__device__ __forceinline__ void ff_acc(ff& acc, ff p) { acc = ff_norm(ff_add(acc, p)); }
 
-// 1/sqrt(x), x > 0: the hardware estimate y (about 2^-23 relative) and one
-// Newton step y + y (1 - x y^2)/2 with the residual 1 - x y^2 formed in pairs
+// y = 1/sqrt(x), x > 0 normalised: the hardware estimate e (about 2^-22.4
+// relative) corrected by e r (1/2 + 3 r / 8), r = 1 - x e^2.  r and the
+// correction are themselves kept in pairs and y is normalised: 1/r^5 takes five
+// times y's error (8e-16 rms this way, 5e-15 with r and the correction as single
+// floats: 3 times the error of the pair terms for 12 operations of about 420).
 __device__ __forceinline__ ff ff_rsqrt(ff x) {
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x.hi));
-    const ff t = ff_mul(x, two_prod(y, y));
-    const ff e = ff_add_f(ff_neg(t), 1.0f);
-    return fast_two_sum(y, 0.5f * y * (e.hi + e.lo));
-}
-
-// exp(x) for -20 <= x <= 0.  Reduction x = (16 m + j) ln2/16 + f, |f| <=
-// ln2/32, exp(x) = 2^m 2^(j/16) exp(f); exp(f) = 1 + f + f^2/2 + f^3/6 in
-// pairs plus the tail f^4 (1/24 + f/120 + f^2/720 + f^3/5040) in float (the
-// tail is below 1e-8, its float rounding below 1e-15).  t2[j] = 2^(j/16),
-// ln2_16 = ln 2 / 16 and sixth = 1/6 as pairs.
-__device__ __forceinline__ ff ff_exp(ff x, const ff* t2, ff ln2_16, ff sixth) {
-    const float kf = rintf(x.hi * 23.083120654223414f);   // 16 / ln 2
-    const int k = (int)kf;
-    const int m = k >> 4, j = k - 16 * m;
-    ff kl = two_prod(kf, ln2_16.hi);
-    kl.lo = fmaf(kf, ln2_16.lo, kl.lo);
-    const ff f = ff_sub(x, kl);
-    const ff f2 = ff_mul(f, f);
-    const ff f3 = ff_mul(f2, f);
-    ff h = ff_add(ff_add_f(f, 1.0f), ff_mul_f(f2, 0.5f));
-    h = ff_add(h, ff_mul(f3, sixth));
-    const float fh = f.hi, f4 = f2.hi * f2.hi;
-    const float tail =
-        f4 * fmaf(fh, fmaf(fh, fmaf(fh, 1.0f / 5040.0f, 1.0f / 720.0f), 1.0f / 120.0f),
-                  1.0f / 24.0f);
-    ff r = ff_mul(ff_add_f(h, tail), t2[j]);
-    r.hi = ldexpf(r.hi, m);
-    r.lo = ldexpf(r.lo, m);
-    return r;
+    float e;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x.hi));
+    const float p = __fmul_rn(e, e), pl = fmaf(e, e, -p);
+    const float t = __fmul_rn(x.hi, p), t0 = fmaf(x.hi, p, -t);
+    const float tl = fmaf(x.lo, p, __fmul_rn(x.hi, pl));
+    const ff a = fast_two_sum(1.0f - t, -t0);        // 1 - t is exact
+    const float r = a.hi - tl;
+    const float rl = ((a.hi - r) - tl) + a.lo;
+    const float h = 0.5f * r, c = __fmul_rn(e, h);
+    const float cl = fmaf(e, 0.5f * rl, fmaf(0.75f * c, r, fmaf(e, h, -c)));
+    ff y = fast_two_sum(e, c);
+    y.lo += cl;
+    return y;
 }

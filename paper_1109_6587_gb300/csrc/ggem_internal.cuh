@@ -263,8 +263,9 @@ struct ggem_plan {
     double* d_cvol = nullptr;          // [pcount_cap] particle volumes / areas scratch
     bool tcsr_ready = false;
     bool ff = false;                   // element-rule local sum in double-float arithmetic
-    void* d_qp_ff = nullptr;           // [cap_qp][2] float4: sorted point offsets, hi / lo
-    void* d_qg_ff = nullptr;           // [cap_qp][2] float4: sorted point strengths, hi / lo
+    float4* d_ff_hi = nullptr;         // [cap_qp] sorted points: offsets hi, gx hi
+    float4* d_ff_lo = nullptr;         // [cap_qp] offsets lo, gx lo
+    float4* d_ff_g = nullptr;          // [cap_qp] gy, gz in pairs
     // FP32 element rule: point lists of the triangles
     ggem::ElemLists32 el;
     size_t nbr_cap = 0;                // entries that el.nbr holds
@@ -356,13 +357,22 @@ cudaError_t local_sum(const GridGeom& geo, const CellGrid& cg, const SortedSourc
 // FP64 element rule: local sum over sorted quadrature points at the sorted
 // mesh nodes tgt (output in caller order), skipping points of triangles that
 // contain the target (only tested when closer than `near`); layer 0 velocity,
-// 1 double layer.  ff_pos / ff_g: float-pair copies of the points selecting
-// the double-float kernel (nullptr: native FP64)
+// 1 double layer (native FP64)
 cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg,
                            const SortedSources<double>& src, const int4* qvs, double near,
                            const SortedSources<double>& tgt, const double* nrm_tgt, int layer,
-                           double* out, int out_stride, cudaStream_t st,
-                           const void* ff_pos = nullptr, const void* ff_g = nullptr);
+                           double* out, int out_stride, cudaStream_t st);
+// the same in double-float arithmetic (ggem_elemff.cu) over the neighbour lists
+// of L: sorted points as hi / lo offset parts with gx in their free words, g =
+// (gy, gz) in pairs
+cudaError_t elemff_positions(const GridGeom& geo, const CellGrid& cg, int n,
+                             const double4_32a* pos, float4* hi, float4* lo, cudaStream_t st);
+cudaError_t elemff_strengths(int n, const int4* qv, const double4_32a* qw, const double* q,
+                             double scale, float4* hi, float4* lo, float4* g, cudaStream_t st);
+cudaError_t elemff_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
+                       const float4* hi, const float4* lo, const float4* g, const int4* qvs,
+                       double near, const SortedSources<double>& tgt, const double* nrm, int layer,
+                       double* out, int out_stride, cudaStream_t st);
 // FP32 element rule (ggem_elem32.cu).  At mesh_set: triangle centroids cen
 // (binned by build_cells into tri_start / pos / perm), then the order within
 // the cells (perm_out; fills tv, shift), the steps per cell (scratch: ncell
@@ -375,10 +385,12 @@ cudaError_t elem32_order(const GridGeom& geo, const CellGrid& cg, int m, const E
                          const float4* pos, const int* perm, int* perm_out, const double* cen,
                          const int* tri, const double* tri_area, cudaStream_t st);
 cudaError_t elem32_steps(const ElemLists32& L, int ncell, int* scratch, cudaStream_t st);
-// neighbour lists of the cells with targets (tgt_start): counts (scratch: ncell
-// ints; fills nstart), or with `fill` the entries
+// neighbour lists of the cells with targets (tgt_start), of L's steps or, with
+// src_start, of the points sorted there (entries: first point, points, 0, offset
+// index): counts (scratch: ncell ints; fills nstart), or with `fill` the entries
 cudaError_t elem32_neighbours(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
-                              const int* tgt_start, int* scratch, bool fill, cudaStream_t st);
+                              const int* tgt_start, const int* src_start, int* scratch,
+                              bool fill, cudaStream_t st);
 cudaError_t elem32_fill(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
                         const QuadRule& rule, const double* x, cudaStream_t st);
 cudaError_t elem32_strengths(const ElemLists32& L, const QuadRule& rule, int nnodes,
@@ -388,8 +400,6 @@ cudaError_t elem32_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists3
                        float* out, int out_stride, cudaStream_t st);
 // distance of a cell from which the FP32 element rule uses list 1
 double elem32_far_distance(double near_edge);
-// float-pair copy of n double4 (x, y, z, w) values: out[2 i] = hi, out[2 i + 1] = lo
-cudaError_t to_float_pairs(int n, const void* in, void* out, cudaStream_t st);
 cudaError_t gather_int4(int n, const int* perm, const int4* in, int4* out, cudaStream_t st);
 
 // exclusive scan of count[0..n) into start[0..n] (start[n] = total)

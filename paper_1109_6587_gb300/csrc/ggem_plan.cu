@@ -317,10 +317,12 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
                                     (v4_t<T>*)P->d_sg, st));
         if (elem && !P->fp64)
             GG_CUDA(elem32_strengths(P->el, P->rule, n, q, P->d_q32, 8.0 * kPi * geo.mu, st));
-        if (elem && P->fp64)
+        if (elem && P->ff)
+            GG_CUDA(elemff_strengths(P->n_qp, P->d_qv_sorted, (const double4_32a*)P->d_qw, q,
+                                     8.0 * kPi * geo.mu, P->d_ff_hi, P->d_ff_lo, P->d_ff_g, st));
+        else if (elem && P->fp64)
             GG_CUDA(qp_strengths(P->n_qp, P->d_qv_sorted, (const double4_32a*)P->d_qw, q,
                                  8.0 * kPi * geo.mu, (double4_32a*)P->d_qg, st));
-        if (elem && P->ff) GG_CUDA(to_float_pairs(P->n_qp, P->d_qg, P->d_qg_ff, st));
     });
     SortedSources<T> src = sources_of<T>(P, true);
     src.n = n;
@@ -356,6 +358,10 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
             if constexpr (sizeof(T) == 4) {
                 GG_CUDA(elem32_sum(geo, P->cg, P->el, 1.01 * P->near_edge, src, P->d_nrm, layer,
                                    loc, 3, ls));
+            } else if (P->ff) {
+                GG_CUDA(elemff_sum(geo, P->cg, P->el, P->d_ff_hi, P->d_ff_lo, P->d_ff_g,
+                                   P->d_qv_sorted, 1.01 * P->near_edge, src, P->d_nrm, layer, loc,
+                                   3, ls));
             } else {
                 SortedSources<double> qs;
                 qs.pos = (double4_32a*)P->d_qp_pos;
@@ -365,7 +371,7 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
                 qs.cell_start = P->d_qp_start;
                 qs.n = P->n_qp;
                 GG_CUDA(local_sum_elem(geo, P->cg, qs, P->d_qv_sorted, 1.01 * P->near_edge, src,
-                                       P->d_nrm, layer, loc, 3, ls, P->d_qp_ff, P->d_qg_ff));
+                                       P->d_nrm, layer, loc, 3, ls));
             }
         });
         stage(P, ST_ELEM, 1, [&] {
@@ -710,10 +716,13 @@ void plan_build(ggem_plan_t* P, const ggem_params& prm) {
             dalloc(P, &P->d_qp_perm, cq);
             dalloc(P, &P->d_qp_start, (size_t)P->ncell + 1);
             GG_CUDA(cudaMalloc(&P->d_qp_pos, cq * v4 + 32));
-            GG_CUDA(cudaMalloc(&P->d_qg, cq * v4 + 32));
-            if (P->ff) {                   // float-pair copies: [point][hi, lo] float4
-                GG_CUDA(cudaMalloc(&P->d_qp_ff, cq * 2 * sizeof(float4) + 32));
-                GG_CUDA(cudaMalloc(&P->d_qg_ff, cq * 2 * sizeof(float4) + 32));
+            if (P->ff) {
+                dalloc(P, &P->d_ff_hi, cq);
+                dalloc(P, &P->d_ff_lo, cq);
+                dalloc(P, &P->d_ff_g, cq);
+                dalloc(P, &P->el.nstart, (size_t)P->ncell + 1);
+            } else {
+                GG_CUDA(cudaMalloc(&P->d_qg, cq * v4 + 32));
             }
         } else {
             // the plan's cells (r_cut / 3); the lists are sized by mesh_set
@@ -772,7 +781,7 @@ void plan_free(ggem_plan_t* P) {
                     P->d_pnodes, P->d_rc, P->d_rscale, P->d_mref, P->d_cx0, P->d_cdf,
                     P->d_cuinf, P->d_cfinf, P->d_cb, P->d_ckap, P->d_clam, P->d_cw, P->d_cq,
                     P->d_cmin, P->d_tstart, P->d_tlist, P->d_cvol, P->d_orec, P->d_orecd,
-                    P->d_ocount, P->d_odisp, P->d_qp_ff, P->d_qg_ff,
+                    P->d_ocount, P->d_odisp, P->d_ff_hi, P->d_ff_lo, P->d_ff_g,
                     P->d_spec, P->d_spec_twx, P->d_spec_twz, P->d_spec_dx,
                     P->d_spec_dz, P->d_spec_mid, P->d_spec_ct, P->d_mlp_tc,
                     P->d_mlp_tcs, P->d_q32, P->d_et_cen, P->d_et_cell,
@@ -784,6 +793,26 @@ void plan_free(ggem_plan_t* P) {
     dfree(P->d_pc_Zb);
     if (P->h_sh) cudaFreeHost(P->h_sh);
     if (P->twin) ggem_plan_destroy(P->twin);
+}
+
+// Neighbour lists of the mesh nodes' cells: the steps of the FP32 lists, or the
+// points sorted at src_start.
+void neighbour_lists(ggem_plan_t* P, const int* src_start) {
+    cudaStream_t st = P->st;
+    ElemLists32& L = P->el;
+    GG_CUDA(elem32_neighbours(P->geo, P->cg, L, P->d_mesh_start, src_start, P->d_cell_count, false,
+                              st));
+    int n = 0;
+    GG_CUDA(cudaMemcpyAsync(&n, L.nstart + P->ncell, sizeof(int), cudaMemcpyDeviceToHost, st));
+    GG_CUDA(cudaStreamSynchronize(st));
+    if ((size_t)n > P->nbr_cap) {
+        dfree(L.nbr);
+        L.nbr = nullptr;
+        P->nbr_cap = 0;
+        dalloc(P, &L.nbr, (size_t)n + n / 8);
+        P->nbr_cap = (size_t)n + n / 8;
+    }
+    GG_CUDA(elem32_neighbours(P->geo, P->cg, L, P->d_mesh_start, src_start, nullptr, true, st));
 }
 
 // FP32 element rule: the triangles (by centroid) into the cells, then the
@@ -800,10 +829,6 @@ void elem32_mesh(ggem_plan_t* P, int m) {
     GG_CUDA(elem32_order(P->geo, P->cg, m, L, P->d_et_pos, P->d_et_perm, P->d_et_perm2,
                          P->d_et_cen, P->d_tri, P->d_tri_area, st));
     GG_CUDA(elem32_steps(L, P->ncell, P->d_cell_count, st));
-    GG_CUDA(elem32_neighbours(P->geo, P->cg, L, P->d_mesh_start, P->d_cell_count, false, st));
-    int nnbr = 0;
-    GG_CUDA(cudaMemcpyAsync(&nnbr, L.nstart + P->ncell, sizeof(int), cudaMemcpyDeviceToHost,
-                            st));
     for (int l = 0; l < kElemLists; ++l)
         GG_CUDA(cudaMemcpyAsync(&L.nsteps[l], L.sstart[l] + P->ncell, sizeof(int),
                                 cudaMemcpyDeviceToHost, st));
@@ -834,14 +859,7 @@ void elem32_mesh(ggem_plan_t* P, int m) {
         dalloc(P, &L.pack, 96 * (total + total / 8));
         P->step_cap = total + total / 8;
     }
-    if ((size_t)nnbr > P->nbr_cap) {
-        dfree(L.nbr);
-        L.nbr = nullptr;
-        P->nbr_cap = 0;
-        dalloc(P, &L.nbr, (size_t)nnbr + nnbr / 8);
-        P->nbr_cap = (size_t)nnbr + nnbr / 8;
-    }
-    GG_CUDA(elem32_neighbours(P->geo, P->cg, L, P->d_mesh_start, nullptr, true, st));
+    neighbour_lists(P, nullptr);
     GG_CUDA(elem32_fill(P->geo, P->cg, L, P->rule, P->d_x, st));
 }
 
@@ -984,11 +1002,16 @@ ggem_status ggem_mesh_set(ggem_plan_t* P, int n_nodes, const double* x, int n_tr
                 GG_CUDA(build_cells<double>(P->geo, P->cg, nq, P->d_qx, P->d_cell_count,
                                             P->d_qp_start, P->d_cursor, P->d_qp_cell,
                                             P->d_qp_perm, (double4_32a*)P->d_qp_pos, st));
-                if (P->ff) GG_CUDA(to_float_pairs(nq, P->d_qp_pos, P->d_qp_ff, st));
+                if (P->ff) {
+                    GG_CUDA(elemff_positions(P->geo, P->cg, nq, (const double4_32a*)P->d_qp_pos,
+                                             P->d_ff_hi, P->d_ff_lo, st));
+                    neighbour_lists(P, P->d_qp_start);
+                }
                 GG_CUDA(gather_int4(nq, P->d_qp_perm, P->d_qv, P->d_qv_sorted, st));
-                // weights into point order too (scratch: the strength buffer)
+                // weights into point order too (scratch: a buffer free until the first
+                // evaluation, or after the copy above)
                 GG_CUDA(qp_sort_weights(nq, P->d_qp_perm, (double4_32a*)P->d_qw,
-                                        (double4_32a*)P->d_qg, st));
+                                        (double4_32a*)(P->ff ? P->d_qp_pos : P->d_qg), st));
             } else {
                 elem32_mesh(P, n_tris);
             }
