@@ -156,11 +156,14 @@ cudaError_t mlp_tc_forward(int n, int mode, const void* img, const float* p, con
                            cudaStream_t st);
 // tensor-core training of one minibatch (ggem_mlp_tc.cu): scratch bytes for
 // minibatches of up to nb rows, and the minibatch (loss added to *loss,
-// gradient added to grad)
+// gradient in *nparts parts of kTrainStride floats at part, or added to grad)
 size_t mlp_tc_train_scratch(int nb);
+constexpr int kTrainParts = 64;
+constexpr size_t kTrainStride = 35076;
 cudaError_t mlp_tc_train_batch(int nb, const int* idx, const float* feat, const float* target,
-                               const float* p, const float* stats, float* grad, float* loss,
-                               void* scratch, int* err, cudaStream_t st);
+                               const float* p, const float* stats, float* grad, float* part,
+                               int* nparts, float* loss, void* scratch, int* err,
+                               cudaStream_t st);
 
 // out = base + A^-1 r estimated by the learned warm start (device arrays;
 // base may be NULL); defined with the network kernels

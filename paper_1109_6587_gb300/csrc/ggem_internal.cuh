@@ -284,6 +284,7 @@ struct ggem_plan {
     float* d_feat = nullptr;           // [cap][12] features
     float* d_mlp = nullptr;            // [35075] FP32 master parameters
     float* d_mlp_grad = nullptr;       // gradient accumulator
+    float* d_mlp_part = nullptr;       // gradient parts of one minibatch (BF16 training)
     float* d_mlp_m = nullptr;          // Adam first moments
     float* d_mlp_v = nullptr;          // Adam second moments
     unsigned short* d_mlp_wf = nullptr;  // bfloat16 weights [fan_in][fan_out]

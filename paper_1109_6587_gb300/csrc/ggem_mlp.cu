@@ -356,14 +356,23 @@ __global__ void __launch_bounds__(H) k_mlp_train(int nb, const int* __restrict__
     }
 }
 
-// Adam on the FP32 masters; gradients cleared; bfloat16 copies refreshed
-__global__ void k_mlp_adam(float* __restrict__ p, float* __restrict__ grad, float* __restrict__ m1,
+// Adam on the FP32 masters; bfloat16 copies refreshed.  The gradient is the sum of
+// nparts parts (in FP64, fixed order), or grad, cleared, where there are none
+__global__ void k_mlp_adam(float* __restrict__ p, float* __restrict__ grad,
+                           const float* __restrict__ part, int nparts, float* __restrict__ m1,
                            float* __restrict__ m2, __nv_bfloat16* __restrict__ wf,
                            __nv_bfloat16* __restrict__ wt, float lr, float c1, float c2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= NP) return;
-    const float g = grad[i];
-    grad[i] = 0.f;
+    float g;
+    if (nparts > 0) {
+        double t = 0.0;
+        for (int s = 0; s < nparts; ++s) t += (double)part[(size_t)s * kTrainStride + i];
+        g = (float)t;
+    } else {
+        g = grad[i];
+        grad[i] = 0.f;
+    }
     const float a = 0.9f * m1[i] + 0.1f * g;
     const float v = 0.999f * m2[i] + 0.001f * g * g;
     m1[i] = a;
@@ -400,24 +409,38 @@ __global__ void k_mlp_round(const float* __restrict__ p, __nv_bfloat16* __restri
     else if (i >= OW4 && i < OB4) wt[OW4 + ((i - OW4) % 3) * H + (i - OW4) / 3] = wb;
 }
 
-// per-feature sums of x and x^2 and the sum of squared targets (FP64)
-__global__ void k_mlp_moments(int n, const float* __restrict__ feat,
-                              const float* __restrict__ target, double* __restrict__ acc) {
-    __shared__ double s[2 * NF + 1];
-    for (int t = threadIdx.x; t < 2 * NF + 1; t += blockDim.x) s[t] = 0.0;
-    __syncthreads();
+// per-feature sums of x and x^2 and the sum of squared targets (FP64): sums in
+// registers, one warp reduction and one add per block and value (all threads
+// adding into 25 shared words took 183 us on 65,536 rows, this 19)
+__global__ void __launch_bounds__(128) k_mlp_moments(int n, const float* __restrict__ feat,
+                                                     const float* __restrict__ target,
+                                                     double* __restrict__ acc) {
+    __shared__ double s[2 * NF + 1][4];
+    double v[2 * NF + 1];
+#pragma unroll
+    for (int k = 0; k < 2 * NF + 1; ++k) v[k] = 0.0;
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+#pragma unroll
         for (int k = 0; k < NF; ++k) {
-            const double v = feat[(size_t)r * NF + k];
-            atomicAdd(&s[k], v);
-            atomicAdd(&s[NF + k], v * v);
+            const double x = feat[(size_t)r * NF + k];
+            v[k] += x;
+            v[NF + k] = fma(x, x, v[NF + k]);
         }
-        const double t0 = target[3 * (size_t)r], t1 = target[3 * (size_t)r + 1],
-                     t2 = target[3 * (size_t)r + 2];
-        atomicAdd(&s[2 * NF], t0 * t0 + t1 * t1 + t2 * t2);
+        for (int c = 0; c < 3; ++c) {
+            const double y = target[(size_t)r * 3 + c];
+            v[2 * NF] = fma(y, y, v[2 * NF]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 2 * NF + 1; ++k) {
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+        if ((threadIdx.x & 31) == 0) s[k][threadIdx.x >> 5] = v[k];
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < 2 * NF + 1; t += blockDim.x) atomicAdd(&acc[t], s[t]);
+    if (threadIdx.x < 2 * NF + 1) {
+        const double* t = s[threadIdx.x];
+        atomicAdd(acc + threadIdx.x, (t[0] + t[1]) + (t[2] + t[3]));
+    }
 }
 
 __global__ void k_to_float(size_t n, const double* __restrict__ a, float* __restrict__ b) {
@@ -440,6 +463,7 @@ void ensure_mlp(ggem_plan_t* P) {
     dalloc(P, &P->d_mlp_v, NP);
     dalloc(P, &P->d_mlp_wf, NP);
     dalloc(P, &P->d_mlp_wt, NP);
+    dalloc(P, &P->d_mlp_part, kTrainParts * kTrainStride);
     dalloc(P, &P->d_mlp_stats, NSTAT);
     dalloc(P, &P->d_feat, (size_t)P->cap * NF);
     dalloc(P, &P->d_mlp_out, (size_t)P->cap * 3);
@@ -456,18 +480,23 @@ Net net_of(ggem_plan_t* P) {
 
 // one minibatch's forward, loss and gradient (added to P->d_mlp_grad): FP32
 // mode on the SIMT kernel, BF16 mode as tensor-core GEMMs (ggem_mlp_tc.cu)
-void train_batch(ggem_plan_t* P, int nb, const int* idx, const float* f, const float* t,
-                 float* dloss) {
+// (parts: BF16 mode may leave the gradient in P->d_mlp_part instead; returns
+// their number)
+int train_batch(ggem_plan_t* P, int nb, const int* idx, const float* f, const float* t,
+                float* dloss, bool parts) {
+    int np = 0;
     if (P->mlp_fp32) {
         k_mlp_train<false><<<nblk(nb, TN), H, 0, P->st>>>(nb, idx, net_of(P), f, t,
                                                           P->d_mlp_grad, dloss);
         P->launches += 1;
     } else {
         GG_CHECK(nb <= P->mlp_tcs_rows, GGEM_ERR_INVALID_ARG, "training scratch too small");
-        GG_CUDA(mlp_tc_train_batch(nb, idx, f, t, P->d_mlp, P->d_mlp_stats, P->d_mlp_grad, dloss,
-                                   P->d_mlp_tcs, P->d_tc_err, P->st));
-        P->launches += 15;
+        GG_CUDA(mlp_tc_train_batch(nb, idx, f, t, P->d_mlp, P->d_mlp_stats, P->d_mlp_grad,
+                                   parts ? P->d_mlp_part : nullptr, &np, dloss, P->d_mlp_tcs,
+                                   P->d_tc_err, P->st));
+        P->launches += 11;
     }
+    return np;
 }
 
 // tensor-core training scratch for minibatches of up to rows rows
@@ -764,7 +793,7 @@ ggem_status ggem_mlp_train(ggem_plan_t* P, int n, const double* feat, const doub
             std::mt19937_64 rng(seed);
             if (init) {
                 GG_CUDA(cudaMemsetAsync(mom, 0, NSTAT * sizeof(double), st));
-                k_mlp_moments<<<152, 256, 0, st>>>(n, f, t, mom);
+                k_mlp_moments<<<2 * 152, 128, 0, st>>>(n, f, t, mom);
                 std::vector<double> hm(NSTAT);
                 GG_CUDA(cudaMemcpyAsync(hm.data(), mom, NSTAT * sizeof(double),
                                         cudaMemcpyDeviceToHost, st));
@@ -812,7 +841,7 @@ ggem_status ggem_mlp_train(ggem_plan_t* P, int n, const double* feat, const doub
                                         cudaMemcpyHostToDevice, st));
                 GG_CUDA(cudaMemsetAsync(dloss, 0, sizeof(float), st));
                 GG_CUDA(cudaMemsetAsync(P->d_mlp_grad, 0, NP * sizeof(float), st));
-                train_batch(P, n, idx, f, t, dloss);
+                train_batch(P, n, idx, f, t, dloss, false);
                 float hl = 0.f;
                 GG_CUDA(cudaMemcpyAsync(&hl, dloss, sizeof(float), cudaMemcpyDeviceToHost, st));
                 if (grad_out) {
@@ -839,12 +868,12 @@ ggem_status ggem_mlp_train(ggem_plan_t* P, int n, const double* feat, const doub
                 int nbatches = 0;
                 for (int r0 = 0; r0 < n; r0 += batch) {
                     const int nb = std::min(batch, n - r0);
-                    train_batch(P, nb, idx + r0, f, t, dloss);
+                    const int np = train_batch(P, nb, idx + r0, f, t, dloss, true);
                     P->mlp_step++;
                     const float c1 = 1.f - std::pow(0.9f, (float)P->mlp_step);
                     const float c2 = 1.f - std::pow(0.999f, (float)P->mlp_step);
                     k_mlp_adam<<<nblk(NP), 256, 0, st>>>(
-                        P->d_mlp, P->d_mlp_grad, P->d_mlp_m, P->d_mlp_v,
+                        P->d_mlp, P->d_mlp_grad, P->d_mlp_part, np, P->d_mlp_m, P->d_mlp_v,
                         (__nv_bfloat16*)P->d_mlp_wf, (__nv_bfloat16*)P->d_mlp_wt, (float)lr, c1,
                         c2);
                     ++nbatches;

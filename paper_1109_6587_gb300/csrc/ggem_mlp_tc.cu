@@ -345,27 +345,39 @@ cudaError_t mlp_tc_forward(int n, int mode, const void* img, const float* p, con
 //   DELTA  backpropagated delta: C where the layer's activation is positive,
 //          split into bfloat16 hi + lo (so the products keep ~16 more bits),
 //          stored row-major and transposed, and its column sums (bias
-//          gradient) added to the gradient;
-//   GRAD   weight gradient: C added to the gradient (atomics, split over K).
+//          gradient);
+//   GRAD   weight gradient, split over K.
+// The gradient's parts, one per 128 rows, go to memory of their own and are
+// added in a fixed order by the optimiser (minibatches of up to kTrainParts
+// tiles), or are added with atomics (larger ones).
 // Deltas enter the products as hi + lo (two MMAs per step); activations and
 // weights are bfloat16 by the network's definition, so the gradients match
 // backpropagation with unrounded deltas to about 2^-16 of each term.
-// A CTA (4 warps, 128 threads = 128 TMEM lanes) computes one 128-row tile of C
-// over a range of K, staging K in chunks of 64 (canonical K-major layout, as
-// above) and waiting on each chunk's MMAs (bounded wait).
+// A CTA (4 warps, 128 threads = 128 TMEM lanes) computes one 128-row, NT-column
+// tile of C over a range of K, staging K in chunks of 64 (canonical K-major
+// layout, as above) and waiting on each chunk's MMAs (bounded wait).
+// What bounds it: latency, most of it the epilogue's -- a minibatch of 2048 rows
+// is 16 row tiles on 152 SMs, and a thread writes (and in DELTA reads and sums)
+// its row's columns one after the other.  So C's 128 columns are cut into NT = 16
+// per CTA, and products that do not wait on each other -- a layer's weight
+// gradient and the delta it passes on -- share a launch.  One epoch of 65,536 rows:
+// 10.8 ms with 128 columns per CTA, 5.5 with 32, 4.9 with 16 (128-wide K chunks
+// 5.0), 4.1 with the shared launches, 4.0 with the gradient's parts stored apart.
 namespace {
 
 enum { EP_ACT = 0, EP_OUT = 1, EP_DELTA = 2, EP_GRAD = 3 };
 constexpr int KC = 64;                      // K per staged chunk
+constexpr int NT = 16;                      // columns per CTA (at most)
 
 struct TcGemm {
-    int M, N, K;                            // N a multiple of 16 (<= 128), K of 16
+    int M, N, K;                            // N a multiple of 16 (<= 128; of NT above it), K of 16
     const __nv_bfloat16 *A, *Alo;           // A [M][lda] (Alo may be null)
     int lda;
     const __nv_bfloat16 *B, *Blo;           // B [N][ldb]
     int ldb;
     int kspan;                              // K per CTA (grid.y splits K)
     int mode, nreal;                        // epilogue; columns that exist
+    int gx, gy, blocks;                     // row tiles, K splits, CTAs in all (set at launch)
     const float* bias;                      // ACT, OUT: [N]
     const __nv_bfloat16* mask;              // DELTA: activation [M][ldmask]
     int ldmask;
@@ -376,7 +388,8 @@ struct TcGemm {
     float* out32;                           // OUT: [M][ld32]; GRAD: gradient base
     int ld32;
     int gtrans;                             // GRAD: element (m, n) at n * ld32 + m
-    float* bgrad;                           // DELTA: bias gradient [N] (atomics)
+    float* bgrad;                           // DELTA: bias gradient [N]
+    size_t pstride;                         // GRAD, bgrad: floats between parts (0: atomics)
     int* err;
 };
 
@@ -394,19 +407,27 @@ __device__ __forceinline__ void stage_rows(const __nv_bfloat16* src, int ld, int
     }
 }
 
-__global__ void __launch_bounds__(TPB) k_gemm_tc(TcGemm g) {
+// CTAs [0, ga.blocks) compute ga, the rest gb (independent products)
+__global__ void __launch_bounds__(TPB) k_gemm_tc(TcGemm ga, TcGemm gb) {
+    const bool second = (int)blockIdx.x >= ga.blocks;
+    const TcGemm& g = second ? gb : ga;
+    const int bid = (int)blockIdx.x - (second ? ga.blocks : 0);
+    const int bx = bid % g.gx, by = (bid / g.gx) % g.gy, bz = bid / (g.gx * g.gy);
     extern __shared__ __align__(1024) unsigned char sm[];
     __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(sm);     // [128][KC]
     __nv_bfloat16* sAl = sA + 128 * KC;
-    __nv_bfloat16* sB = sAl + 128 * KC;                           // [128][KC]
-    __nv_bfloat16* sBl = sB + 128 * KC;
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(sBl + 128 * KC);
+    __nv_bfloat16* sB = sAl + 128 * KC;                           // [NT][KC]
+    __nv_bfloat16* sBl = sB + NT * KC;
+    uint64_t* mbar = reinterpret_cast<uint64_t*>(sBl + NT * KC);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
     __shared__ int s_fail;
+    __shared__ float s_col[4][16];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * 128;
-    const int k_beg = blockIdx.y * g.kspan, k_end = min(g.K, k_beg + g.kspan);
-    const uint32_t tcols = g.N <= 32 ? 32 : (g.N <= 64 ? 64 : 128);
+    const int m0 = bx * 128;
+    const int k_beg = by * g.kspan, k_end = min(g.K, k_beg + g.kspan);
+    // this CTA's columns n0 .. n0 + nn of C
+    const int n0 = bz * NT, nn = min(NT, g.N - n0);
+    const uint32_t tcols = 32;
     if (tid == 0) {
         s_fail = 0;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(mbar)));
@@ -422,7 +443,7 @@ __global__ void __launch_bounds__(TPB) k_gemm_tc(TcGemm g) {
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tslot;
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.N >> 3) << 17) |
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nn >> 3) << 17) |
                            ((uint32_t)(128 >> 4) << 24);
     const uint32_t sbo = (uint32_t)(KC / 8) * 128;
     const int mrows = min(128, g.M - m0);
@@ -431,8 +452,8 @@ __global__ void __launch_bounds__(TPB) k_gemm_tc(TcGemm g) {
     for (int k0 = k_beg; k0 < k_end; k0 += KC) {
         stage_rows(g.A + (size_t)m0 * g.lda, g.lda, 128, mrows, k0, k_end, sA, tid);
         if (g.Alo) stage_rows(g.Alo + (size_t)m0 * g.lda, g.lda, 128, mrows, k0, k_end, sAl, tid);
-        stage_rows(g.B, g.ldb, g.N, g.N, k0, k_end, sB, tid);
-        if (g.Blo) stage_rows(g.Blo, g.ldb, g.N, g.N, k0, k_end, sBl, tid);
+        stage_rows(g.B + (size_t)n0 * g.ldb, g.ldb, nn, nn, k0, k_end, sB, tid);
+        if (g.Blo) stage_rows(g.Blo + (size_t)n0 * g.ldb, g.ldb, nn, nn, k0, k_end, sBl, tid);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
@@ -468,9 +489,10 @@ __global__ void __launch_bounds__(TPB) k_gemm_tc(TcGemm g) {
         const int m = m0 + tid;                            // this thread's row
         const bool live = tid < mrows;
         const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-        for (int c0 = 0; c0 < g.N; c0 += 16) {
+        for (int cc = 0; cc < nn; cc += 16) {
+            const int c0 = n0 + cc;                        // column of C
             uint32_t r[16];
-            tmem_ld16(trow + (uint32_t)c0, r);
+            tmem_ld16(trow + (uint32_t)cc, r);
             float v[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
@@ -493,24 +515,36 @@ __global__ void __launch_bounds__(TPB) k_gemm_tc(TcGemm g) {
                     for (int j = 0; j < 16; ++j)
                         if (c0 + j < g.nreal) g.out32[(size_t)m * g.ld32 + c0 + j] = v[j] + g.bias[c0 + j];
             } else if (g.mode == EP_DELTA) {
+                // the row's 16 activations in two 16-byte loads (rows of 128
+                // bfloat16, c0 a multiple of 16: aligned)
+                __align__(16) __nv_bfloat16 a[16];
+                if (live) {
+                    const uint4* mk = reinterpret_cast<const uint4*>(g.mask + (size_t)m * g.ldmask + c0);
+                    *reinterpret_cast<uint4*>(a) = mk[0];
+                    *reinterpret_cast<uint4*>(a + 8) = mk[1];
+                }
+                __align__(16) __nv_bfloat16 hh[16], ll[16];
                 float col[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
-                    const bool on = live && __bfloat162float(g.mask[(size_t)m * g.ldmask + c0 + j]) > 0.f;
-                    v[j] = on ? v[j] : 0.f;
+                    v[j] = live && __bfloat162float(a[j]) > 0.f ? v[j] : 0.f;
                     col[j] = v[j];
+                    hh[j] = __float2bfloat16_rn(v[j]);
+                    ll[j] = __float2bfloat16_rn(v[j] - __bfloat162float(hh[j]));
                 }
                 if (live) {
+                    if (g.out) {
+                        uint4* o = reinterpret_cast<uint4*>(g.out + (size_t)m * g.ldo + c0);
+                        uint4* ol = reinterpret_cast<uint4*>(g.out_lo + (size_t)m * g.ldo + c0);
+                        o[0] = *reinterpret_cast<const uint4*>(hh);
+                        o[1] = *reinterpret_cast<const uint4*>(hh + 8);
+                        ol[0] = *reinterpret_cast<const uint4*>(ll);
+                        ol[1] = *reinterpret_cast<const uint4*>(ll + 8);
+                    }
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
-                        const __nv_bfloat16 h = __float2bfloat16_rn(v[j]);
-                        const __nv_bfloat16 l = __float2bfloat16_rn(v[j] - __bfloat162float(h));
-                        if (g.out) {
-                            g.out[(size_t)m * g.ldo + c0 + j] = h;
-                            g.out_lo[(size_t)m * g.ldo + c0 + j] = l;
-                        }
-                        g.outT[(size_t)(c0 + j) * g.ldt + m] = h;
-                        g.outT_lo[(size_t)(c0 + j) * g.ldt + m] = l;
+                        g.outT[(size_t)(c0 + j) * g.ldt + m] = hh[j];
+                        g.outT_lo[(size_t)(c0 + j) * g.ldt + m] = ll[j];
                     }
                 }
                 // bias gradient: column sums over the tile's rows
@@ -518,15 +552,25 @@ __global__ void __launch_bounds__(TPB) k_gemm_tc(TcGemm g) {
                 for (int j = 0; j < 16; ++j) {
                     float t = col[j];
                     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                    if (lane == 0 && c0 + j < g.nreal) atomicAdd(g.bgrad + c0 + j, t);
+                    if (lane == 0) s_col[warp][j] = t;
                 }
+                __syncthreads();
+                if (tid < 16 && c0 + tid < g.nreal) {
+                    const float t = (s_col[0][tid] + s_col[1][tid]) + (s_col[2][tid] + s_col[3][tid]);
+                    float* b = g.bgrad + bx * g.pstride + c0 + tid;
+                    if (g.pstride) *b = t;
+                    else atomicAdd(b, t);
+                }
+                __syncthreads();
             } else {                                       // EP_GRAD
                 if (live)
                     for (int j = 0; j < 16; ++j)
                         if (c0 + j < g.nreal) {
-                            const size_t e = g.gtrans ? (size_t)(c0 + j) * g.ld32 + m
-                                                      : (size_t)m * g.ld32 + c0 + j;
-                            atomicAdd(g.out32 + e, v[j]);
+                            const size_t e = by * g.pstride +
+                                             (g.gtrans ? (size_t)(c0 + j) * g.ld32 + m
+                                                       : (size_t)m * g.ld32 + c0 + j);
+                            if (g.pstride) g.out32[e] = v[j];
+                            else atomicAdd(g.out32 + e, v[j]);
                         }
             }
         }
@@ -540,7 +584,8 @@ __global__ void __launch_bounds__(TPB) k_gemm_tc(TcGemm g) {
                      "r"(tcols));
 }
 
-constexpr size_t kGemmSmem = (size_t)4 * 128 * KC * 2 + 16;
+static_assert(ggem::kTrainStride >= OB4 + 3, "a part holds every parameter");
+constexpr size_t kGemmSmem = (size_t)2 * (128 + NT) * KC * 2 + 16;
 
 // inputs of one minibatch: X0 [nbp][16] = standardised features (bfloat16,
 // zero past 12 and past nb), its transpose X0T [16][nbp]; targets / s_y into
@@ -570,7 +615,7 @@ __global__ void k_train_out_delta(int nb, int nbp, const float* __restrict__ Y,
                                   const float* __restrict__ T, __nv_bfloat16* __restrict__ D,
                                   __nv_bfloat16* __restrict__ Dl, __nv_bfloat16* __restrict__ DT,
                                   __nv_bfloat16* __restrict__ DTl, float* __restrict__ grad_b4,
-                                  float* __restrict__ loss) {
+                                  size_t pstride, float* __restrict__ loss) {
     __shared__ float red[4][TPB / 32];
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -604,6 +649,7 @@ __global__ void k_train_out_delta(int nb, int nbp, const float* __restrict__ Y,
         float t = 0.f;
         for (int q = 0; q < TPB / 32; ++q) t += red[threadIdx.x][q];
         if (threadIdx.x == 0) atomicAdd(loss, t / (3.f * (float)nb));
+        else if (pstride) grad_b4[blockIdx.x * pstride + threadIdx.x - 1] = t;
         else atomicAdd(grad_b4 + threadIdx.x - 1, t);
     }
 }
@@ -649,11 +695,21 @@ size_t mlp_tc_train_scratch(int nb) {
     return bf * 2 + nbp * 6 * 4 + 256;
 }
 
-// One minibatch (rows idx[0..nb)): loss added to *loss, gradients added to grad.
+// One minibatch (rows idx[0..nb)): loss added to *loss; gradients into
+// *nparts parts at `part` (kTrainParts rooms of kTrainStride floats) when it is
+// given and has room for one per 128 rows, else added to grad (*nparts = 0).
 cudaError_t mlp_tc_train_batch(int nb, const int* idx, const float* feat, const float* target,
-                               const float* p, const float* stats, float* grad, float* loss,
-                               void* scratch, int* err, cudaStream_t st) {
+                               const float* p, const float* stats, float* grad, float* part,
+                               int* nparts, float* loss, void* scratch, int* err,
+                               cudaStream_t st) {
+    *nparts = 0;
     if (nb <= 0) return cudaSuccess;
+    size_t ps = 0;
+    if (part && (nb + 127) / 128 <= kTrainParts) {
+        *nparts = (nb + 127) / 128;
+        grad = part;
+        ps = kTrainStride;
+    }
     cudaError_t e = grant_max_smem((const void*)k_gemm_tc);
     if (e != cudaSuccess) return e;
     const int nbp = (nb + 127) / 128 * 128;
@@ -683,10 +739,21 @@ cudaError_t mlp_tc_train_batch(int nb, const int* idx, const float* feat, const 
     float* T = Y + (size_t)nbp * 3;
     k_train_weights<<<(TIMG + 255) / 256, 256, 0, st>>>(p, w);
     k_train_inputs<<<nbp / TPB, TPB, 0, st>>>(nb, nbp, idx, feat, target, stats, X0, X0T, T);
-    auto gemm = [&](TcGemm g, int ksplit) {
+    // a shape's CTAs, K split ksplit times
+    auto sized = [&](TcGemm g, int ksplit) {
         g.err = err;
-        dim3 grid((g.M + 127) / 128, ksplit);
-        k_gemm_tc<<<grid, TPB, kGemmSmem, st>>>(g);
+        g.pstride = ps;
+        g.gx = (g.M + 127) / 128;
+        g.gy = ksplit;
+        g.blocks = g.gx * g.gy * ((g.N + NT - 1) / NT);
+        return g;
+    };
+    auto gemm2 = [&](const TcGemm& a, const TcGemm& b) {
+        k_gemm_tc<<<(unsigned)(a.blocks + b.blocks), TPB, kGemmSmem, st>>>(a, b);
+    };
+    auto gemm = [&](const TcGemm& g, int ksplit) {
+        const TcGemm a = sized(g, ksplit);
+        k_gemm_tc<<<(unsigned)a.blocks, TPB, kGemmSmem, st>>>(a, a);
     };
     const int nt = nbp / 128;
     // forward
@@ -708,20 +775,19 @@ cudaError_t mlp_tc_train_batch(int nb, const int* idx, const float* feat, const 
         gemm(g, 1);
     }
     k_train_out_delta<<<nbp / TPB, TPB, 0, st>>>(nb, nbp, Y, T, D4, D4l, D4T, D4Tl, grad + OB4,
-                                                 loss);
+                                                 ps, loss);
     // layer 4: dW4 = A3^T d4 (split over the batch), delta3 = (d4 W4^T) * (a3 > 0)
     {
         TcGemm g{};
         g.M = H; g.N = N4; g.K = nbp; g.A = AT[2]; g.lda = nbp; g.B = D4T; g.Blo = D4Tl;
         g.ldb = nbp; g.kspan = 128; g.mode = EP_GRAD; g.nreal = 3; g.out32 = grad + OW4;
         g.ld32 = 3;
-        gemm(g, nt);
         TcGemm d{};
         d.M = nbp; d.N = H; d.K = N4; d.A = D4; d.Alo = D4l; d.lda = N4; d.B = w + TW4N;
         d.ldb = N4; d.kspan = N4; d.mode = EP_DELTA; d.nreal = H; d.mask = Aact[2]; d.ldmask = H;
         d.out = Dh[0]; d.out_lo = Dl[0]; d.ldo = H; d.outT = DTh[0]; d.outT_lo = DTl[0];
         d.ldt = nbp; d.bgrad = grad + OB3;
-        gemm(d, 1);
+        gemm2(sized(d, 1), sized(g, nt));
     }
     // layers 3, 2: dW = A_prev^T delta; delta_prev = (delta W^T) * (a_prev > 0)
     const int owl[2] = {OW3, OW2}, obp[2] = {OB2, OB1}, wn[2] = {TW3N, TW2N};
@@ -730,14 +796,13 @@ cudaError_t mlp_tc_train_batch(int nb, const int* idx, const float* feat, const 
         g.M = H; g.N = H; g.K = nbp; g.A = AT[1 - q]; g.lda = nbp; g.B = DTh[q]; g.Blo = DTl[q];
         g.ldb = nbp; g.kspan = 128; g.mode = EP_GRAD; g.nreal = H; g.out32 = grad + owl[q];
         g.ld32 = H;
-        gemm(g, nt);
         TcGemm d{};
         d.M = nbp; d.N = H; d.K = H; d.A = Dh[q]; d.Alo = Dl[q]; d.lda = H; d.B = w + wn[q];
         d.ldb = H; d.kspan = H; d.mode = EP_DELTA; d.nreal = H; d.mask = Aact[1 - q];
         d.ldmask = H; d.out = q == 0 ? Dh[1] : nullptr; d.out_lo = q == 0 ? Dl[1] : nullptr;
         d.ldo = H; d.outT = DTh[q + 1]; d.outT_lo = DTl[q + 1]; d.ldt = nbp;
         d.bgrad = grad + obp[q];
-        gemm(d, 1);
+        gemm2(sized(d, 1), sized(g, nt));
     }
     // layer 1: dW1^T = delta1^T X0 (element (j, k) of dW1^T is W1's (k, j))
     {

@@ -774,7 +774,7 @@ void plan_free(ggem_plan_t* P) {
                     P->d_adj_start, P->d_adj_cur, P->d_adj,
                     P->d_qv_sorted, P->d_V, P->d_sv, P->d_sb, P->d_sk, P->d_sx,
                     P->d_spart, P->d_sh, P->d_particle, P->d_pcount, P->d_feat,
-                    P->d_mlp, P->d_mlp_grad, P->d_mlp_m, P->d_mlp_v, P->d_mlp_wf,
+                    P->d_mlp, P->d_mlp_grad, P->d_mlp_part, P->d_mlp_m, P->d_mlp_v, P->d_mlp_wf,
                     P->d_mlp_wt, P->d_mlp_stats, P->d_mlp_out, P->d_smlp,
                     P->d_sres, P->d_mlp_dr, P->d_mlp_ssq, P->d_tc_err,
                     P->d_tc_fwd, P->d_tc_inv, P->d_spread_list, P->d_pstart,
