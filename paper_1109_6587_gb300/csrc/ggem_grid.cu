@@ -275,16 +275,16 @@ cudaError_t cheb_apply(int Ny, const T* M, const T* in, T* out, long cols, cudaS
 }
 
 // ------------------------------------------------------- interpolation
-// Degree-4 Lagrange weights at offset t for nodes -2..2.
+// Degree-4 Lagrange weights at offset t for nodes -2..2 (no division: the
+// products of the nodes' differences are 24, -6, 4, -6, 24).
 template <typename T> __device__ __forceinline__ void lag5_uniform(T t, T w[5]) {
-#pragma unroll
-    for (int p = 0; p < 5; ++p) {
-        T v = 1;
-#pragma unroll
-        for (int q = 0; q < 5; ++q)
-            if (q != p) v *= (t - (T)(q - 2)) / (T)(p - q);
-        w[p] = v;
-    }
+    const T a = t + (T)2, b = t + (T)1, c = t - (T)1, d = t - (T)2;
+    const T ab = a * b, cd = c * d;
+    w[0] = b * t * cd * (T)(1.0 / 24.0);
+    w[1] = a * t * cd * (T)(-1.0 / 6.0);
+    w[2] = ab * cd * (T)0.25;
+    w[3] = ab * t * d * (T)(-1.0 / 6.0);
+    w[4] = ab * t * c * (T)(1.0 / 24.0);
 }
 
 template <typename T> struct InterpArgs {
@@ -302,10 +302,14 @@ template <typename T> struct InterpArgs {
     double self_coef;
     double* out;
     int out_stride;
+    const T* ylag;      // [Ny - 4][6]: scale and weights of each 5-node y stencil
+    double* out2;       // mode 3: the stress
 };
 
 template <typename T>
-__device__ __forceinline__ void interp_store(const InterpArgs<T>& a, int t, const T* acc);
+__device__ __forceinline__ void interp_store(const InterpArgs<T>& a, int t, const T* acc,
+                                             int mode, double* out, int out_stride,
+                                             const T* local);
 
 template <typename T> __device__ __forceinline__ T wexp(T x);
 template <> __device__ __forceinline__ float wexp<float>(float x) { return expf(x); }
@@ -314,12 +318,21 @@ template <> __device__ __forceinline__ double wexp<double>(double x) { return ex
 // mode 0: velocity (3 comps): out = local + interp - self
 // mode 1: stress (6 comps):   out = local + interp
 // mode 2: double layer:       out_j = local_j + n_k sigma_jk / mu
-template <typename T>
-__global__ void __launch_bounds__(128) k_interp(InterpArgs<T> a) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= a.n) return;
+// mode 3: both velocity and stress (9 comps), into out and out2
+// G threads per target share its 25 (y, z) rows of 5 x-values.  One thread per
+// target where the targets fill the chip; 8 where they do not (the chain of
+// dependent loads of one target is then the kernel's time: 162 targets in FP64 76
+// -> 18 us, 1,296 in FP32 29 -> 14, 10,007 with velocity and stress in one launch
+// instead of two 65 -> 55).  The y weights take the stencil's node differences
+// from a table (scale and the reciprocals of their products per stencil), so a
+// target divides nowhere: 64,200 targets 78 -> 72 us, 2,568,000 1.21 -> 1.12 ms
+// (stress and velocity averaged; the gather of 125 x 3 or 6 values is what is left).
+template <typename T, int NC, int G>
+__global__ void __launch_bounds__(64) k_interp(InterpArgs<T> a) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = min(e / G, a.n - 1), g = e % G;     // (lanes past the end repeat the last target)
     const GridGeom& geo = a.geo;
-    double xt = a.x[3 * t], yt = a.x[3 * t + 1], zt = a.x[3 * t + 2];
+    double xt = a.x[3 * (size_t)t], yt = a.x[3 * (size_t)t + 1], zt = a.x[3 * (size_t)t + 2];
     // grid coordinates in FP64 (positions up to the box size), by multiplies:
     // GB300 runs FP64 at 1/64 of FP32 and an FP64 divide is a long sequence
     double ux = xt * (1.0 / geo.dx), uz = zt * (1.0 / geo.dz);
@@ -343,50 +356,65 @@ __global__ void __launch_bounds__(128) k_interp(InterpArgs<T> a) {
         double d = fabs(yt - a.yj[jc + 1]);
         if (d < dbest) { dbest = d; jbest = jc + 1; }
     }
-    int js = min(max(jbest - 2, 0), geo.Ny - 5);
-    double yn[5];
+    const int js = min(max(jbest - 2, 0), geo.Ny - 5);
+    {
+        // scaled differences to the target (each FP64 difference rounded once to T)
+        const T* yl = a.ylag + 6 * (size_t)js;
+        T d[5];
 #pragma unroll
-    for (int p = 0; p < 5; ++p) yn[p] = a.yj[js + p];
-    // Lagrange weights in y: the five FP64 differences to the target and the
-    // ten between the nodes, each rounded once to T
-    T dt[5], dn[5][5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) dt[q] = (T)(yt - yn[q]);
-#pragma unroll
-    for (int p = 0; p < 5; ++p)
-#pragma unroll
-        for (int q = p + 1; q < 5; ++q) {
-            dn[p][q] = (T)(yn[p] - yn[q]);
-            dn[q][p] = -dn[p][q];
-        }
-#pragma unroll
-    for (int p = 0; p < 5; ++p) {
-        T v = 1;
-#pragma unroll
-        for (int q = 0; q < 5; ++q)
-            if (q != p) v *= dt[q] / dn[p][q];
-        wy[p] = v;
+        for (int q = 0; q < 5; ++q) d[q] = (T)(yt - a.yj[js + q]) * yl[0];
+        const T d01 = d[0] * d[1], d34 = d[3] * d[4];
+        wy[0] = d[1] * d[2] * d34 * yl[1];
+        wy[1] = d[0] * d[2] * d34 * yl[2];
+        wy[2] = d01 * d34 * yl[3];
+        wy[3] = d01 * d[2] * d[4] * yl[4];
+        wy[4] = d01 * d[2] * d[3] * yl[5];
     }
     int ib = (int)(((long)i0 - 2) % geo.Nx); ib += (ib < 0) ? geo.Nx : 0;
     int kb = (int)(((long)k0 - 2) % geo.Nz); kb += (kb < 0) ? geo.Nz : 0;
-    const int nc = (a.mode == 0) ? 3 : 6;
-    T acc[6] = {0, 0, 0, 0, 0, 0};
-    const size_t plane = (size_t)geo.Nz * geo.Nx;
-    for (int p = 0; p < 5; ++p) {
-        const T* gy = a.grid + ((size_t)(js + p) * a.ncomp_total + a.comp0) * plane;
-        for (int q = 0; q < 5; ++q) {
-            int kk = kb + q; kk -= (kk >= geo.Nz) ? geo.Nz : 0;
-            T wyz = wy[p] * wz[q];
-            const T* gz = gy + (size_t)kk * geo.Nx;
+    T acc[NC];
 #pragma unroll
-            for (int r = 0; r < 5; ++r) {
-                int ii = ib + r; ii -= (ii >= geo.Nx) ? geo.Nx : 0;
-                T w = wyz * wx[r];
-                for (int c = 0; c < nc; ++c) acc[c] += w * gz[c * plane + ii];
-            }
+    for (int c = 0; c < NC; ++c) acc[c] = (T)0;
+    const size_t plane = (size_t)geo.Nz * geo.Nx;
+    auto row = [&](int p, int q, T wyp, T wzq) {
+        const T* gy = a.grid + ((size_t)(js + p) * a.ncomp_total + a.comp0) * plane;
+        int kk = kb + q; kk -= (kk >= geo.Nz) ? geo.Nz : 0;
+        const T wyz = wyp * wzq;
+        const T* gz = gy + (size_t)kk * geo.Nx;
+#pragma unroll
+        for (int r = 0; r < 5; ++r) {
+            int ii = ib + r; ii -= (ii >= geo.Nx) ? geo.Nx : 0;
+            const T w = wyz * wx[r];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[c] += w * gz[c * plane + ii];
         }
+    };
+    if (G == 1) {
+        for (int p = 0; p < 5; ++p)
+            for (int q = 0; q < 5; ++q) row(p, q, wy[p], wz[q]);
+    } else {
+        for (int i = g; i < 25; i += G) {
+            const int p = i / 5, q = i - 5 * p;
+            T wyp = wy[0], wzq = wz[0];
+#pragma unroll
+            for (int k = 1; k < 5; ++k) {
+                wyp = p == k ? wy[k] : wyp;
+                wzq = q == k ? wz[k] : wzq;
+            }
+            row(p, q, wyp, wzq);
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
     }
-    interp_store<T>(a, t, acc);
+    if (g != 0 || e / G >= a.n) return;
+    if (NC == 9) {
+        interp_store<T>(a, t, acc, 0, a.out, 3, a.local);
+        interp_store<T>(a, t, acc + 3, 1, a.out2, 6, a.local + 3);
+    } else {
+        interp_store<T>(a, t, acc, a.mode, a.out, a.out_stride, a.local);
+    }
 }
 
 // Spectral evaluation of the global field at the targets (GGEM_OFFGRID_SPECTRAL),
@@ -480,7 +508,7 @@ __global__ void __launch_bounds__(128, 8) k_interp_spectral(InterpArgs<T> a, Spe
         for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         acc[c] = v;
     }
-    if (lane == 0) interp_store<T>(a, t, acc);
+    if (lane == 0) interp_store<T>(a, t, acc, a.mode, a.out, a.out_stride, a.local);
 }
 
 // Rectangular contraction out[p][col] = sum_n M[p][n] in[n][col] (M: R x C),
@@ -546,16 +574,18 @@ __global__ void k_spec_pad(const c2_t<T>* __restrict__ spec, long nplanes, int N
 }
 
 template <typename T>
-__device__ __forceinline__ void interp_store(const InterpArgs<T>& a, int t, const T* acc) {
-    double* o = a.out + (size_t)t * a.out_stride;
-    const T* lo = a.local ? a.local + (size_t)t * a.local_stride : nullptr;
-    if (a.mode == 0) {
+__device__ __forceinline__ void interp_store(const InterpArgs<T>& a, int t, const T* acc,
+                                             int mode, double* out, int out_stride,
+                                             const T* local) {
+    double* o = out + (size_t)t * out_stride;
+    const T* lo = local ? local + (size_t)t * a.local_stride : nullptr;
+    if (mode == 0) {
         for (int c = 0; c < 3; ++c) {
             double v = (double)acc[c] + (lo ? (double)lo[c] : 0.0);
             if (a.qself) v -= a.self_coef * (a.wself ? a.wself[t] : 1.0) * a.qself[3 * t + c];
             o[c] = v;
         }
-    } else if (a.mode == 1) {
+    } else if (mode == 1) {
         for (int c = 0; c < 6; ++c) o[c] = (double)acc[c] + (lo ? (double)lo[c] : 0.0);
     } else {
         double n0 = a.nrm[3 * t], n1 = a.nrm[3 * t + 1], n2 = a.nrm[3 * t + 2];
@@ -571,20 +601,34 @@ __device__ __forceinline__ void interp_store(const InterpArgs<T>& a, int t, cons
     }
 }
 
+template <typename T, int NC>
+static void launch_interp(const InterpArgs<T>& a, int nsm, cudaStream_t st) {
+    // 8 threads per target below 4 warps per SM (of one thread per target)
+    if ((long)a.n < 128L * nsm)
+        k_interp<T, NC, 8><<<(unsigned)((8L * a.n + 63) / 64), 64, 0, st>>>(a);
+    else
+        k_interp<T, NC, 1><<<(unsigned)((a.n + 63) / 64), 64, 0, st>>>(a);
+}
+
 template <typename T>
-cudaError_t interp_combine(const GridGeom& geo, const double* yj, const T* grid, int ncomp_total,
-                           int comp0, int n_tgt, const double* x_tgt, const T* local,
-                           int local_stride, const double* nrm, const double* qself,
-                           const double* wself, double self_coef, int mode, double* out,
-                           int out_stride, cudaStream_t st, const SpecGrid* spec) {
+cudaError_t interp_combine(const GridGeom& geo, const double* yj, const T* ylag, const T* grid,
+                           int ncomp_total, int comp0, int n_tgt, const double* x_tgt,
+                           const T* local, int local_stride, const double* nrm,
+                           const double* qself, const double* wself, double self_coef, int mode,
+                           double* out, int out_stride, int nsm, cudaStream_t st,
+                           const SpecGrid* spec, double* out2) {
     if (n_tgt <= 0) return cudaSuccess;
-    InterpArgs<T> a{geo, yj, grid, ncomp_total, comp0, mode, n_tgt, x_tgt, local,
-                    local_stride, nrm, qself, wself, self_coef, out, out_stride};
+    InterpArgs<T> a{geo, yj, grid, ncomp_total, comp0, mode, n_tgt, x_tgt, local, local_stride,
+                    nrm, qself, wself, self_coef, out, out_stride, ylag, out2};
     if (spec) {
         // a warp per target, 4 per block
         k_interp_spectral<T><<<(n_tgt + 3) / 4, 128, 0, st>>>(a, *spec);
+    } else if (mode == 3) {
+        launch_interp<T, 9>(a, nsm, st);
+    } else if (mode == 0) {
+        launch_interp<T, 3>(a, nsm, st);
     } else {
-        k_interp<T><<<(n_tgt + 127) / 128, 128, 0, st>>>(a);
+        launch_interp<T, 6>(a, nsm, st);
     }
     return cudaGetLastError();
 }
@@ -617,10 +661,11 @@ cudaError_t spectral_pad(const GridGeom& geo, const T* spec, int nplanes, int Mx
                                         cudaStream_t, int);                                    \
     template cudaError_t cheb_apply<T>(int, const T*, const T*, T*, long, cudaStream_t, int*,  \
                                        int, const void*);                                      \
-    template cudaError_t interp_combine<T>(const GridGeom&, const double*, const T*, int, int, \
-                                           int, const double*, const T*, int, const double*,   \
-                                           const double*, const double*, double, int, double*, \
-                                           int, cudaStream_t, const SpecGrid*);                   \
+    template cudaError_t interp_combine<T>(const GridGeom&, const double*, const T*, const T*, \
+                                           int, int, int, const double*, const T*, int,         \
+                                           const double*, const double*, const double*, double, \
+                                           int, double*, int, int, cudaStream_t,                \
+                                           const SpecGrid*, double*);                           \
     template cudaError_t spectral_pad<T>(const GridGeom&, const T*, int, int, int, const T*,   \
                                          const T*, T*, cudaStream_t);                          \
     template cudaError_t cheb_rect<T>(int, int, const T*, const T*, T*, long, cudaStream_t);

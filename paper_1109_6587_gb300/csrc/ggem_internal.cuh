@@ -137,6 +137,7 @@ struct ggem_plan {
     double* d_minv = nullptr;          // [4][nmodes] inverse influence matrix
     double* d_kscoef = nullptr;        // [3][Ny] recurrence coefficients
     void* d_ydiff = nullptr;           // [Ny][Ny] T, y_j - y_k
+    void* d_ylag = nullptr;            // [Ny - 4][6] T, y interpolation stencils
 
     // workspaces
     void* d_gridA = nullptr;           // max(9,3)*Ny*Nz*Nx T
@@ -489,12 +490,16 @@ struct SpecGrid {
 // evaluated by 5-point Lagrange interpolation, or (spec != nullptr) from the
 // oversampled grid by the Gaussian window in x, z and the barycentric
 // Chebyshev formula in y.
+// ylag: [Ny - 4][6] per y stencil of 5 nodes, the scale 1 / (y_0 - y_4) and the
+// reciprocals of the products of the scaled node differences; mode 3: velocity
+// into out and stress into out2 (Lagrange only; comp0 = 0, local 9 per target).
 template <typename T>
-cudaError_t interp_combine(const GridGeom& geo, const double* yj, const T* grid, int ncomp_total,
-                           int comp0, int n_tgt, const double* x_tgt, const T* local,
-                           int local_stride, const double* nrm, const double* qself,
-                           const double* wself, double self_coef, int mode, double* out,
-                           int out_stride, cudaStream_t st, const SpecGrid* spec = nullptr);
+cudaError_t interp_combine(const GridGeom& geo, const double* yj, const T* ylag, const T* grid,
+                           int ncomp_total, int comp0, int n_tgt, const double* x_tgt,
+                           const T* local, int local_stride, const double* nrm,
+                           const double* qself, const double* wself, double self_coef, int mode,
+                           double* out, int out_stride, int nsm, cudaStream_t st,
+                           const SpecGrid* spec = nullptr, double* out2 = nullptr);
 
 // Spectral planes [nplanes][Nz][Nx/2] (complex T, after the Chebyshev
 // inverse) -> deconvolved, zero-padded planes [nplanes][Mz][Mx/2] of the

@@ -244,17 +244,25 @@ void point_forces_impl(ggem_plan_t* P, int n_src, const double* xs, const double
     SpecGrid sg = spec_grid(P);
     sg.order = tgt_is_src ? P->d_perm : nullptr;    // sources in cell order
     const SpecGrid* spec = P->offgrid == GGEM_OFFGRID_SPECTRAL ? &sg : nullptr;
+    const double sc = 4.0 * geo.alpha / std::sqrt(kPi) / (8.0 * kPi * geo.mu);
+    const double* qs = tgt_is_src ? g : nullptr;
+    const T* yl = (const T*)P->d_ylag;
+    const T* gb = (const T*)P->d_gridB;
+    if (u && s && !spec) {
+        stage(P, ST_INTERP, 1, [&] {
+            GG_CUDA(interp_combine<T>(geo, P->d_yj, yl, gb, nout, 0, nt, xtt, loc, stride,
+                                      nullptr, qs, nullptr, sc, 3, u, 3, P->nsm, st, nullptr, s));
+        });
+        return;
+    }
     stage(P, ST_INTERP, (u ? 1 : 0) + (s ? 1 : 0), [&] {
-        if (u) {
-            double sc = 4.0 * geo.alpha / std::sqrt(kPi) / (8.0 * kPi * geo.mu);
-            GG_CUDA(interp_combine<T>(geo, P->d_yj, (const T*)P->d_gridB, nout, 0, nt, xtt, loc,
-                                      stride, nullptr, tgt_is_src ? g : nullptr, nullptr, sc, 0,
-                                      u, 3, st, spec));
-        }
+        if (u)
+            GG_CUDA(interp_combine<T>(geo, P->d_yj, yl, gb, nout, 0, nt, xtt, loc, stride,
+                                      nullptr, qs, nullptr, sc, 0, u, 3, P->nsm, st, spec));
         if (s)
-            GG_CUDA(interp_combine<T>(geo, P->d_yj, (const T*)P->d_gridB, nout, u ? 3 : 0, nt,
-                                      xtt, loc + (u ? 3 : 0), stride, nullptr, nullptr, nullptr,
-                                      0.0, 1, s, 6, st, spec));
+            GG_CUDA(interp_combine<T>(geo, P->d_yj, yl, gb, nout, u ? 3 : 0, nt, xtt,
+                                      loc + (u ? 3 : 0), stride, nullptr, nullptr, nullptr, 0.0,
+                                      1, s, 6, P->nsm, st, spec));
     });
 }
 
@@ -394,12 +402,13 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
             // nodal form: remove the free-space global self term (4 alpha/sqrt(pi)) A_b q_b;
             // the element rule integrates the near field itself
             double sc = elem ? 0.0 : 4.0 * geo.alpha / std::sqrt(kPi);
-            GG_CUDA(interp_combine<T>(geo, P->d_yj, (const T*)P->d_gridB, 3, 0, n, P->d_x, loc,
-                                      3, nullptr, elem ? nullptr : q, P->d_area, sc, 0, out, 3,
-                                      st, spec));
+            GG_CUDA(interp_combine<T>(geo, P->d_yj, (const T*)P->d_ylag, (const T*)P->d_gridB, 3,
+                                      0, n, P->d_x, loc, 3, nullptr, elem ? nullptr : q,
+                                      P->d_area, sc, 0, out, 3, P->nsm, st, spec));
         } else {
-            GG_CUDA(interp_combine<T>(geo, P->d_yj, (const T*)P->d_gridB, 6, 0, n, P->d_x, loc,
-                                      3, P->d_nrm, nullptr, nullptr, 0.0, 2, out, 3, st, spec));
+            GG_CUDA(interp_combine<T>(geo, P->d_yj, (const T*)P->d_ylag, (const T*)P->d_gridB, 6,
+                                      0, n, P->d_x, loc, 3, P->d_nrm, nullptr, nullptr, 0.0, 2,
+                                      out, 3, P->nsm, st, spec));
         }
     });
 }
@@ -567,6 +576,31 @@ void plan_build(ggem_plan_t* P, const ggem_params& prm) {
             std::vector<float> yf(yd.begin(), yd.end());
             dalloc(P, (float**)&P->d_ydiff, yf.size());
             GG_CUDA(cudaMemcpy(P->d_ydiff, yf.data(), yf.size() * sizeof(float),
+                               cudaMemcpyHostToDevice));
+        }
+    }
+    {
+        // y interpolation stencils js = 0 .. Ny - 5: the scale s = 1 / (y_js -
+        // y_js+4) and 1 / prod_{q != p} s (y_p - y_q)
+        std::vector<double> yl((size_t)(Ny - 4) * 6);
+        for (int js = 0; js + 5 <= Ny; ++js) {
+            const double sc = 1.0 / (yj[js] - yj[js + 4]);
+            yl[6 * (size_t)js] = sc;
+            for (int p = 0; p < 5; ++p) {
+                double d = 1.0;
+                for (int q = 0; q < 5; ++q)
+                    if (q != p) d *= (yj[js + p] - yj[js + q]) * sc;
+                yl[6 * (size_t)js + 1 + p] = 1.0 / d;
+            }
+        }
+        if (P->fp64) {
+            dalloc(P, (double**)&P->d_ylag, yl.size());
+            GG_CUDA(cudaMemcpy(P->d_ylag, yl.data(), yl.size() * sizeof(double),
+                               cudaMemcpyHostToDevice));
+        } else {
+            std::vector<float> yf(yl.begin(), yl.end());
+            dalloc(P, (float**)&P->d_ylag, yf.size());
+            GG_CUDA(cudaMemcpy(P->d_ylag, yf.data(), yf.size() * sizeof(float),
                                cudaMemcpyHostToDevice));
         }
     }
@@ -762,7 +796,7 @@ void plan_free(ggem_plan_t* P) {
         cudaStreamDestroy(P->st2);
     }
     void* ptrs[] = {P->d_yj, P->d_cheb_fwd, P->d_cheb_inv, P->d_tw_x, P->d_tw_z, P->d_ksb,
-                    P->d_minv, P->d_ydiff, P->d_sdi, P->d_sdf, P->d_mesh_sdi, P->d_mesh_sdf,
+                    P->d_minv, P->d_ydiff, P->d_ylag, P->d_sdi, P->d_sdf, P->d_mesh_sdi, P->d_mesh_sdf,
                     P->d_kscoef, P->d_thom, P->d_kschunk, P->d_isq, P->d_gridA, P->d_gridB, P->d_wall,
                     P->d_cell_count, P->d_cell_start, P->d_cursor, P->d_src_cell,
                     P->d_perm, P->d_spos, P->d_sg, P->d_src_x, P->d_local, P->d_in0, P->d_in1,
