@@ -94,14 +94,20 @@ __global__ void k_adj_fill(int m, const int* __restrict__ tri, const int* __rest
 // triangles' regular points).  layer 0: out += G^l terms (single);
 // layer 1: out += T^l terms with n-tilde (double).  out is the local-sum
 // output [n][3] in caller order, already scaled like it (1/(8 pi mu) G g = G w q).
-template <typename T>
-__global__ void __launch_bounds__(128) k_elem_correct(
+// L = 16: a half-warp per node, a lane per quadrature point (FP64, and FP32 calls
+// too small to fill the chip with a thread per node); L = 1: a thread per node
+// (each triangle's FP64 differences then serve its 16 points).  1,296 nodes in FP64,
+// 11 blocks of a thread per node before: 596 -> 66 us; 64,200 nodes 2.31 -> 2.07 ms;
+// 1,296 nodes in FP32 31 -> 14 us.
+template <typename T, int L>
+__global__ void __launch_bounds__(64) k_elem_correct(
     int n, int layer, T alpha, T rc2, const double* __restrict__ x, const int* __restrict__ tri,
     const double* __restrict__ tri_nrm, const double* __restrict__ nrm,
     const int* __restrict__ adj_start, const int* __restrict__ adj,
     const T* __restrict__ q, QuadRule rule, T* __restrict__ out, int out_stride) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= n) return;
+    const int e0 = blockIdx.x * blockDim.x + threadIdx.x;
+    // (lanes past the end repeat the last node and write nothing)
+    const int b = min(e0 / L, n - 1), l = e0 % L;
     const T al = alpha, al2 = alpha * alpha;
     const T sp = (T)1.7724538509055160273;
     const T c1 = (T)2 * al / sp, c2 = (T)12 * al / sp, c3 = (T)8 * al * al2 / sp,
@@ -109,9 +115,22 @@ __global__ void __launch_bounds__(128) k_elem_correct(
     T nz0 = 0, nz1 = 0, nz2 = 0;
     if (layer == 1) { nz0 = (T)nrm[3 * b]; nz1 = (T)nrm[3 * b + 1]; nz2 = (T)nrm[3 * b + 2]; }
     T rt[4], rw[4], rc_[4], rs_[4], rm[4], rwt[4];
+#pragma unroll
     for (int i = 0; i < 4; ++i) {
         rt[i] = (T)rule.t[i]; rw[i] = (T)rule.w[i]; rc_[i] = (T)rule.cth[i];
         rs_[i] = (T)rule.sth[i]; rm[i] = (T)rule.rmax[i]; rwt[i] = (T)rule.wth[i];
+    }
+    if (L > 1) {                        // this lane's point: entry 0 of each
+        const int qa = l >> 2, qc = l & 3;
+#pragma unroll
+        for (int i = 1; i < 4; ++i) {
+            rc_[0] = qa == i ? rc_[i] : rc_[0];
+            rs_[0] = qa == i ? rs_[i] : rs_[0];
+            rm[0] = qa == i ? rm[i] : rm[0];
+            rwt[0] = qa == i ? rwt[i] : rwt[0];
+            rt[0] = qc == i ? rt[i] : rt[0];
+            rw[0] = qc == i ? rw[i] : rw[0];
+        }
     }
     T acc0 = 0, acc1 = 0, acc2 = 0;
     for (int e = adj_start[b]; e < adj_start[b + 1]; ++e) {
@@ -133,8 +152,8 @@ __global__ void __launch_bounds__(128) k_elem_correct(
         T cx = e2[1] * e3[2] - e2[2] * e3[1], cy = e2[2] * e3[0] - e2[0] * e3[2],
           cz = e2[0] * e3[1] - e2[1] * e3[0];
         T omega = sqrt(cx * cx + cy * cy + cz * cz);     // |x_xi x x_eta| = 2 A_k
-        for (int qa = 0; qa < 4; ++qa)
-            for (int qc = 0; qc < 4; ++qc) {
+        for (int pt = 0; pt < 16 / L; ++pt) {
+                const int qa = L > 1 ? 0 : pt >> 2, qc = L > 1 ? 0 : pt & 3;
                 T rmax = rm[qa];
                 T rho = rmax * rt[qc];
                 T xi = rho * rc_[qa];
@@ -177,6 +196,15 @@ __global__ void __launch_bounds__(128) k_elem_correct(
                 }
             }
     }
+    if (L > 1) {
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) {
+            acc0 += __shfl_xor_sync(0xffffffffu, acc0, o);
+            acc1 += __shfl_xor_sync(0xffffffffu, acc1, o);
+            acc2 += __shfl_xor_sync(0xffffffffu, acc2, o);
+        }
+    }
+    if (l != 0 || e0 / L >= n) return;
     T* o = out + (size_t)b * out_stride;
     o[0] += acc0;
     o[1] += acc1;
@@ -256,18 +284,22 @@ template <typename T>
 cudaError_t elem_correct(int n, int layer, const GridGeom& geo, const double* x, const int* tri,
                          const double* tri_nrm, const double* nrm, const int* adj_start,
                          const int* adj, const T* q, const QuadRule& rule, T* out,
-                         int out_stride, cudaStream_t st) {
-    if (n > 0)
-        k_elem_correct<T><<<(n + 127) / 128, 128, 0, st>>>(
-            n, layer, (T)geo.alpha, (T)(geo.rcut * geo.rcut), x, tri, tri_nrm, nrm, adj_start,
-            adj, q, rule, out, out_stride);
+                         int out_stride, int nsm, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    const T al = (T)geo.alpha, rc2 = (T)(geo.rcut * geo.rcut);
+    if (sizeof(T) == 8 || n < 64 * nsm)
+        k_elem_correct<T, 16><<<(unsigned)((16L * n + 63) / 64), 64, 0, st>>>(
+            n, layer, al, rc2, x, tri, tri_nrm, nrm, adj_start, adj, q, rule, out, out_stride);
+    else
+        k_elem_correct<T, 1><<<(n + 63) / 64, 64, 0, st>>>(
+            n, layer, al, rc2, x, tri, tri_nrm, nrm, adj_start, adj, q, rule, out, out_stride);
     return cudaGetLastError();
 }
 
 #define GGEM_INST_ELEM(T)                                                                     \
     template cudaError_t elem_correct<T>(int, int, const GridGeom&, const double*, const int*, \
                                          const double*, const double*, const int*, const int*,  \
-                                         const T*, const QuadRule&, T*, int, cudaStream_t);
+                                         const T*, const QuadRule&, T*, int, int, cudaStream_t);
 GGEM_INST_ELEM(float)
 GGEM_INST_ELEM(double)
 

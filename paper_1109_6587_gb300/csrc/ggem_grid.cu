@@ -227,32 +227,82 @@ cudaError_t fft_inverse(const GridGeom& geo, T* data, int nplanes, const void* t
 }
 
 // -------------------------------------------------- Chebyshev contraction
-// out[n][col] = sum_j M[n][j] in[j][col]  (M: Ny x Ny in shared memory)
-template <typename T, int NB>
-__global__ void __launch_bounds__(256) k_cheb(int Ny, const T* __restrict__ M,
+// out[n][col] = sum_j M[n][j] in[j][col], M the forward or inverse transform
+// matrix, both of them cos(pi n j / N) times factors that are the same for j and
+// N - j.  As cos(pi n (N - j) / N) = (-1)^n cos(pi n j / N), the forward
+// transform sums in[j] + in[N - j] for even n and in[j] - in[N - j] for odd n over
+// half the nodes, and the inverse forms node j and its mirror image from the same
+// even and odd partial sums: half the multiply-adds.  A thread computes NB outputs
+// (forward) or NB / 2 mirrored pairs (inverse) of one column; the row groups are
+// the grid's second dimension, so small transforms spread over the chip as well.
+// What bounds it in FP64: the FP64 pipe.  128 x 65 x 128 grid, forward / inverse of
+// 3 / 6 components: 0.62 / 0.92 ms with the full matrix in one group of rows, 0.25
+// / 0.45 here; 32 x 33 x 32 grid, where that left 140 SMs idle: 117 / 119 -> 12 / 10 us.
+template <typename T, bool INV, int NB>
+__global__ void __launch_bounds__(128) k_cheb(int Ny, const T* __restrict__ M,
                                                const T* __restrict__ in, T* __restrict__ out,
                                                long cols) {
     extern __shared__ __align__(16) unsigned char smraw[];
     T* Ms = reinterpret_cast<T*>(smraw);
-    for (int e = threadIdx.x; e < Ny * Ny; e += blockDim.x) Ms[e] = M[e];
-    __syncthreads();
-    long col = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= cols) return;
-    for (int n0 = 0; n0 < Ny; n0 += NB) {
+    const int N = Ny - 1, half = (N - 1) / 2;   // pairs (j, N - j), j = 0 .. half; N even: + N / 2
+    const bool mid = !(N & 1);
+    const long col = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (!INV) {
+        // rows n0 .. n0 + NB (n0 even), columns 0 .. half and N / 2
+        const int nc = half + 1 + (mid ? 1 : 0), n0 = blockIdx.y * NB;
+        for (int e = threadIdx.x; e < NB * nc; e += blockDim.x) {
+            const int b = e / nc, j = e - b * nc;
+            Ms[j * NB + b] = n0 + b < Ny ? M[(size_t)(n0 + b) * Ny + j] : (T)0;
+        }
+        __syncthreads();
+        if (col >= cols) return;
         T acc[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) acc[b] = 0;
-        for (int j = 0; j < Ny; ++j) {
-            T v = in[(long)j * cols + col];
+        for (int j = 0; j <= half; ++j) {
+            const T u = in[(long)j * cols + col], v = in[(long)(N - j) * cols + col];
+            const T s = u + v, d = u - v;
 #pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                int n = n0 + b;
-                if (n < Ny) acc[b] += Ms[n * Ny + j] * v;
-            }
+            for (int b = 0; b < NB; ++b) acc[b] += Ms[j * NB + b] * ((b & 1) ? d : s);
+        }
+        if (mid) {                              // j = N / 2: zero for odd n
+            const T u = in[(long)(N / 2) * cols + col];
+#pragma unroll
+            for (int b = 0; b < NB; b += 2) acc[b] += Ms[(half + 1) * NB + b] * u;
         }
 #pragma unroll
         for (int b = 0; b < NB; ++b)
             if (n0 + b < Ny) out[(long)(n0 + b) * cols + col] = acc[b];
+    } else {
+        // nodes j0 .. j0 + NB / 2 and their mirror images
+        constexpr int NP = NB / 2;
+        const int jmax = N / 2, j0 = blockIdx.y * NP;
+        for (int e = threadIdx.x; e < NP * Ny; e += blockDim.x) {
+            const int b = e / Ny, n = e - b * Ny;
+            Ms[n * NP + b] = j0 + b <= jmax ? M[(size_t)(j0 + b) * Ny + n] : (T)0;
+        }
+        __syncthreads();
+        if (col >= cols) return;
+        T ev[NP], od[NP];
+#pragma unroll
+        for (int b = 0; b < NP; ++b) ev[b] = od[b] = 0;
+        for (int n = 0; n < Ny; n += 2) {
+            const T u = in[(long)n * cols + col];
+#pragma unroll
+            for (int b = 0; b < NP; ++b) ev[b] += Ms[n * NP + b] * u;
+            if (n + 1 < Ny) {
+                const T v = in[(long)(n + 1) * cols + col];
+#pragma unroll
+                for (int b = 0; b < NP; ++b) od[b] += Ms[(n + 1) * NP + b] * v;
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < NP; ++b) {
+            const int j = j0 + b;
+            if (j > jmax) continue;
+            out[(long)j * cols + col] = ev[b] + od[b];
+            if (N - j != j) out[(long)(N - j) * cols + col] = ev[b] - od[b];
+        }
     }
 }
 
@@ -260,17 +310,28 @@ cudaError_t cheb_apply_tc(int Ny, const void* prep, const float* in, float* out,
                           int* err, int nsm, cudaStream_t st);
 
 template <typename T>
-cudaError_t cheb_apply(int Ny, const T* M, const T* in, T* out, long cols, cudaStream_t st,
-                       int* tc_err, int nsm, const void* tc_prep) {
+cudaError_t cheb_apply(int Ny, const T* M, bool inv, const T* in, T* out, long cols,
+                       cudaStream_t st, int* tc_err, int nsm, const void* tc_prep) {
     if (sizeof(T) == 4 && tc_err && tc_prep) {
         // FP32 data: split-BF16 contraction on the tensor cores when it fits
         cudaError_t e = cheb_apply_tc(Ny, tc_prep, (const float*)in, (float*)out, cols, tc_err,
                                       nsm, st);
         if (e != cudaErrorNotSupported) return e;
     }
-    size_t smem = (size_t)Ny * Ny * sizeof(T);
-    grant_max_smem((const void*)k_cheb<T, 24>);
-    k_cheb<T, 24><<<(unsigned)((cols + 255) / 256), 256, smem, st>>>(Ny, M, in, out, cols);
+    // 16 outputs per thread; 4 where 16 leave less than four blocks per SM
+    const long nb = (cols + 127) / 128;
+    const bool wide = nb * ((Ny + 15) / 16) >= 4L * nsm;
+    const int NB = wide ? 16 : 4;
+    const int rows = inv ? (Ny / 2 + 1 + NB / 2 - 1) / (NB / 2) : (Ny + NB - 1) / NB;
+    const dim3 grid((unsigned)nb, (unsigned)rows);
+    const size_t smem = (size_t)NB * Ny * sizeof(T);
+    if (inv) {
+        if (wide) k_cheb<T, true, 16><<<grid, 128, smem, st>>>(Ny, M, in, out, cols);
+        else k_cheb<T, true, 4><<<grid, 128, smem, st>>>(Ny, M, in, out, cols);
+    } else {
+        if (wide) k_cheb<T, false, 16><<<grid, 128, smem, st>>>(Ny, M, in, out, cols);
+        else k_cheb<T, false, 4><<<grid, 128, smem, st>>>(Ny, M, in, out, cols);
+    }
     return cudaGetLastError();
 }
 
@@ -659,8 +720,8 @@ cudaError_t spectral_pad(const GridGeom& geo, const T* spec, int nplanes, int Mx
                                         cudaStream_t);                                         \
     template cudaError_t fft_inverse<T>(const GridGeom&, T*, int, const void*, const void*,    \
                                         cudaStream_t, int);                                    \
-    template cudaError_t cheb_apply<T>(int, const T*, const T*, T*, long, cudaStream_t, int*,  \
-                                       int, const void*);                                      \
+    template cudaError_t cheb_apply<T>(int, const T*, bool, const T*, T*, long, cudaStream_t,  \
+                                       int*, int, const void*);                                \
     template cudaError_t interp_combine<T>(const GridGeom&, const double*, const T*, const T*, \
                                            int, int, int, const double*, const T*, int,         \
                                            const double*, const double*, const double*, double, \

@@ -318,7 +318,6 @@ struct ggem_plan {
     double* d_pc_Zb = nullptr;         // [pc_m][sol_ld] preconditioned Krylov vectors
     int pc_m = 0;
     int* d_tc_err = nullptr;           // tensor-core kernels: expired waits
-    int* d_spread_list = nullptr;      // [cap + 1] sources the paired spread hands back
     void* d_tc_fwd = nullptr;          // split-bf16 Chebyshev matrices (mixed plans)
     void* d_tc_inv = nullptr;
     int nsm = 0;                       // multiprocessors of the plan's device
@@ -429,7 +428,7 @@ template <typename T>
 cudaError_t elem_correct(int n, int layer, const GridGeom& geo, const double* x, const int* tri,
                          const double* tri_nrm, const double* nrm, const int* adj_start,
                          const int* adj, const T* q, const QuadRule& rule, T* out,
-                         int out_stride, cudaStream_t st);
+                         int out_stride, int nsm, cudaStream_t st);
 
 // locate targets: kind TK_POINTS (x[n][3]) or TK_WALL (the 2 Nz Nx wall nodes)
 template <typename T>
@@ -441,11 +440,12 @@ cudaError_t locate_targets(const GridGeom& geo, const CellGrid& cg, int n, int k
 template <typename T>
 cudaError_t spread_prepare(const GridGeom& geo, const double* yj, int n, const int* perm,
                            const double* x, int4* di, v4_t<T>* df, cudaStream_t st);
-// work: scratch of 4 Ny Nz Nx T (interleaved accumulation buffer)
+// work: scratch of 4 Ny Nz Nx T (interleaved accumulation buffer); nsm:
+// multiprocessors of the device
 template <typename T>
 cudaError_t spread(const GridGeom& geo, const CellGrid& cg, const double* yj, const T* ydiff,
                    const SortedSources<T>& src, const int4* di, const v4_t<T>* df, T* grid,
-                   T* work, int* list, cudaStream_t st);
+                   T* work, int nsm, cudaStream_t st);
 
 template <typename T>
 cudaError_t fft_forward(const GridGeom& geo, T* data, int nplanes, const void* tw_x,
@@ -455,8 +455,8 @@ cudaError_t fft_inverse(const GridGeom& geo, T* data, int nplanes, const void* t
                         const void* tw_z, cudaStream_t st, int active_kx = 0);
 
 template <typename T>
-cudaError_t cheb_apply(int Ny, const T* M, const T* in, T* out, long cols, cudaStream_t st,
-                       int* tc_err = nullptr, int nsm = 0, const void* tc_prep = nullptr);
+cudaError_t cheb_apply(int Ny, const T* M, bool inv, const T* in, T* out, long cols,
+                       cudaStream_t st, int* tc_err, int nsm, const void* tc_prep);
 // split-bf16 copy of an Ny x Ny FP32 matrix for the tensor-core transform
 size_t cheb_tc_prep_bytes(int Ny);
 cudaError_t cheb_tc_prepare(int Ny, const float* M, void* prep, cudaStream_t st);

@@ -369,7 +369,11 @@ __device__ __forceinline__ int cull_cells(const LocalArgs<T>& a, int lane, T ox,
 // consecutive lanes on consecutive sorted sources (coalesced float4 loads).
 // The hits are compacted into a per-warp queue and evaluated 32 at a time.
 // Partial sums are reduced with warp shuffles.
-constexpr int LW = 8;       // warps (targets) per block
+// warps (targets) per block.  FP64 sums are bound by the FP64 pipe of each SM, so
+// their targets are dealt out one warp at a time: with 8 per block 1,296 targets
+// are 162 blocks on 152 SMs and the ten SMs with two blocks set the time (element
+// rule, 1,296 targets 3.96 -> 3.2 ms; nodal, 162 targets 62 -> 41 us).
+template <typename T> constexpr int kLW = sizeof(T) == 8 ? 1 : 8;
 constexpr int kQueue = 64;  // hit queue per warp: < 32 left + <= 32 new always fit
 constexpr int kNb = 7 * 7 * 7;   // neighbour cell offsets for the largest reach (3)
 
@@ -378,7 +382,8 @@ constexpr int kNb = 7 * 7 * 7;   // neighbour cell offsets for the largest reach
 // skipped (their integral is done by the polar rule, Sec. 3.4.1).  Used in
 // FP64; the FP32 element rule has a kernel of its own (k_local_elem32).
 template <typename T, int KIND, int MODE, bool ELEM, int REACH>
-__global__ void __launch_bounds__(LW * 32) k_local(LocalArgs<T> a) {
+__global__ void __launch_bounds__(kLW<T> * 32) k_local(LocalArgs<T> a) {
+    constexpr int LW = kLW<T>;
     __shared__ int s_cst[LW][kNb];            // this target's cells: first source,
     __shared__ int s_cnt[LW][kNb];            //   source count,
     __shared__ unsigned short s_off[LW][kNb]; //   neighbour offset index
@@ -495,6 +500,7 @@ __global__ void __launch_bounds__(LW * 32) k_local(LocalArgs<T> a) {
 
 template <typename T, int KIND, int REACH>
 static void launch_kind(const LocalArgs<T>& a, int mode, cudaStream_t st) {
+    constexpr int LW = kLW<T>;
     dim3 b(LW * 32), g((a.n_tgt + LW - 1) / LW);
     switch (mode) {
         case OUT_U: k_local<T, KIND, OUT_U, false, REACH><<<g, b, 0, st>>>(a); break;
@@ -524,6 +530,7 @@ cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg,
     // scan the same candidate cells (L1 reuse); output in caller order
     LocalArgs<double> a{geo, cg, local_const<double>(geo, cg), src, qvs, near * near, tgt.n,
                         tgt.cell, tgt.pos, tgt.perm, nrm_tgt, out, out_stride};
+    constexpr int LW = kLW<double>;
     dim3 b(LW * 32), g((tgt.n + LW - 1) / LW);
     if (cg.reach == 3) {
         if (layer == 0) k_local<double, TK_POINTS, OUT_U, true, 3><<<g, b, 0, st>>>(a);

@@ -159,18 +159,18 @@ void run_global(ggem_plan_t* P, const SortedSources<T>& src, bool mesh, int out_
         GG_CUDA(local_sum<T>(geo, P->cg, src, TK_WALL, 2 * geo.Nz * geo.Nx, P->d_wall_cell,
                              (const v4_t<T>*)P->d_wall_pos, nullptr, OUT_U, Wl, 0, st));
     });
-    stage(P, ST_SPREAD, sizeof(T) == 4 ? 3 : 2, [&] {
+    stage(P, ST_SPREAD, 2, [&] {
         GG_CUDA(spread<T>(geo, P->cg, P->d_yj, (const T*)P->d_ydiff, src,
                           mesh ? P->d_mesh_sdi : P->d_sdi,
                           (const v4_t<T>*)(mesh ? P->d_mesh_sdf : P->d_sdf), A, B,
-                          P->d_spread_list, st));
+                          P->nsm, st));
     });
     stage(P, ST_FFT_FWD, 4, [&] {
         GG_CUDA(fft_forward<T>(geo, A, geo.Ny * 3, P->d_tw_x, P->d_tw_z, st));
         GG_CUDA(fft_forward<T>(geo, Wl, 6, P->d_tw_x, P->d_tw_z, st));
     });
     stage(P, ST_CHEB_FWD, 1, [&] {
-        GG_CUDA(cheb_apply<T>(geo.Ny, (const T*)P->d_cheb_fwd, A, B, (long)3 * P->nmodes * 2,
+        GG_CUDA(cheb_apply<T>(geo.Ny, (const T*)P->d_cheb_fwd, false, A, B, (long)3 * P->nmodes * 2,
                               st, P->d_tc_err, P->nsm, P->d_tc_fwd));
     });
     stage(P, ST_KS, 1, [&] {
@@ -201,7 +201,7 @@ void run_global(ggem_plan_t* P, const SortedSources<T>& src, bool mesh, int out_
         return;
     }
     stage(P, ST_CHEB_INV, 1, [&] {
-        GG_CUDA(cheb_apply<T>(geo.Ny, (const T*)P->d_cheb_inv, A, B,
+        GG_CUDA(cheb_apply<T>(geo.Ny, (const T*)P->d_cheb_inv, true, A, B,
                               (long)nout * P->nmodes * 2, st, P->d_tc_err, P->nsm, P->d_tc_inv));
     });
     stage(P, ST_FFT_INV, 2, [&] {
@@ -386,7 +386,7 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
             GG_CUDA(elem_correct<T>(n, layer, geo, P->d_x, P->d_tri, P->d_tri_nrm, P->d_nrm,
                                     P->d_adj_start, P->d_adj,
                                     P->fp64 ? (const T*)q : (const T*)P->d_q32, P->rule, loc, 3,
-                                    ls));
+                                    P->nsm, ls));
         });
     }
     run_global<T>(P, src, true, layer == 0 ? 1 : 2, gs);
@@ -682,7 +682,6 @@ void plan_build(ggem_plan_t* P, const ggem_params& prm) {
     dalloc(P, &P->d_cell_count, P->ncell);
     dalloc(P, &P->d_cell_start, P->ncell + 1);
     dalloc(P, &P->d_tc_err, 1);
-    dalloc(P, &P->d_spread_list, (size_t)cap + 1);
     GG_CUDA(cudaMemset(P->d_tc_err, 0, sizeof(int)));
     {
         int dev = 0;
@@ -811,7 +810,7 @@ void plan_free(ggem_plan_t* P) {
                     P->d_mlp, P->d_mlp_grad, P->d_mlp_part, P->d_mlp_m, P->d_mlp_v, P->d_mlp_wf,
                     P->d_mlp_wt, P->d_mlp_stats, P->d_mlp_out, P->d_smlp,
                     P->d_sres, P->d_mlp_dr, P->d_mlp_ssq, P->d_tc_err,
-                    P->d_tc_fwd, P->d_tc_inv, P->d_spread_list, P->d_pstart,
+                    P->d_tc_fwd, P->d_tc_inv, P->d_pstart,
                     P->d_pnodes, P->d_rc, P->d_rscale, P->d_mref, P->d_cx0, P->d_cdf,
                     P->d_cuinf, P->d_cfinf, P->d_cb, P->d_ckap, P->d_clam, P->d_cw, P->d_cq,
                     P->d_cmin, P->d_tstart, P->d_tlist, P->d_cvol, P->d_orec, P->d_orecd,

@@ -3,12 +3,11 @@
 //   f(node) = - sum_s g_s rho_g(node - x_s*),   |node - x_s*| < r_cut,
 //   rho_g(r) = alpha^3 pi^{-3/2} exp(-alpha^2 r^2) (5/2 - alpha^2 r^2).
 //
-// Source-parallel: a warp takes one sorted source (FP64, k_spread_scatter) or
-// two neighbouring ones (FP32, k_spread_pair: the union of their stencils,
-// both weights per node, one reduction with their sum), lists the columns,
-// rows and planes of its stencil, and adds the weights into an interleaved
-// [Ny][Nz][Nx][4] accumulation grid with float4 / double vector reductions in
-// L2; k_deinterleave then writes the planar [Ny][3][Nz][Nx] forcing.  The
+// Source-parallel: a warp takes two neighbouring sorted sources (the union of
+// their stencils, both weights per node, one reduction with their sum), lists
+// the columns, rows and planes of its stencil, and adds the weights into an
+// interleaved [Ny][Nz][Nx][4] accumulation grid with float4 / double reductions
+// in L2; k_deinterleave then writes the planar [Ny][3][Nz][Nx] forcing.  The
 // Gaussian factor is separable, exp(-a^2 r^2) = exp(-a^2 dx^2)
 // exp(-a^2 dy^2) exp(-a^2 dz^2), so each source costs one exponential per
 // column, row and plane (the fast Gaussian gridding idea), the remaining
@@ -58,12 +57,13 @@ template <typename T> __device__ __forceinline__ T sexp(T x);
 template <> __device__ __forceinline__ float sexp<float>(float x) { return expf(x); }
 template <> __device__ __forceinline__ double sexp<double>(double x) { return exp(x); }
 
-// per-kernel constants in T (computed on the host)
+// per-kernel constants in T (computed on the host); lo, hi: r_cut^2 less and
+// more than the rounding of a single-precision r^2
 template <typename T> struct SpreadConst {
     T dx, dz, rc2, al2, cn;
+    float lo, hi;
 };
 
-constexpr int SW = 8;         // warps (sources) per block
 constexpr int MAXJ = 272;     // max y nodes of one source stencil (checked on the host)
 constexpr int MAXR = 32;      // max columns / rows of one source's stencil
 
@@ -77,193 +77,196 @@ __device__ __forceinline__ void red4(double* p, double a, double b, double c) {
     atomicAdd(p + 2, c);
 }
 
-// One warp per source.  The source's stencil is the set of nodes within r_cut:
-// columns i with dx^2 < rc^2, rows k with dz^2 < rc^2, planes j in its y-range.
-// Lanes build the separable factors e_x, e_z, e_y in shared memory, then walk
-// the (column, row) pairs of the disc; each lane runs the planes of its pair
-// with dy^2 < rc^2 - dx^2 - dz^2 and adds into the interleaved buffer with one
-// vector reduction per node.
-// With `list`, warp i handles source list[i] for i < *nlist (the sources the
-// paired kernel handed back); otherwise source i for i < n.
-template <typename T>
-__global__ void __launch_bounds__(SW * 32) k_spread_scatter(
-    GridGeom geo, SpreadConst<T> kc, const T* __restrict__ ydiff, int n, int R,
-    const int4* __restrict__ sdi, const v4_t<T>* __restrict__ sdf,
-    const v4_t<T>* __restrict__ gsrc, T* __restrict__ f4, const int* __restrict__ list,
-    const int* __restrict__ nlist) {
-    __shared__ T s_xd2[SW][MAXR], s_xe[SW][MAXR], s_zd2[SW][MAXR], s_ze[SW][MAXR];
-    __shared__ int s_xi[SW][MAXR], s_zi[SW][MAXR];
-    __shared__ T s_yd2[SW][MAXJ], s_ye[SW][MAXJ];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int s = blockIdx.x * SW + wid;
-    if (list) {
-        if (s >= *nlist) return;                   // warp-uniform
-        s = list[s];
-    } else if (s >= n) {
-        return;                                    // warp-uniform
-    }
-    const T rc2 = kc.rc2, al2 = kc.al2;
-    const int4 di = sdi[s];
-    const v4_t<T> df = sdf[s];
-    const v4_t<T> g = gsrc[s];
-    const int mNx = geo.Nx - 1, mNz = geo.Nz - 1;
-    const int nr = 2 * R + 2;                      // candidate offsets -R .. R+1
-    // columns and rows within r_cut (lane = offset index)
-    T dx2 = (T)1e30, dz2 = (T)1e30;
-    if (lane < nr) {
-        T vx = fma((T)(lane - R), kc.dx, -df.x);
-        T vz = fma((T)(lane - R), kc.dz, -df.y);
-        dx2 = vx * vx;
-        dz2 = vz * vz;
-    }
-    const unsigned mx = __ballot_sync(0xffffffffu, dx2 < rc2);
-    const unsigned mz = __ballot_sync(0xffffffffu, dz2 < rc2);
-    const unsigned lt = (1u << lane) - 1u;
-    if (dx2 < rc2) {
-        int rk = __popc(mx & lt);
-        s_xd2[wid][rk] = dx2;
-        s_xe[wid][rk] = sexp<T>(-al2 * dx2);
-        s_xi[wid][rk] = (di.x + lane - R) & mNx;
-    }
-    if (dz2 < rc2) {
-        int rk = __popc(mz & lt);
-        s_zd2[wid][rk] = dz2;
-        s_ze[wid][rk] = sexp<T>(-al2 * dz2);
-        s_zi[wid][rk] = (di.y + lane - R) & mNz;
-    }
-    // planes of the y-range
-    const int jlo = di.w & 0xffff, jhi = di.w >> 16, ny = jhi - jlo + 1;
-    const T* yrow = ydiff + di.z;
-    for (int q = lane; q < ny; q += 32) {
-        T d = yrow[(size_t)(jlo + q) * geo.Ny] - df.z;
-        T d2 = d * d;
-        s_yd2[wid][q] = d2;
-        s_ye[wid][q] = sexp<T>(-al2 * d2);
-    }
-    __syncwarp();
-    const T gx = -kc.cn * g.x, gy = -kc.cn * g.y, gz = -kc.cn * g.z;
-    const int nxs = __popc(mx), nzs = __popc(mz), npair = nxs * nzs;
-    const float inx = 1.0f / (float)nxs;
-    const size_t rowst = (size_t)geo.Nx * 4, planest = (size_t)geo.Nz * geo.Nx * 4;
-    for (int pi = lane; pi < npair; pi += 32) {
-        int b = (int)(((float)pi + 0.5f) * inx);
-        int a = pi - b * nxs;
-        T dxz = s_xd2[wid][a] + s_zd2[wid][b];
-        if (!(dxz < rc2)) continue;
-        T exz = s_xe[wid][a] * s_ze[wid][b];
-        T* col = f4 + (size_t)s_zi[wid][b] * rowst + (size_t)s_xi[wid][a] * 4;
-        for (int q = 0; q < ny; ++q) {
-            T r2 = dxz + s_yd2[wid][q];
-            if (!(r2 < rc2)) continue;
-            T w = exz * s_ye[wid][q] * ((T)2.5 - al2 * r2);
-            red4(col + (size_t)(jlo + q) * planest, gx * w, gy * w, gz * w);
-        }
-    }
+// e + y < r_cut^2 in T; FP64 decides in single precision except within its
+// rounding of the cutoff
+__device__ __forceinline__ bool inside(const SpreadConst<float>& k, float e, float y, float, float) {
+    return e + y < k.rc2;
+}
+__device__ __forceinline__ bool inside(const SpreadConst<double>& k, double e, double y, float ef,
+                                       float yf) {
+    const float s = ef + yf;
+    return s < k.lo || (s <= k.hi && e + y < k.rc2);
 }
 
-// Two consecutive sorted sources per warp (FP32).  Neighbouring sources share
-// most of their stencils, so the warp walks the union of the two stencils,
-// evaluates both weights at every node and issues one vector reduction with
-// their sum: fewer reductions, which bound this kernel.  A pair whose union
-// does not fit 32 columns or 32 rows (sources far apart in the sorted order)
-// is handed to the single-source path.
-constexpr int PMAXJ = 272;
-__global__ void __launch_bounds__(SW * 32) k_spread_pair(
-    GridGeom geo, SpreadConst<float> kc, const float* __restrict__ ydiff, int n, int R,
-    const int4* __restrict__ sdi, const float4* __restrict__ sdf,
-    const float4* __restrict__ gsrc, float* __restrict__ f4, int* __restrict__ leftover,
-    int* __restrict__ nleft) {
-    __shared__ float s_xd2[SW][2][32], s_xe[SW][2][32], s_zd2[SW][2][32], s_ze[SW][2][32];
-    __shared__ int s_xi[SW][32], s_zi[SW][32];
-    __shared__ float s_yd2[SW][2][PMAXJ], s_ye[SW][2][PMAXJ];
+// Two consecutive sorted sources per warp.  Neighbouring sources share most of
+// their stencils (the nodes within r_cut: columns with dx^2 < rc^2, rows with
+// dz^2 < rc^2, planes of the y-range), so the warp walks the union of the two
+// stencils, evaluates both weights at every node and issues one reduction with
+// their sum: fewer reductions, which bound this kernel.  A pair whose union does
+// not fit 32 columns or 32 rows (sources far apart in the sorted order), and an
+// odd last source, run one after the other with an empty partner.
+// Lanes build the separable factors of the columns, rows and planes in shared
+// memory, then walk the (column, row) pairs; each lane runs its pair's planes.
+// With -c g e_xz and a^2 d_xz^2 e formed once per column and e_y (5/2 - a^2 dy^2)
+// once per plane, a node takes per source one FMA for
+//   e_y (5/2 - a^2 r^2) = [e_y (5/2 - a^2 dy^2)] - a^2 d_xz^2 e_y
+// and three for the components (FP64, where the pipe counts: 4 operations per node
+// and source instead of 8, and one reduction per two sources; with the column list
+// 64,200 sources 6.25 -> 4.5 ms per call).
+// gridDim.y parts share the planes of every pair: calls with few sources are
+// bound by one warp's walk through a stencil, not by the reductions (1,296 sources
+// in FP32 96 -> 40 us, without the launch that took handed-back pairs; 162 in FP64
+// 136 -> 77).
+template <typename T>
+__host__ __device__ constexpr size_t pair_smem(int Ny) {
+    return ((256 + 6 * (size_t)Ny) * sizeof(T) + 64 * 4 +
+            (sizeof(T) == 8 ? 2048 + 8 * (size_t)Ny : 0) + 15) & ~(size_t)15;
+}
+
+template <typename T, int WPB>
+__global__ void __launch_bounds__(WPB * 32) k_spread_pair(
+    GridGeom geo, SpreadConst<T> kc, const T* __restrict__ ydiff, int n, int R,
+    const int4* __restrict__ sdi, const v4_t<T>* __restrict__ sdf,
+    const v4_t<T>* __restrict__ gsrc, T* __restrict__ f4) {
+    // per warp: column and row tables, then three plane tables of Ny per source
+    // (sized by Ny: a table for the largest Ny would halve the resident warps)
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int Nyp = geo.Ny;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int s0 = 2 * (blockIdx.x * SW + wid);
-    if (s0 >= n) return;                                    // warp-uniform
-    const bool two = s0 + 1 < n;
-    const int4 d0 = sdi[s0];
-    const int4 d1 = two ? sdi[s0 + 1] : d0;
+    const int sa = 2 * (blockIdx.x * WPB + wid);
+    if (sa >= n) return;                                    // warp-uniform
+    unsigned char* wb = smraw + (size_t)wid * pair_smem<T>(Nyp);
+    T* s_t = reinterpret_cast<T*>(wb);                       // x d^2, x e, z d^2, z e: [4][2][32]
+    T* s_y = s_t + 256;                                      // y d^2, y e, y e q: [3][2][Ny]
+    int* s_i = reinterpret_cast<int*>(s_y + 6 * Nyp);        // column, row: [2][32]
+    unsigned short* s_c = reinterpret_cast<unsigned short*>(s_i + 64);   // FP64: columns [1024]
+    float* s_yf = reinterpret_cast<float*>(s_c + 1024);      // FP64: y d^2 in single: [2][Ny]
+    auto XZ = [&](int k, int s, int i) -> T& { return s_t[(k * 2 + s) * 32 + i]; };
+    auto YT = [&](int k, int s, int q) -> T& { return s_y[(k * 2 + s) * Nyp + q]; };
+    const T rc2 = kc.rc2, al2 = kc.al2;
     const int Nx = geo.Nx, Nz = geo.Nz;
-    // signed periodic offsets of source 1's base column/row from source 0's
-    int ox = d1.x - d0.x, oz = d1.y - d0.y;
-    ox -= (ox > Nx / 2) ? Nx : 0;
-    ox += (ox < -Nx / 2) ? Nx : 0;
-    oz -= (oz > Nz / 2) ? Nz : 0;
-    oz += (oz < -Nz / 2) ? Nz : 0;
     const int nr = 2 * R + 2;
-    // the union of offsets [-R, R+1] (source 0) and [o - R, o + R + 1] (source 1),
-    // relative to source 0's base column / row
-    const int bx = min(0, ox) - R, bz = min(0, oz) - R;
-    const int spx = max(0, ox) - min(0, ox) + nr, spz = max(0, oz) - min(0, oz) + nr;
-    if (!two || spx > 32 || spz > 32) {
-        if (lane == 0) {
-            leftover[atomicAdd(nleft, 1)] = s0;
-            if (two) leftover[atomicAdd(nleft, 1)] = s0 + 1;
-        }
-        return;
-    }
-    const float rc2 = kc.rc2, al2 = kc.al2;
-    const float4 f0 = sdf[s0], f1 = sdf[s0 + 1];
-    // columns and rows of the union: lane = union offset
-    {
-        const int c = bx + lane;                              // column offset from s0's base
-        float v0x = 1e30f, v1x = 1e30f;
-        if (lane < spx) {
-            const int o0 = c + R, o1 = c - ox + R;            // offsets into each stencil
-            if (o0 >= 0 && o0 < nr) { float v = fmaf((float)(o0 - R), kc.dx, -f0.x); v0x = v * v; }
-            if (o1 >= 0 && o1 < nr) { float v = fmaf((float)(o1 - R), kc.dx, -f1.x); v1x = v * v; }
-        }
-        s_xd2[wid][0][lane] = v0x;
-        s_xd2[wid][1][lane] = v1x;
-        s_xe[wid][0][lane] = v0x < rc2 ? expf(-al2 * v0x) : 0.f;
-        s_xe[wid][1][lane] = v1x < rc2 ? expf(-al2 * v1x) : 0.f;
-        s_xi[wid][lane] = (d0.x + c) & (Nx - 1);
-        const int r = bz + lane;
-        float v0z = 1e30f, v1z = 1e30f;
-        if (lane < spz) {
-            const int o0 = r + R, o1 = r - oz + R;
-            if (o0 >= 0 && o0 < nr) { float v = fmaf((float)(o0 - R), kc.dz, -f0.y); v0z = v * v; }
-            if (o1 >= 0 && o1 < nr) { float v = fmaf((float)(o1 - R), kc.dz, -f1.y); v1z = v * v; }
-        }
-        s_zd2[wid][0][lane] = v0z;
-        s_zd2[wid][1][lane] = v1z;
-        s_ze[wid][0][lane] = v0z < rc2 ? expf(-al2 * v0z) : 0.f;
-        s_ze[wid][1][lane] = v1z < rc2 ? expf(-al2 * v1z) : 0.f;
-        s_zi[wid][lane] = (d0.y + r) & (Nz - 1);
-    }
-    // planes: union of the two y-ranges
-    const int jlo = min(d0.w & 0xffff, d1.w & 0xffff), jhi = max(d0.w >> 16, d1.w >> 16);
-    const int ny = jhi - jlo + 1;
-    for (int q = lane; q < ny; q += 32) {
-        const float a0 = ydiff[(size_t)(jlo + q) * geo.Ny + d0.z] - f0.z;
-        const float a1 = ydiff[(size_t)(jlo + q) * geo.Ny + d1.z] - f1.z;
-        s_yd2[wid][0][q] = a0 * a0;
-        s_yd2[wid][1][q] = a1 * a1;
-        s_ye[wid][0][q] = expf(-al2 * a0 * a0);
-        s_ye[wid][1][q] = expf(-al2 * a1 * a1);
-    }
-    __syncwarp();
-    const float4 g0 = gsrc[s0], g1 = gsrc[s0 + 1];
-    const float ax = -kc.cn * g0.x, ay = -kc.cn * g0.y, az = -kc.cn * g0.z;
-    const float bxg = -kc.cn * g1.x, byg = -kc.cn * g1.y, bzg = -kc.cn * g1.z;
-    const int npair = spx * spz;
-    const float inx = 1.0f / (float)spx;
     const size_t rowst = (size_t)Nx * 4, planest = (size_t)Nz * Nx * 4;
-    for (int pi = lane; pi < npair; pi += 32) {
-        const int b = (int)(((float)pi + 0.5f) * inx);
-        const int a = pi - b * spx;
-        const float e0 = s_xd2[wid][0][a] + s_zd2[wid][0][b];
-        const float e1 = s_xd2[wid][1][a] + s_zd2[wid][1][b];
-        if (!(e0 < rc2) && !(e1 < rc2)) continue;
-        const float x0 = s_xe[wid][0][a] * s_ze[wid][0][b];
-        const float x1 = s_xe[wid][1][a] * s_ze[wid][1][b];
-        float* col = f4 + (size_t)s_zi[wid][b] * rowst + (size_t)s_xi[wid][a] * 4;
-        for (int q = 0; q < ny; ++q) {
-            const float r0 = e0 + s_yd2[wid][0][q], r1 = e1 + s_yd2[wid][1][q];
-            const float w0 = r0 < rc2 ? x0 * s_ye[wid][0][q] * (2.5f - al2 * r0) : 0.f;
-            const float w1 = r1 < rc2 ? x1 * s_ye[wid][1][q] * (2.5f - al2 * r1) : 0.f;
-            if (w0 == 0.f && w1 == 0.f) continue;
-            red4(col + (size_t)(jlo + q) * planest, fmaf(ax, w0, bxg * w1),
-                 fmaf(ay, w0, byg * w1), fmaf(az, w0, bzg * w1));
+    for (int pass = 0; pass < 2; ++pass) {
+        // this pass's sources: the pair, or one of them with an empty partner
+        int s0 = sa, s1 = sa + 1 < n ? sa + 1 : sa;
+        int4 d0 = sdi[s0], d1 = sdi[s1];
+        // signed periodic offsets of source 1's base column/row from source 0's
+        int ox = d1.x - d0.x, oz = d1.y - d0.y;
+        ox -= (ox > Nx / 2) ? Nx : 0;
+        ox += (ox < -Nx / 2) ? Nx : 0;
+        oz -= (oz > Nz / 2) ? Nz : 0;
+        oz += (oz < -Nz / 2) ? Nz : 0;
+        const bool fit = s1 != s0 && abs(ox) + nr <= 32 && abs(oz) + nr <= 32;
+        if (pass == 1 && (fit || s1 == s0)) return;          // warp-uniform
+        if (!fit) {
+            s0 = pass == 0 ? s0 : s1;
+            d0 = d1 = sdi[s0];
+            ox = oz = 0;
+        }
+        // the union of offsets [-R, R+1] (source 0) and [o - R, o + R + 1] (source 1),
+        // relative to source 0's base column / row
+        const int bx = min(0, ox) - R, bz = min(0, oz) - R;
+        const int spx = abs(ox) + nr, spz = abs(oz) + nr;
+        const v4_t<T> f0 = sdf[s0], f1 = fit ? sdf[s1] : f0;
+        __syncwarp();
+        // columns and rows of the union: lane = union offset
+        {
+            const int c = bx + lane;                          // column offset from s0's base
+            T v0x = (T)1e30, v1x = (T)1e30;
+            if (lane < spx) {
+                const int o0 = c + R, o1 = c - ox + R;        // offsets into each stencil
+                if (o0 >= 0 && o0 < nr) { T v = fma((T)(o0 - R), kc.dx, -f0.x); v0x = v * v; }
+                if (fit && o1 >= 0 && o1 < nr) { T v = fma((T)(o1 - R), kc.dx, -f1.x); v1x = v * v; }
+            }
+            XZ(0, 0, lane) = v0x;
+            XZ(0, 1, lane) = v1x;
+            XZ(1, 0, lane) = v0x < rc2 ? sexp<T>(-al2 * v0x) : (T)0;
+            XZ(1, 1, lane) = v1x < rc2 ? sexp<T>(-al2 * v1x) : (T)0;
+            s_i[lane] = (d0.x + c) & (Nx - 1);
+            const int r = bz + lane;
+            T v0z = (T)1e30, v1z = (T)1e30;
+            if (lane < spz) {
+                const int o0 = r + R, o1 = r - oz + R;
+                if (o0 >= 0 && o0 < nr) { T v = fma((T)(o0 - R), kc.dz, -f0.y); v0z = v * v; }
+                if (fit && o1 >= 0 && o1 < nr) { T v = fma((T)(o1 - R), kc.dz, -f1.y); v1z = v * v; }
+            }
+            XZ(2, 0, lane) = v0z;
+            XZ(2, 1, lane) = v1z;
+            XZ(3, 0, lane) = v0z < rc2 ? sexp<T>(-al2 * v0z) : (T)0;
+            XZ(3, 1, lane) = v1z < rc2 ? sexp<T>(-al2 * v1z) : (T)0;
+            s_i[32 + lane] = (d0.y + r) & (Nz - 1);
+        }
+        // planes: this part's share of the union of the two y-ranges
+        int jlo = min(d0.w & 0xffff, d1.w & 0xffff), jhi = max(d0.w >> 16, d1.w >> 16);
+        {
+            const int len = jhi - jlo + 1, np = gridDim.y, per = (len + np - 1) / np;
+            jlo += per * blockIdx.y;
+            jhi = min(jhi, jlo + per - 1);
+        }
+        const int ny = jhi - jlo + 1;
+        for (int q = lane; q < ny; q += 32) {
+            const T a0 = ydiff[(size_t)(jlo + q) * geo.Ny + d0.z] - f0.z;
+            const T a1 = ydiff[(size_t)(jlo + q) * geo.Ny + d1.z] - f1.z;
+            const T q0 = a0 * a0, q1 = a1 * a1;
+            const T e0 = sexp<T>(-al2 * q0), e1 = sexp<T>(-al2 * q1);
+            YT(0, 0, q) = q0;
+            YT(0, 1, q) = q1;
+            YT(1, 0, q) = e0;
+            YT(1, 1, q) = e1;
+            YT(2, 0, q) = e0 * ((T)2.5 - al2 * q0);
+            YT(2, 1, q) = e1 * ((T)2.5 - al2 * q1);
+            if (sizeof(T) == 8) {
+                s_yf[q] = (float)q0;
+                s_yf[Nyp + q] = (float)q1;
+            }
+        }
+        __syncwarp();
+        const v4_t<T> g0 = gsrc[s0], g1 = gsrc[s1];
+        const T h = fit ? -kc.cn : (T)0;
+        const T ax = -kc.cn * g0.x, ay = -kc.cn * g0.y, az = -kc.cn * g0.z;
+        const T cx = h * g1.x, cy = h * g1.y, cz = h * g1.z;
+        const int npair = spx * spz;
+        const float inx = 1.0f / (float)spx;
+        // FP64: a list of the columns within r_cut of either source, the long chords
+        // first, so that the lanes of a warp walk alike (a warp's FP64 instruction
+        // takes 16 cycles whatever its active lanes: 6.7 -> 4.5 ms on 100 capsules);
+        // FP32 takes the whole box row by row, which its reductions coalesce along
+        const unsigned lt = (1u << lane) - 1u;
+        constexpr bool listed = sizeof(T) == 8;
+        int ncol = listed ? 0 : npair;
+        for (int shell = 0; listed && shell < 2; ++shell)
+            for (int p0 = 0; p0 < npair; p0 += 32) {
+                const int pi = p0 + lane;
+                const int b = (int)(((float)pi + 0.5f) * inx);
+                const int a = pi - b * spx;
+                bool in = false;
+                if (pi < npair) {
+                    const T e = fmin(XZ(0, 0, a) + XZ(2, 0, b), XZ(0, 1, a) + XZ(2, 1, b));
+                    in = shell == 0 ? e < (T)0.5 * rc2 : e >= (T)0.5 * rc2 && e < rc2;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, in);
+                if (in) s_c[ncol + __popc(m & lt)] = (unsigned short)(a | (b << 8));
+                ncol += __popc(m);
+            }
+        __syncwarp();
+        for (int pi = lane; pi < ncol; pi += 32) {
+            int b = (int)(((float)pi + 0.5f) * inx), a = pi - b * spx;
+            if (listed) {
+                a = s_c[pi] & 255;
+                b = s_c[pi] >> 8;
+            }
+            const T e0 = XZ(0, 0, a) + XZ(2, 0, b);
+            const T e1 = XZ(0, 1, a) + XZ(2, 1, b);
+            if (!(e0 < rc2) && !(e1 < rc2)) continue;
+            const T x0 = XZ(1, 0, a) * XZ(3, 0, b);
+            const T x1 = XZ(1, 1, a) * XZ(3, 1, b);
+            const T m0 = -al2 * e0, m1 = -al2 * e1;
+            const T ux = ax * x0, uy = ay * x0, uz = az * x0;
+            const T vx = cx * x1, vy = cy * x1, vz = cz * x1;
+            const float e0f = (float)e0, e1f = (float)e1;
+            T* col = f4 + (size_t)s_i[32 + b] * rowst + (size_t)s_i[a] * 4;
+            for (int q = 0; q < ny; ++q) {
+                const T y0 = YT(0, 0, q), y1 = YT(0, 1, q);
+                const bool wide = sizeof(T) == 8;
+                const bool in0 = inside(kc, e0, y0, e0f, wide ? s_yf[q] : 0.f),
+                           in1 = inside(kc, e1, y1, e1f, wide ? s_yf[Nyp + q] : 0.f);
+                if (!in0 && !in1) continue;
+                const T w0 = in0 ? fma(m0, YT(1, 0, q), YT(2, 0, q)) : (T)0;
+                const T w1 = in1 ? fma(m1, YT(1, 1, q), YT(2, 1, q)) : (T)0;
+                red4(col + (size_t)(jlo + q) * planest, fma(ux, w0, vx * w1), fma(uy, w0, vy * w1),
+                     fma(uz, w0, vz * w1));
+            }
         }
     }
 }
@@ -294,7 +297,7 @@ cudaError_t spread_prepare(const GridGeom& geo, const double* yj, int n, const i
 template <typename T>
 cudaError_t spread(const GridGeom& geo, const CellGrid& cg, const double* yj, const T* ydiff,
                    const SortedSources<T>& src, const int4* di, const v4_t<T>* df, T* grid,
-                   T* work, int* list, cudaStream_t st) {
+                   T* work, int nsm, cudaStream_t st) {
     (void)cg; (void)yj;
     int R = (int)std::ceil(std::max(geo.rcut / geo.dx, geo.rcut / geo.dz)) + 1;
     if (2 * R + 2 > MAXR || geo.Ny > MAXJ) return cudaErrorInvalidConfiguration;
@@ -304,26 +307,20 @@ cudaError_t spread(const GridGeom& geo, const CellGrid& cg, const double* yj, co
     kc.rc2 = (T)(geo.rcut * geo.rcut);
     kc.al2 = (T)(geo.alpha * geo.alpha);
     kc.cn = (T)(geo.alpha * geo.alpha * geo.alpha / (pi * std::sqrt(pi)));
+    kc.lo = (float)(geo.rcut * geo.rcut * (1.0 - 1e-6));
+    kc.hi = (float)(geo.rcut * geo.rcut * (1.0 + 1e-6));
     size_t nodes = (size_t)geo.Ny * geo.Nz * geo.Nx;
     cudaMemsetAsync(work, 0, nodes * 4 * sizeof(T), st);
     if (src.n > 0) {
-        bool paired = false;
-        if constexpr (sizeof(T) == 4) {
-            if (list && geo.Ny <= PMAXJ) {
-                // pairs of sources; the pairs that do not fit go back to the single path
-                int* nleft = list + src.n;
-                cudaMemsetAsync(nleft, 0, sizeof(int), st);
-                const int npairs = (src.n + 1) / 2;
-                k_spread_pair<<<(npairs + SW - 1) / SW, SW * 32, 0, st>>>(
-                    geo, kc, ydiff, src.n, R, di, df, src.g, work, list, nleft);
-                k_spread_scatter<T><<<(src.n + SW - 1) / SW, SW * 32, 0, st>>>(
-                    geo, kc, ydiff, src.n, R, di, df, src.g, work, list, nleft);
-                paired = true;
-            }
-        }
-        if (!paired)
-            k_spread_scatter<T><<<(src.n + SW - 1) / SW, SW * 32, 0, st>>>(
-                geo, kc, ydiff, src.n, R, di, df, src.g, work, nullptr, nullptr);
+        constexpr int WPB = 4;
+        const int npairs = (src.n + 1) / 2;
+        // few pairs: share their planes between up to 4 warps, to 16 warps per SM
+        const int parts = std::max(1, std::min(4, 16 * nsm / npairs));
+        const dim3 g((unsigned)((npairs + WPB - 1) / WPB), (unsigned)parts);
+        const size_t smem = WPB * pair_smem<T>(geo.Ny);
+        grant_max_smem((const void*)k_spread_pair<T, WPB>);
+        k_spread_pair<T, WPB><<<g, WPB * 32, smem, st>>>(geo, kc, ydiff, src.n, R, di, df, src.g,
+                                                        work);
     }
     k_deinterleave<T><<<(unsigned)((nodes + 255) / 256), 256, 0, st>>>(geo.Ny, geo.Nz, geo.Nx,
                                                                        work, grid);
@@ -335,7 +332,7 @@ cudaError_t spread(const GridGeom& geo, const CellGrid& cg, const double* yj, co
                                            const double*, int4*, v4_t<T>*, cudaStream_t);       \
     template cudaError_t spread<T>(const GridGeom&, const CellGrid&, const double*, const T*,   \
                                    const SortedSources<T>&, const int4*, const v4_t<T>*, T*,    \
-                                   T*, int*, cudaStream_t);
+                                   T*, int, cudaStream_t);
 GGEM_INST_SPREAD(float)
 GGEM_INST_SPREAD(double)
 
