@@ -6,18 +6,22 @@
 // triangles once per quadrature rule:
 //   list 0  the 16 collapsed Gauss points of Eq. (int_l),
 //   list 1  the 7-point rule of degree 5 (Radon 1948),
+//   list 2  the 3-point rule of degree 2 (Strang and Fix 1973),
 // and each (target, cell) pair uses one of the lists: list 1 where the whole
-// cell is at least kFarEdges = 4 longest edges from the target, list 0
-// elsewhere.  Both rules integrate the same product of the linear density and
-// the kernel; over one triangle of edge h at distance d they differ by the
+// cell is at least kFarEdges = 4 longest edges from the target, list 2 where it
+// also is at least kDimRadius / alpha away, list 0 elsewhere.  The rules
+// integrate the same product of the linear density and the kernel; over one triangle of edge h at distance d they differ by the
 // kernel's Taylor terms beyond degree 4, of order (0.6 h / d)^5, and the kernel
 // falls off as exp(-alpha^2 d^2) besides.  Measured in FP64 with N(0,1)
 // densities on suspensions of 642- and 162-node spheres and biconcave cells, h / r_cut
 // from 0.02 to 0.16, the whole double-layer sums differ by (rms, over the rms
 // sum) 0.3e-8 to 1.1e-8 at 5 edges, 1.0e-8 to 5.5e-8 at 4 and 2.7e-8 to 1.3e-7 at
 // 3.5: at 4 the difference stays below the unit rounding of FP32 (6e-8), while
-// two orders of summation differ by 2e-7 to 7e-7.  In candidates per target the
-// list halves the work of dense suspensions and takes a third off dilute ones.
+// two orders of summation differ by 2e-7 to 7e-7.  List 2 lives on the kernel's
+// decay: beyond kDimRadius = 3 the terms carry exp(-9), and with alpha h <= 0.33
+// the sums differ by 6e-10 to 2.3e-8 (2.8: up to 5.2e-8; alpha h = 0.5: 2.2e-7,
+// where the list is not used).  In candidates per target the lists halve the work of
+// dense suspensions and take a third off dilute ones.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -30,8 +34,8 @@ namespace ggem {
 namespace {
 
 // ------------------------------------------------------------- the rules
-constexpr int kPts[kElemLists] = {16, 7};
-constexpr double kFarEdges = 4.0;
+constexpr int kPts[kElemLists] = {16, 7, 3};
+constexpr double kFarEdges = 4.0, kDimRadius = 3.0, kDimEdge = 0.33;
 
 // search reach in cells and its neighbour offsets
 constexpr int R32 = kElemReach, kSide = 2 * R32 + 1, kOffsets = kSide * kSide * kSide;
@@ -50,6 +54,13 @@ RuleTab rule_tab(int list, const QuadRule& g) {
             r.phi[a][1] = xi;
             r.phi[a][2] = eta;
             r.w[a] = g.w[a & 3] * g.w[a >> 2] * (1.0 - eta);
+        }
+        return r;
+    }
+    if (list == 2) {
+        for (int a = 0; a < 3; ++a) {
+            for (int v = 0; v < 3; ++v) r.phi[a][v] = v == a ? 2.0 / 3.0 : 1.0 / 6.0;
+            r.w[a] = 1.0 / 6.0;
         }
         return r;
     }
@@ -150,19 +161,25 @@ __global__ void k_step_map(int ncell, const int* __restrict__ start,
     for (int s = sstart[c], k = 0; s < sstart[c + 1]; ++s, ++k) map[s] = make_int4(a, b, 64 * k, 0);
 }
 
-// Neighbour lists of the cells that hold targets: the non-empty triangle cells
-// at offsets -R..R whose box comes within r_cut of the cell's box, as entries
-// (list 0: first step, steps; list 1: first step; offset index + steps of list
-// 1 << 10).  Dilute suspensions leave most of the (2R + 1)^3 neighbours empty
-// (30 to 90 of 343 are kept), and a list serves all targets of its cell, so
-// the sum's culling per target reads two or three rounds of 32 entries instead
-// of testing every offset.  A warp per cell; FILL writes the entries at start[c],
-// otherwise their number goes to cnt[c].
+// Neighbour lists of the cells that hold targets: the non-empty cells at
+// offsets -R..R whose box comes within r_cut of the cell's box, as entries (first
+// step of each list, triangles; or, over points alone, first point and points)
+// with their offset index apart.  Dilute suspensions leave most of the (2R + 1)^3
+// neighbours empty (30 to 90 of 343 are kept), and a list serves all targets of
+// its cell, so the sum's culling per target reads two or three rounds of 32
+// entries instead of testing every offset.  A warp per cell; FILL writes the
+// entries at start[c], otherwise their number goes to cnt[c].
+struct NbrSource {
+    const int* count_start;              // [ncell + 1] triangles (or points) of each cell
+    const int* sstart[kElemLists];       // first step of each cell (points: all null)
+    int base[kElemLists];
+};
+
 template <bool FILL>
 __global__ void k_neighbours(CellGrid cg, float hx, float hy, float hz, float reach2,
-                             const int* __restrict__ tgt_start, const int* __restrict__ ss0,
-                             const int* __restrict__ ss1, int base1, const int* __restrict__ start,
-                             int* __restrict__ cnt, int4* __restrict__ out) {
+                             const int* __restrict__ tgt_start, NbrSource src,
+                             const int* __restrict__ start, int* __restrict__ cnt,
+                             int4* __restrict__ out, unsigned short* __restrict__ off) {
     const int ncell = cg.ncx * cg.ncy * cg.ncz;
     const int c0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (c0 >= ncell) return;                     // warp-uniform
@@ -189,17 +206,23 @@ __global__ void k_neighbours(CellGrid cg, float hx, float hy, float hz, float re
                     czz += (czz < 0) ? cg.ncz : 0;
                     czz -= (czz >= cg.ncz) ? cg.ncz : 0;
                     const int c = (czz * cg.ncy + cyy) * cg.ncx + cxx;
-                    e.x = ss0[c];
-                    e.y = ss0[c + 1] - e.x;
-                    keep = e.y > 0;
+                    const int st = src.count_start[c], k = src.count_start[c + 1] - st;
+                    keep = k > 0;
                     if (FILL && keep) {
-                        e.z = ss1 ? base1 + ss1[c] : 0;
-                        e.w = oi | (ss1 ? (ss1[c + 1] - ss1[c]) << 10 : 0);
+                        if (src.sstart[0])
+                            e = make_int4(src.sstart[0][c], src.base[1] + src.sstart[1][c],
+                                          src.base[2] + src.sstart[2][c], k);
+                        else
+                            e = make_int4(st, 0, 0, k);
                     }
                 }
             }
             const unsigned m = __ballot_sync(0xffffffffu, keep);
-            if (FILL && keep) out[start[c0] + n + __popc(m & lt)] = e;
+            if (FILL && keep) {
+                const int slot = start[c0] + n + __popc(m & lt);
+                out[slot] = e;
+                off[slot] = (unsigned short)oi;
+            }
             n += __popc(m);
         }
     }
@@ -261,7 +284,7 @@ struct StrengthTab {
     float c[kElemLists][16][3];      // phi_v w
 };
 
-// strengths of both lists: a warp per step (list 0's steps first), a lane per
+// strengths of the lists: a warp per step (list 0's steps first), a lane per
 // slot pair, g = scale 2A sum_v (phi_v w) q_v.  The vertices come from the
 // sorted triangles (16 bytes per triangle, shared by its points), so the pass
 // moves little more than the strengths it writes: 1.05 ms per evaluation with
@@ -291,8 +314,9 @@ __device__ __forceinline__ void step_strengths(int lane, int4 mp, const int4* __
     o[64] = make_float4(g[0][1], g[1][1], g[0][2], g[1][2]);
 }
 
-__global__ void k_list_strengths(int n0, int n1, const int4* __restrict__ map0,
-                                 const int4* __restrict__ map1, const int4* __restrict__ tv,
+__global__ void k_list_strengths(int n0, int n1, int n2, const int4* __restrict__ map0,
+                                 const int4* __restrict__ map1, const int4* __restrict__ map2,
+                                 const int4* __restrict__ tv,
                                  const float* __restrict__ q, float scale, StrengthTab tab,
                                  float4* __restrict__ pack) {
     __shared__ float c[kElemLists][16][3];
@@ -300,10 +324,11 @@ __global__ void k_list_strengths(int n0, int n1, const int4* __restrict__ map0,
         (&c[0][0][0])[e] = (&tab.c[0][0][0])[e];
     __syncthreads();
     const int step = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (step >= n0 + n1) return;                 // warp-uniform
+    if (step >= n0 + n1 + n2) return;            // warp-uniform
     float4* o = pack + (size_t)step * 96 + lane;
     if (step < n0) step_strengths<kPts[0]>(lane, map0[step], tv, q, scale, c[0], o);
-    else step_strengths<kPts[1]>(lane, map1[step - n0], tv, q, scale, c[1], o);
+    else if (step < n0 + n1) step_strengths<kPts[1]>(lane, map1[step - n0], tv, q, scale, c[1], o);
+    else step_strengths<kPts[2]>(lane, map2[step - n0 - n1], tv, q, scale, c[2], o);
 }
 
 // --------------------------------------------------------------- the sum
@@ -392,7 +417,8 @@ struct Elem32Args {
     const int* tperm;                //   caller index
     const int* nstart;               // [ncell + 1] neighbour list of each target cell
     const int4* nbr;
-    float lim1;                      // squared distance from which a cell uses list 1
+    const unsigned short* noff;
+    float lim1, lim2;                // squared distances from which a cell uses lists 1, 2
     const int4* vert;                // list 0: vertices of each 16-slot group
     const double* nrm;               // [n][3] target normals (caller order)
     float* out;
@@ -420,7 +446,7 @@ __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, f
         int st = 0, cnt = 0, oi = 0;
         if (i + lane < end) {
             const int4 e = a.nbr[i + lane];
-            oi = e.w & 1023;
+            oi = a.noff[i + lane];
             const int ix = oi % kSide - R32, iy = (oi / kSide) % kSide - R32,
                       iz = oi / (kSide * kSide) - R32;
             const float gx = ix > 0 ? (float)ix * a.k.hx - ox
@@ -432,9 +458,11 @@ __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, f
             const float d2 = gx * gx + gy * gy + gz * gz;
             nearc = d2 <= near2;
             keep = d2 <= reach2;
-            const bool far = d2 >= a.lim1;
-            st = far ? e.z : e.x;
-            cnt = far ? e.w >> 10 : e.y;
+            // steps: the cell's points of the list, 64 at a time
+            const int l = d2 >= a.lim2 ? 2 : (d2 >= a.lim1 ? 1 : 0);
+            st = l == 2 ? e.z : (l == 1 ? e.y : e.x);
+            constexpr int p0 = kPts[0], p1 = kPts[1], p2 = kPts[2];
+            cnt = (e.w * (l == 2 ? p2 : (l == 1 ? p1 : p0)) + 63) >> 6;
         }
         const unsigned m = __ballot_sync(0xffffffffu, keep);
         if (keep) {
@@ -474,8 +502,9 @@ __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, f
 // is the number of candidates and the work per cell.  One launch, single and
 // double layer averaged, 4000 biconcave cells: 107.5 ms with every point of list
 // 0 and all 343 neighbour offsets tested per target; 76 ms with list 1 from 5
-// edges; 72.7 ms with the neighbour lists; 68.0 ms with list 1 from 4 edges.
-// 382 spheres at volume fraction 0.1, double layer: 23.6 -> 12.4 ms.  Cells of
+// edges; 72.7 ms with the neighbour lists; 68.0 ms with list 1 from 4 edges;
+// 66.4 ms with list 2.  382 spheres at volume fraction 0.1, double layer: 23.6 ->
+// 12.4 ms without list 2, 11.3 ms with it.  Cells of
 // r_cut / 4 or / 5 have fewer candidates and more cells: 145.7 and 148.1 against
 // 145.5 ms per two launches (list 1 from 5 edges).
 template <int LAYER>
@@ -573,7 +602,13 @@ float coord_scale(double alpha) { return (float)(alpha * 1.2011224087864498); }
 // A point of a triangle around the target can be farther from it than the
 // triangle's longest edge only by rounding; `near` carries that margin.  A far
 // cell never is a near one (kFarEdges > 1).
-double elem32_far_distance(double near_edge) { return kFarEdges * near_edge; }
+void elem32_far_distances(double near_edge, double alpha, double rcut, double* far) {
+    far[0] = 0.0;
+    far[1] = kFarEdges * near_edge;
+    far[2] = alpha * near_edge <= kDimEdge ? std::max(far[1], kDimRadius / alpha) : rcut;
+    for (int l = 1; l < kElemLists; ++l)
+        if (!(far[l] < 0.85 * rcut)) far[l] = INFINITY;
+}
 
 cudaError_t elem32_steps(const ElemLists32& L, int ncell, int* scratch, cudaStream_t st) {
     for (int l = 0; l < kElemLists; ++l) {
@@ -589,17 +624,22 @@ cudaError_t elem32_neighbours(const GridGeom& geo, const CellGrid& cg, const Ele
                               bool fill, cudaStream_t st) {
     const int ncell = cg.ncx * cg.ncy * cg.ncz;
     const float reach2 = (float)(geo.rcut * geo.rcut * 1.0002);
-    const int* ss0 = src_start ? src_start : L.sstart[0];
-    const int* ss1 = src_start ? nullptr : L.sstart[1];
+    NbrSource src{};
+    src.count_start = src_start ? src_start : L.tri_start;
+    for (int l = 0, base = 0; l < kElemLists && !src_start; ++l) {
+        src.sstart[l] = L.sstart[l];
+        src.base[l] = base;
+        base += L.nsteps[l];
+    }
+    const float hx = (float)cg.hx, hy = (float)cg.hy, hz = (float)cg.hz;
     const unsigned nb = (unsigned)((ncell + 7) / 8);
     if (fill) {
-        k_neighbours<true><<<nb, 256, 0, st>>>(cg, (float)cg.hx, (float)cg.hy, (float)cg.hz, reach2,
-                                              tgt_start, ss0, ss1, L.nsteps[0], L.nstart, nullptr,
-                                              L.nbr);
+        k_neighbours<true><<<nb, 256, 0, st>>>(cg, hx, hy, hz, reach2, tgt_start, src, L.nstart,
+                                              nullptr, L.nbr, L.noff);
         return cudaGetLastError();
     }
-    k_neighbours<false><<<nb, 256, 0, st>>>(cg, (float)cg.hx, (float)cg.hy, (float)cg.hz, reach2,
-                                           tgt_start, ss0, ss1, 0, nullptr, scratch, nullptr);
+    k_neighbours<false><<<nb, 256, 0, st>>>(cg, hx, hy, hz, reach2, tgt_start, src, nullptr,
+                                           scratch, nullptr, nullptr);
     return scan_counts(ncell, scratch, L.nstart, st);
 }
 
@@ -638,8 +678,11 @@ cudaError_t elem32_fill(const GridGeom& geo, const CellGrid& cg, const ElemLists
         if (l == 0)
             k_list_positions<kPts[0]><<<(ns + 7) / 8, 256, 0, st>>>(ns, L.map[0], L.tv, L.shift, x,
                                                                   tab, sc, pk, L.vert);
-        else
+        else if (l == 1)
             k_list_positions<kPts[1]><<<(ns + 7) / 8, 256, 0, st>>>(ns, L.map[1], L.tv, L.shift, x,
+                                                                  tab, sc, pk, nullptr);
+        else
+            k_list_positions<kPts[2]><<<(ns + 7) / 8, 256, 0, st>>>(ns, L.map[2], L.tv, L.shift, x,
                                                                   tab, sc, pk, nullptr);
         base += ns;
     }
@@ -656,11 +699,11 @@ cudaError_t elem32_strengths(const ElemLists32& L, const QuadRule& rule, int nno
         for (int a = 0; a < kPts[l]; ++a)
             for (int v = 0; v < 3; ++v) tab.c[l][a][v] = (float)(r.phi[a][v] * r.w[a]);
     }
-    const int ns = L.nsteps[0] + L.nsteps[1];
+    const int ns = L.nsteps[0] + L.nsteps[1] + L.nsteps[2];
     if (ns > 0)
-        k_list_strengths<<<(ns + 7) / 8, 256, 0, st>>>(L.nsteps[0], L.nsteps[1], L.map[0],
-                                                       L.map[1], L.tv, q32, (float)scale, tab,
-                                                       L.pack);
+        k_list_strengths<<<(ns + 7) / 8, 256, 0, st>>>(L.nsteps[0], L.nsteps[1], L.nsteps[2],
+                                                       L.map[0], L.map[1], L.map[2], L.tv, q32,
+                                                       (float)scale, tab, L.pack);
     return cudaGetLastError();
 }
 
@@ -677,7 +720,12 @@ cudaError_t elem32_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists3
     a.tperm = tgt.perm;
     a.nstart = L.nstart;
     a.nbr = L.nbr;
-    a.lim1 = L.nsteps[1] > 0 ? (float)(L.far * L.far * sc * sc) : 3e38f;
+    a.noff = L.noff;
+    float lim[kElemLists];
+    for (int l = 1; l < kElemLists; ++l)
+        lim[l] = L.nsteps[l] > 0 ? (float)(L.far[l] * L.far[l] * sc * sc) : 3e38f;
+    a.lim1 = lim[1];
+    a.lim2 = lim[2];
     a.vert = L.vert;
     a.nrm = nrm;
     a.out = out;

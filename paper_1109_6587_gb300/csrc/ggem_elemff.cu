@@ -79,6 +79,7 @@ struct FFArgs {
     const int* tperm;                //   caller index
     const int* nstart;               // neighbour lists of the target cells
     const int4* nbr;
+    const unsigned short* noff;
     const float4* hi;                // sorted points
     const float4* lo;
     const float4* g;
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(FW * 32, 6) k_local_elem_ff(FFArgs a) {
             int ix = 0, iy = 0, iz = 0;
             if (i + lane < nend) {
                 e = a.nbr[i + lane];
-                const int oi = e.w & 1023;
+                const int oi = a.noff[i + lane];
                 ix = oi % kSideF - RF;
                 iy = (oi / kSideF) % kSideF - RF;
                 iz = oi / (kSideF * kSideF) - RF;
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(FW * 32, 6) k_local_elem_ff(FFArgs a) {
             if (keep) {
                 const int slot = nc + __popc(mk & lt);
                 s_st[wid][slot] = e.x;
-                s_cnt[wid][slot] = e.y | (nearc ? (int)0x80000000 : 0);
+                s_cnt[wid][slot] = e.w | (nearc ? (int)0x80000000 : 0);
                 const ff tx = split_on_grid(ox - (ix + 0.5) * a.hx, a.mag),
                          ty = split_on_grid(oy - (iy + 0.5) * a.hy, a.mag),
                          tz = split_on_grid(oz - (iz + 0.5) * a.hz, a.mag);
@@ -326,6 +327,7 @@ cudaError_t elemff_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists3
     a.tperm = tgt.perm;
     a.nstart = L.nstart;
     a.nbr = L.nbr;
+    a.noff = L.noff;
     a.hi = hi;
     a.lo = lo;
     a.g = g;

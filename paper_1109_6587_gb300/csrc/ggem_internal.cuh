@@ -92,7 +92,7 @@ __device__ __forceinline__ void locate(const GridGeom& geo, const CellGrid& cg, 
 
 // FP32 element rule: point lists per quadrature rule of the triangles, binned
 // by centroid (ggem_elem32.cu).  Cells at least r_cut / kElemReach wide.
-constexpr int kElemLists = 2, kElemReach = 3;
+constexpr int kElemLists = 3, kElemReach = 3;
 struct ElemLists32 {
     int* tri_start = nullptr;             // [ncell + 1] sorted triangles of each cell
     int4* tv = nullptr;                   // [m] sorted triangles: vertices, 2A (float bits)
@@ -103,8 +103,9 @@ struct ElemLists32 {
     float4* pack = nullptr;               // [steps][3][32]: the lists one after the other
     int4* vert = nullptr;                 // [4 steps of list 0] vertices of each 16-slot group
     int* nstart = nullptr;                // [ncell + 1] neighbour list of each target cell
-    int4* nbr = nullptr;                  // its entries
-    double far = 0.0;                     // distance of a cell from which it uses list 1
+    int4* nbr = nullptr;                  // its entries: first step per list, triangles
+    unsigned short* noff = nullptr;       //   and offset index
+    double far[kElemLists] = {};          // distance of a cell from which it uses each list
 };
 
 // 4x4 Gauss-Legendre product rule on [0,1]^2 and the polar-rule angles
@@ -387,8 +388,8 @@ cudaError_t elem32_order(const GridGeom& geo, const CellGrid& cg, int m, const E
                          const int* tri, const double* tri_area, cudaStream_t st);
 cudaError_t elem32_steps(const ElemLists32& L, int ncell, int* scratch, cudaStream_t st);
 // neighbour lists of the cells with targets (tgt_start), of L's steps or, with
-// src_start, of the points sorted there (entries: first point, points, 0, offset
-// index): counts (scratch: ncell ints; fills nstart), or with `fill` the entries
+// src_start, of the points sorted there (entries: first point, 0, 0, points):
+// counts (scratch: ncell ints; fills nstart), or with `fill` the entries
 cudaError_t elem32_neighbours(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
                               const int* tgt_start, const int* src_start, int* scratch,
                               bool fill, cudaStream_t st);
@@ -399,8 +400,9 @@ cudaError_t elem32_strengths(const ElemLists32& L, const QuadRule& rule, int nno
 cudaError_t elem32_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
                        double near, const SortedSources<float>& tgt, const double* nrm, int layer,
                        float* out, int out_stride, cudaStream_t st);
-// distance of a cell from which the FP32 element rule uses list 1
-double elem32_far_distance(double near_edge);
+// distances of a cell from which the FP32 element rule uses each list (infinite:
+// the list is not built)
+void elem32_far_distances(double near_edge, double alpha, double rcut, double* far);
 cudaError_t gather_int4(int n, const int* perm, const int4* in, int4* out, cudaStream_t st);
 
 // exclusive scan of count[0..n) into start[0..n] (start[n] = total)

@@ -819,8 +819,9 @@ void plan_free(ggem_plan_t* P) {
                     P->d_spec_dz, P->d_spec_mid, P->d_spec_ct, P->d_mlp_tc,
                     P->d_mlp_tcs, P->d_q32, P->d_et_cen, P->d_et_cell,
                     P->d_et_perm, P->d_et_perm2, P->d_et_pos, P->el.tri_start, P->el.tv,
-                    P->el.shift, P->el.sstart[0], P->el.sstart[1], P->el.map[0], P->el.map[1],
-                    P->el.pack, P->el.vert, P->el.nstart, P->el.nbr};
+                    P->el.shift, P->el.sstart[0], P->el.sstart[1], P->el.sstart[2], P->el.map[0],
+                    P->el.map[1], P->el.map[2], P->el.pack, P->el.vert, P->el.nstart,
+                    P->el.nbr, P->el.noff};
     for (void* p : ptrs) dfree(p);
     precond_free(P);
     dfree(P->d_pc_Zb);
@@ -840,17 +841,20 @@ void neighbour_lists(ggem_plan_t* P, const int* src_start) {
     GG_CUDA(cudaStreamSynchronize(st));
     if ((size_t)n > P->nbr_cap) {
         dfree(L.nbr);
+        dfree(L.noff);
         L.nbr = nullptr;
+        L.noff = nullptr;
         P->nbr_cap = 0;
         dalloc(P, &L.nbr, (size_t)n + n / 8);
+        dalloc(P, &L.noff, (size_t)n + n / 8);
         P->nbr_cap = (size_t)n + n / 8;
     }
     GG_CUDA(elem32_neighbours(P->geo, P->cg, L, P->d_mesh_start, src_start, nullptr, true, st));
 }
 
 // FP32 element rule: the triangles (by centroid) into the cells, then the
-// neighbour lists of the mesh nodes' cells and the point lists, grown where the mesh needs more steps than they
-// hold.  List 1 is built where cells beyond its distance are common: at 0.85
+// neighbour lists of the mesh nodes' cells and the point lists, grown where the
+// mesh needs more steps than they hold.  A list is built where cells beyond its distance are common: at 0.85
 // r_cut and more the few percent of points it would save cost as much again in
 // strengths.
 void elem32_mesh(ggem_plan_t* P, int m) {
@@ -866,8 +870,9 @@ void elem32_mesh(ggem_plan_t* P, int m) {
         GG_CUDA(cudaMemcpyAsync(&L.nsteps[l], L.sstart[l] + P->ncell, sizeof(int),
                                 cudaMemcpyDeviceToHost, st));
     GG_CUDA(cudaStreamSynchronize(st));
-    L.far = elem32_far_distance(P->near_edge);
-    if (!(L.far < 0.85 * P->geo.rcut)) L.nsteps[1] = 0;
+    elem32_far_distances(P->near_edge, P->geo.alpha, P->geo.rcut, L.far);
+    for (int l = 1; l < kElemLists; ++l)
+        if (!std::isfinite(L.far[l])) L.nsteps[l] = 0;
     size_t total = 0;
     for (int l = 0; l < kElemLists; ++l) {
         const size_t ns = L.nsteps[l];

@@ -66,3 +66,27 @@ def test_lists_match_oracle(ggem, name):
         # a cancelling sum that these lists have no part in)
         if name != "one_triangle":
             assert_close(v, O.double_layer(s, q, quadrature="element", targets=tg), TOL_MIXED)
+
+
+@pytest.mark.parametrize("alpha_h", [0.32, 0.34])
+def test_dim_list_matches_oracle(ggem, alpha_h):
+    """The 3-point list on both sides of its rule (alpha times the longest edge
+    0.33), with most of the pairs beyond 3 / alpha."""
+    import torch
+    box = W.Box(16.0, 16.0, 6.0, -3.0, 32, 33, 32)
+    s = W.suspension(4, box, level=2, radius=0.9)
+    edge = max(np.linalg.norm(s.x[s.tri[:, i]] - s.x[s.tri[:, (i + 1) % 3]], axis=1).max()
+               for i in range(3))
+    alpha = alpha_h / edge
+    q = np.random.default_rng(6).standard_normal(s.x.shape)
+    P = ggem.Plan.for_box(box, alpha=alpha, precision="mixed", quadrature="element",
+                          max_points=len(s.x), max_tris=len(s.tri))
+    P.mesh_set(s.x, s.tri)
+    tg = np.arange(0, len(s.x), 5)
+    w = P.single_layer(torch.as_tensor(q, device="cuda")).cpu().numpy()[tg]
+    v = P.double_layer(torch.as_tensor(q, device="cuda")).cpu().numpy()[tg]
+    P.check()
+    P.close()
+    kw = dict(quadrature="element", targets=tg, alpha=alpha)
+    assert_close(w, O.single_layer(s, q, **kw), TOL_MIXED)
+    assert_close(v, O.double_layer(s, q, **kw), TOL_MIXED)
