@@ -15,12 +15,18 @@ i = 0 .. 72 (exp(-36) is below the last bit of a double): the Chebyshev
 interpolant at the first-kind points, in monomials, by mpmath at 50 digits;
 degrees 0..6 as float pairs, 7..9 as floats (their terms are below 2e-8).
 Run: python gen_fftab.py > ggem_fftab.cuh
+
+The FP64 sums take the same functions in doubles, of degree 10 (truncation below
+2e-17 of each function's largest value).
+Run: python gen_fftab.py fp64 > ggem_smooth64.cuh
 """
+import sys
+
 import mpmath as mp
 import numpy as np
 
 mp.mp.dps = 50
-NINT, DEG, PAIRS = 73, 9, 7
+NINT, DEG, PAIRS, DEG64 = 73, 9, 7, 10
 
 
 def smooth(m, s):
@@ -32,9 +38,9 @@ FUNCS = [lambda s: C * (smooth(0, s) + mp.exp(-s / 2)), lambda s: C * smooth(2, 
          lambda s: C * smooth(4, s) / 3, lambda s: C * mp.exp(-s / 2) / 6]
 
 
-def interpolant(f, i):
+def interpolant(f, i, deg=DEG):
     """Monomial coefficients in u of f(i + u), |u| <= 1/2."""
-    n = DEG + 1
+    n = deg + 1
     v = [mp.cos(mp.pi * (k + mp.mpf(1) / 2) / n) for k in range(n)]
     y = [f(i + x / 2) for x in v]
     c = [2 * mp.fsum(y[k] * mp.cos(j * mp.pi * (k + mp.mpf(1) / 2) / n) for k in range(n)) / n
@@ -88,5 +94,23 @@ def main():
     print("};")
 
 
+def main64():
+    print("// Generated by gen_fftab.py fp64 (mpmath, 50 digits): A_g, B_g, D_g, E_g on |s - i| <= 1/2,")
+    print("// degree %d in u = s - i.  kSmooth64[function][degree][interval]." % DEG64)
+    print("#pragma once")
+    print("#define GGEM_SMOOTH64_NINT %d" % NINT)
+    print("#define GGEM_SMOOTH64_DEG %d" % DEG64)
+    print("__device__ const double kSmooth64[4][%d][%d] = {" % (DEG64 + 1, NINT))
+    for f in FUNCS:
+        tab = [interpolant(f, i, DEG64) for i in range(NINT)]
+        print("    {")
+        for k in range(DEG64 + 1):
+            row = [float(tab[i][k]).hex() for i in range(NINT)]
+            print("        {" + ",\n         ".join(", ".join(row[j:j + 4])
+                                                    for j in range(0, NINT, 4)) + "},")
+        print("    },")
+    print("};")
+
+
 if __name__ == "__main__":
-    main()
+    main64() if sys.argv[1:] == ["fp64"] else main()

@@ -477,8 +477,9 @@ __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, f
     return nc;
 }
 
-// One warp per target (neighbouring targets in cell order).  The warp lists
-// the cells within r_cut and walks them in 64-point steps, every lane taking
+// S = 1: one warp per target (neighbouring targets in cell order); S = LWE: a
+// block per target, its warps taking the cells in turn.  The warp lists the
+// cells within r_cut and walks them in 64-point steps, every lane taking
 // two adjacent candidates and evaluating both with paired FP32 arithmetic: no
 // hit queue, as about 80 % of the candidates lie within r_cut.  A step is
 // 1,536 bytes in three rows of 32 lanes x 16 bytes (x0 x1 y0 y1 | z0 z1 gx0 gx1
@@ -507,15 +508,16 @@ __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, f
 // 12.4 ms without list 2, 11.3 ms with it.  Cells of
 // r_cut / 4 or / 5 have fewer candidates and more cells: 145.7 and 148.1 against
 // 145.5 ms per two launches (list 1 from 5 edges).
-template <int LAYER>
+template <int LAYER, int S>
 __global__ void __launch_bounds__(LWE * 32, 12) k_local_elem32(Elem32Args a,
                                                           const float4* __restrict__ pk) {
     __shared__ int s_st[LWE][kCap];
     __shared__ int s_cnt[LWE][kCap];
     __shared__ unsigned short s_off[LWE][kCap];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = blockIdx.x * LWE + wid;
-    if (t >= a.n_tgt) return;                     // warp-uniform
+    static_assert(S == 1 || S == LWE, "a target has one warp or a block");
+    const int t = S > 1 ? blockIdx.x : blockIdx.x * LWE + wid;
+    if (t >= a.n_tgt) return;                     // warp-uniform (S > 1: block-uniform)
     const float4 p = a.tpos[t];
     const int c = a.tcell[t], oidx = a.tperm[t];
     const int nend = a.nstart[c + 1];
@@ -532,7 +534,7 @@ __global__ void __launch_bounds__(LWE * 32, 12) k_local_elem32(Elem32Args a,
     for (int i = a.nstart[c]; i < nend;) {
         const int nc = cull_cells_batch(a, lane, ox, oy, oz, i, nend, s_st[wid], s_cnt[wid],
                                         s_off[wid]);
-        for (int ci = 0; ci < nc; ++ci) {
+        for (int ci = S > 1 ? wid : 0; ci < nc; ci += S) {
             const int st = s_st[wid][ci], end = st + s_cnt[wid][ci];
             const int oi = s_off[wid][ci] & 0x7fff;
             const bool nearc = s_off[wid][ci] >> 15;
@@ -586,6 +588,22 @@ __global__ void __launch_bounds__(LWE * 32, 12) k_local_elem32(Elem32Args a,
         ux += __shfl_xor_sync(0xffffffffu, ux, o);
         uy += __shfl_xor_sync(0xffffffffu, uy, o);
         uz += __shfl_xor_sync(0xffffffffu, uz, o);
+    }
+    if (S > 1) {
+        // the parts of the target's warps, added in order
+        __shared__ float s_part[LWE][3];
+        if (lane == 0) {
+            s_part[wid][0] = ux;
+            s_part[wid][1] = uy;
+            s_part[wid][2] = uz;
+        }
+        __syncthreads();
+        if (wid != 0) return;
+        for (int w = 1; w < S; ++w) {
+            ux += s_part[w][0];
+            uy += s_part[w][1];
+            uz += s_part[w][2];
+        }
     }
     if (lane == 0) {
         float* o = a.out + (size_t)oidx * a.out_stride;
@@ -709,7 +727,7 @@ cudaError_t elem32_strengths(const ElemLists32& L, const QuadRule& rule, int nno
 
 cudaError_t elem32_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
                        double near, const SortedSources<float>& tgt, const double* nrm, int layer,
-                       float* out, int out_stride, cudaStream_t st) {
+                       float* out, int out_stride, int nsm, cudaStream_t st) {
     if (tgt.n <= 0) return cudaSuccess;
     const double sp = 1.7724538509055160273, pi = 3.14159265358979323846, al = geo.alpha;
     const double sc = (double)coord_scale(al), c4 = 4.0 * al * al * al / sp;
@@ -747,11 +765,17 @@ cudaError_t elem32_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists3
     // shared-memory carveout (25 %: the 64 KB configuration) so that the rest
     // of the SM's 256 KB serves as L1 for the candidates the warps of a block
     // re-read (a preference; cheap per launch)
-    const void* kf = layer == 0 ? (const void*)k_local_elem32<0> : (const void*)k_local_elem32<1>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
-    const dim3 b(LWE * 32), g((tgt.n + LWE - 1) / LWE);
-    if (layer == 0) k_local_elem32<0><<<g, b, 0, st>>>(a, L.pack);
-    else k_local_elem32<1><<<g, b, 0, st>>>(a, L.pack);
+    // A block per target where there are few: four warps share its latencies and the
+    // SMs' shares even out.  One against four warps, double / single layer (us): 1,296
+    // targets 88 -> 43 / 90 -> 45, 5,184 133 -> 111 / 113 -> 107, 16,200 289 -> 262 / 246
+    // -> 246, 24,300 466 -> 436 / 397 -> 410, 64,200 on finer spheres 2.63 -> 2.66 / 2.18
+    // -> 2.57 ms: every warp culls the whole neighbour list, which a full chip feels.
+    const bool split = tgt.n <= 96 * nsm;
+    void (*kf)(Elem32Args, const float4*) =
+        split ? (layer == 0 ? k_local_elem32<0, LWE> : k_local_elem32<1, LWE>)
+              : (layer == 0 ? k_local_elem32<0, 1> : k_local_elem32<1, 1>);
+    cudaFuncSetAttribute((const void*)kf, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
+    kf<<<split ? tgt.n : (tgt.n + LWE - 1) / LWE, LWE * 32, 0, st>>>(a, L.pack);
     return cudaGetLastError();
 }
 

@@ -349,11 +349,12 @@ enum TargetKind { TK_SORTED = 0, TK_POINTS = 1, TK_WALL = 2 };
 enum { OUT_U = 1, OUT_S = 2, OUT_DBL = 4 };
 
 // targets: TK_SORTED = the sorted sources themselves (output via perm);
-// TK_POINTS / TK_WALL = targets located by locate_targets (cell, offsets)
+// TK_POINTS / TK_WALL = targets located by locate_targets (cell, offsets); nsm:
+// multiprocessors, by which few targets are told from many (0: one warp per target)
 template <typename T>
 cudaError_t local_sum(const GridGeom& geo, const CellGrid& cg, const SortedSources<T>& src,
                       int kind, int n_tgt, const int* tcell, const v4_t<T>* tpos,
-                      const double* nrm_tgt, int out_mode, T* out, int out_stride,
+                      const double* nrm_tgt, int out_mode, T* out, int out_stride, int nsm,
                       cudaStream_t st);
 
 // FP64 element rule: local sum over sorted quadrature points at the sorted
@@ -399,7 +400,7 @@ cudaError_t elem32_strengths(const ElemLists32& L, const QuadRule& rule, int nno
                              const double* q, float* q32, double scale, cudaStream_t st);
 cudaError_t elem32_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
                        double near, const SortedSources<float>& tgt, const double* nrm, int layer,
-                       float* out, int out_stride, cudaStream_t st);
+                       float* out, int out_stride, int nsm, cudaStream_t st);
 // distances of a cell from which the FP32 element rule uses each list (infinite:
 // the list is not built)
 void elem32_far_distances(double near_edge, double alpha, double rcut, double* far);

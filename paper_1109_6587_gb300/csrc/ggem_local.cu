@@ -9,7 +9,10 @@
 // most one image of a source lies within r_cut even where a small grid
 // visits a cell twice.
 #include "ggem_internal.cuh"
+#include <algorithm>
+
 #include "ggem_erfcx.cuh"
+#include "ggem_smooth64.cuh"
 
 namespace ggem {
 
@@ -140,6 +143,7 @@ cudaError_t gather_strengths(int n, const int* perm, const double* q, const doub
 template <typename T> struct LocalConst {
     T al, al2, rc2, c1, c2, c3, c4, fU, fS, hx, hy, hz;
     T ke;   // -alpha^2 log2(e): exp(-alpha^2 r^2) = 2^(ke r^2)
+    T s2, lam, lam3, lam5;   // FP64 tables: 2 alpha^2, powers of sqrt(2) alpha
 };
 
 template <typename T> LocalConst<T> local_const(const GridGeom& geo, const CellGrid& cg) {
@@ -152,6 +156,10 @@ template <typename T> LocalConst<T> local_const(const GridGeom& geo, const CellG
     k.fU = (T)(1.0 / (8.0 * pi * geo.mu)); k.fS = (T)(1.0 / (8.0 * pi));
     k.hx = (T)cg.hx; k.hy = (T)cg.hy; k.hz = (T)cg.hz;
     k.ke = (T)(-a * a * 1.4426950408889634074);
+    const double s2 = 2.0 * a * a, lam = a * 1.4142135623730950488;
+    k.s2 = (T)s2; k.lam = (T)lam; k.lam3 = (T)(s2 * lam); k.lam5 = (T)(s2 * s2 * lam);
+    // the tables end at s = 72.5, where the kernels are below 2e-17 of 1/r
+    if (sizeof(T) == 8) k.rc2 = (T)std::min((double)k.rc2, (GGEM_SMOOTH64_NINT - 0.6) / s2);
     return k;
 }
 
@@ -272,6 +280,70 @@ __device__ __forceinline__ void pair_terms(const LocalConst<T>& k, T dx, T dy, T
     }
 }
 
+// Two of the smooth parts A_g, B_g (F = 0) or D_g, E_g (F = 2) at s = 2 alpha^2 r^2.
+// The coefficients come through L1 (12 KB for the two; 20 loads of at most five
+// lines per 32 pairs, against some 900 cycles of FP64 arithmetic).
+template <int F>
+__device__ __forceinline__ void smooth64(double s2, double r2, double& p, double& q) {
+    const double m = fma(r2, s2, 6755399441055744.0);     // nearest integer in the low bits
+    const int i = __double2loint(m) & 127;
+    const double u = fma(r2, s2, -(m - 6755399441055744.0));
+    const double* a = &kSmooth64[F][0][0] + i;
+    const double* b = &kSmooth64[F + 1][0][0] + i;
+    constexpr int N = GGEM_SMOOTH64_NINT;
+    p = __ldg(a + GGEM_SMOOTH64_DEG * N);
+    q = __ldg(b + GGEM_SMOOTH64_DEG * N);
+#pragma unroll
+    for (int d = GGEM_SMOOTH64_DEG - 1; d >= 0; --d) {
+        p = fma(p, u, __ldg(a + d * N));
+        q = fma(q, u, __ldg(b + d * N));
+    }
+}
+
+// The same terms in FP64, one output kind at a time: the singular parts 1/r, 1/r^3,
+// 1/r^5 and the smooth ones from tables, no exponential and no erfc.  The double
+// layer is summed over 6 (the caller multiplies), its last term's scalar E x.g in
+// a.sxx.  About 55 FP64 instructions per pair where exp and erfcx took about 95:
+// element rule, 1,296 targets, 40,960 points 3.2 -> 2.0 ms.
+template <int MODE>
+__device__ __forceinline__ void pair_terms64(const LocalConst<double>& k, double dx, double dy,
+                                             double dz, double r2, const double4_32a& g,
+                                             double nx, double ny, double nz, PairAcc<double>& a) {
+    const double ir = rsqrt(r2), ir2 = ir * ir;
+    const double xg = fma(dz, g.z, fma(dy, g.y, dx * g.x));
+    double p, q;
+    if (MODE == OUT_U) {
+        smooth64<0>(k.s2, r2, p, q);
+        const double A = fma(-k.lam, p, ir), B = fma(-k.lam3, q, ir2 * ir) * xg;
+        a.ux = fma(B, dx, fma(A, g.x, a.ux));
+        a.uy = fma(B, dy, fma(A, g.y, a.uy));
+        a.uz = fma(B, dz, fma(A, g.z, a.uz));
+    } else {
+        smooth64<2>(k.s2, r2, p, q);
+        const double D = fma(k.lam5, p, -(ir2 * ir2 * ir)), E = k.lam3 * q;      // over 6
+        if (MODE == OUT_S) {
+            // d_i (D xg d_k + E g_k) + E g_i d_k, and E xg on the diagonal
+            const double Dx = D * xg, Ex = E * xg;
+            const double ex = E * g.x, ey = E * g.y, ez = E * g.z;
+            const double tx = fma(Dx, dx, ex), ty = fma(Dx, dy, ey), tz = fma(Dx, dz, ez);
+            a.sxx += fma(tx, dx, fma(ex, dx, Ex));
+            a.syy += fma(ty, dy, fma(ey, dy, Ex));
+            a.szz += fma(tz, dz, fma(ez, dz, Ex));
+            a.sxy += fma(ty, dx, ex * dy);
+            a.sxz += fma(tz, dx, ex * dz);
+            a.syz += fma(tz, dy, ey * dz);
+        } else {
+            const double xn = fma(dz, nz, fma(dy, ny, dx * nx));
+            const double gn = fma(g.z, nz, fma(g.y, ny, g.x * nx));
+            const double cd = fma(D * xg, xn, E * gn), cg = E * xn;
+            a.sxx = fma(E, xg, a.sxx);
+            a.ux = fma(cd, dx, fma(cg, g.x, a.ux));
+            a.uy = fma(cd, dy, fma(cg, g.y, a.uy));
+            a.uz = fma(cd, dz, fma(cg, g.z, a.uz));
+        }
+    }
+}
+
 // scaled output of one target in caller order
 template <typename T, int MODE>
 __device__ __forceinline__ void store_target(const LocalConst<T>& k, const PairAcc<T>& a, T* o) {
@@ -311,29 +383,34 @@ __device__ __forceinline__ void load_target(const LocalArgs<T>& a, int t, T& ox,
 
 // The warp's list of neighbour cells at offsets -R..R (cells are at least
 // r_cut/R wide): the non-empty ones whose nearest point lies within r_cut of
-// the target (a slightly widened r_cut, so rounding can only keep more).
-// Writes first source, count and offset index of each into the warp's
+// the target (a slightly widened r_cut, so FP32 rounding can only keep more).
+// Of S warps with the same target, warp w takes every S-th offset: neighbouring
+// cells go to different warps.  Writes first source, count and offset index of each into the warp's
 // shared-memory lists; returns their number (warp-uniform).
-template <typename T, int R>
-__device__ __forceinline__ int cull_cells(const LocalArgs<T>& a, int lane, T ox, T oy, T oz,
-                                          int cx, int cy, int cz, int* s_cst, int* s_cnt,
-                                          unsigned short* s_off) {
+template <typename T, int R, int S>
+__device__ __forceinline__ int cull_cells(const LocalArgs<T>& a, int w, int lane, float ox,
+                                          float oy, float oz, int cx, int cy, int cz,
+                                          int* s_cst, int* s_cnt, unsigned short* s_off) {
     const CellGrid& cg = a.cg;
     const unsigned lt = (1u << lane) - 1u;
-    const T reach2 = a.k.rc2 * (T)1.0001;
+    const float reach2 = (float)a.k.rc2 * 1.0001f;
+    const float hx = (float)a.k.hx, hy = (float)a.k.hy, hz = (float)a.k.hz;
     constexpr int side = 2 * R + 1, nb = side * side * side;
     int nc = 0;
-    for (int r = 0; r < (nb + 31) / 32; ++r) {
-        const int oi = r * 32 + lane;
+    for (int r = 0; r < (nb + 32 * S - 1) / (32 * S); ++r) {
+        const int oi = (r * 32 + lane) * S + w;
         bool keep = false;
         int st = 0, cnt = 0;
         if (oi < nb) {
             const int ix = oi % side - R, iy = (oi / side) % side - R, iz = oi / (side * side) - R;
             const int cyy = cy + iy;
             if (cyy >= 0 && cyy < cg.ncy) {
-                const T gx = ix > 0 ? (T)ix * a.k.hx - ox : (ix < 0 ? ox - (T)(ix + 1) * a.k.hx : (T)0);
-                const T gy = iy > 0 ? (T)iy * a.k.hy - oy : (iy < 0 ? oy - (T)(iy + 1) * a.k.hy : (T)0);
-                const T gz = iz > 0 ? (T)iz * a.k.hz - oz : (iz < 0 ? oz - (T)(iz + 1) * a.k.hz : (T)0);
+                const float gx = ix > 0 ? (float)ix * hx - ox
+                                        : (ix < 0 ? ox - (float)(ix + 1) * hx : 0.f);
+                const float gy = iy > 0 ? (float)iy * hy - oy
+                                        : (iy < 0 ? oy - (float)(iy + 1) * hy : 0.f);
+                const float gz = iz > 0 ? (float)iz * hz - oz
+                                        : (iz < 0 ? oz - (float)(iz + 1) * hz : 0.f);
                 if (gx * gx + gy * gy + gz * gz <= reach2) {
                     // ncx, ncz >= 2 R (L > 2 r_cut): one wrap suffices for |i| <= R
                     int cxx = cx + ix, czz = cz + iz;
@@ -361,19 +438,31 @@ __device__ __forceinline__ int cull_cells(const LocalArgs<T>& a, int lane, T ox,
     return nc;
 }
 
+// 0 < r2 < rc2 and r2 < lim, r2 a sum of squares or NaN.  In FP64 on the bit
+// patterns (non-negative doubles order like integers; NaN orders above all): an FP64
+// comparison costs as much as an addition.
+__device__ __forceinline__ bool in_range(float r2, float rc2) { return r2 < rc2 && r2 > 0.f; }
+__device__ __forceinline__ bool below(float r2, float lim) { return r2 < lim; }
+__device__ __forceinline__ bool in_range(double r2, double rc2) {
+    return (unsigned long long)__double_as_longlong(r2) - 1ull <
+           (unsigned long long)__double_as_longlong(rc2) - 1ull;
+}
+__device__ __forceinline__ bool below(double r2, double lim) {
+    return (unsigned long long)__double_as_longlong(r2) <
+           (unsigned long long)__double_as_longlong(lim);
+}
+
 // u_i = sum G^l_ij g_j ; sigma_ik = sum T^l_ijk g_j ; v_i = n_k sigma_ik
 // (unscaled in the loop; the caller-facing factors are applied at the end).
 //
-// One warp per target.  The warp lists the neighbour cells (offsets -R..R)
-// that come within r_cut of the target, then walks them one at a time with
+// One or four warps per target.  Each warp lists its neighbour cells (offsets
+// -R..R) that come within r_cut of the target, then walks them one at a time with
 // consecutive lanes on consecutive sorted sources (coalesced float4 loads).
 // The hits are compacted into a per-warp queue and evaluated 32 at a time.
-// Partial sums are reduced with warp shuffles.
-// warps (targets) per block.  FP64 sums are bound by the FP64 pipe of each SM, so
-// their targets are dealt out one warp at a time: with 8 per block 1,296 targets
-// are 162 blocks on 152 SMs and the ten SMs with two blocks set the time (element
-// rule, 1,296 targets 3.96 -> 3.2 ms; nodal, 162 targets 62 -> 41 us).
-template <typename T> constexpr int kLW = sizeof(T) == 8 ? 1 : 8;
+// Partial sums are reduced with warp shuffles, and over the warps of a target
+// in a fixed order.
+template <typename T> constexpr int kLW = sizeof(T) == 8 ? 1 : 8;   // warps per block, S = 1
+constexpr int kSplit = 4;   // warps per target, and per block, where targets are split
 constexpr int kQueue = 64;  // hit queue per warp: < 32 left + <= 32 new always fit
 constexpr int kNb = 7 * 7 * 7;   // neighbour cell offsets for the largest reach (3)
 
@@ -381,36 +470,44 @@ constexpr int kNb = 7 * 7 * 7;   // neighbour cell offsets for the largest reach
 // (caller index t); points of triangles having the target as a vertex are
 // skipped (their integral is done by the polar rule, Sec. 3.4.1).  Used in
 // FP64; the FP32 element rule has a kernel of its own (k_local_elem32).
-template <typename T, int KIND, int MODE, bool ELEM, int REACH>
-__global__ void __launch_bounds__(kLW<T> * 32) k_local(LocalArgs<T> a) {
-    constexpr int LW = kLW<T>;
-    __shared__ int s_cst[LW][kNb];            // this target's cells: first source,
-    __shared__ int s_cnt[LW][kNb];            //   source count,
-    __shared__ unsigned short s_off[LW][kNb]; //   neighbour offset index
+template <typename T, int KIND, int MODE, bool ELEM, int REACH, int S>
+__global__ void __launch_bounds__((S > 1 ? S : kLW<T>) * 32) k_local(LocalArgs<T> a) {
+    constexpr int LW = S > 1 ? S : kLW<T>, NB = (kNb + 32 * S - 1) / (32 * S) * 32;
+    constexpr bool TAB = sizeof(T) == 8 && MODE != (OUT_U | OUT_S);   // FP64 tables
+    constexpr bool ERF = sizeof(T) == 8 && !TAB;
+    __shared__ int s_cst[LW][NB];             // this warp's cells: first source,
+    __shared__ int s_cnt[LW][NB];             //   source count,
+    __shared__ unsigned short s_off[LW][NB];  //   neighbour offset index
     __shared__ v4_t<T> s_qd[LW][kQueue];     // queued hits: displacement, r^2
     __shared__ int s_qs[LW][kQueue];         // queued hits: sorted source index
-    __shared__ double s_tab[sizeof(T) == 8 ? (GGEM_ERFCX64_DEG + 1) * GGEM_ERFCX64_NINT : 1];
-    if (sizeof(T) == 8) {
+    __shared__ double s_tab[ERF ? (GGEM_ERFCX64_DEG + 1) * GGEM_ERFCX64_NINT : 1];
+    if (ERF) {
         for (int e = threadIdx.x; e < (GGEM_ERFCX64_DEG + 1) * GGEM_ERFCX64_NINT; e += blockDim.x)
             s_tab[e] = kErfcxTab64[e];
         __syncthreads();
     }
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = blockIdx.x * LW + wid;
-    if (t >= a.n_tgt) return;                     // warp-uniform
+    const int t = S > 1 ? blockIdx.x : blockIdx.x * LW + wid;
+    if (t >= a.n_tgt) return;                     // warp-uniform (S > 1: block-uniform)
     int cx, cy, cz, oidx;
     T ox, oy, oz;
     load_target<T, KIND>(a, t, ox, oy, oz, cx, cy, cz, oidx);
     constexpr int R = REACH, side = 2 * R + 1;
     const unsigned lt = (1u << lane) - 1u;
-    const int nc = cull_cells<T, R>(a, lane, ox, oy, oz, cx, cy, cz, s_cst[wid], s_cnt[wid],
-                                    s_off[wid]);
+    const int nc = cull_cells<T, R, S>(a, S > 1 ? wid : 0, lane, (float)ox, (float)oy, (float)oz,
+                                       cx, cy, cz, s_cst[wid], s_cnt[wid], s_off[wid]);
     T nx = 0, ny = 0, nz = 0;
     if (MODE & OUT_DBL) {
         nx = (T)a.nrm[3 * oidx]; ny = (T)a.nrm[3 * oidx + 1]; nz = (T)a.nrm[3 * oidx + 2];
     }
     const T rc2 = a.k.rc2;
     PairAcc<T> acc;
+    auto eval = [&](const v4_t<T>& d, const v4_t<T>& g) {
+        if constexpr (TAB)
+            pair_terms64<MODE>(a.k, d.x, d.y, d.z, d.w, g, nx, ny, nz, acc);
+        else
+            pair_terms<T, MODE>(a.k, d.x, d.y, d.z, d.w, g, nx, ny, nz, acc, s_tab);
+    };
     // Lanes test consecutive sources of one cell at a time; hits go to a
     // per-warp ring queue (ballot + popc ranks) and the pair arithmetic runs on
     // 32 queued hits at a time, so no lane idles through it on a miss.
@@ -433,8 +530,8 @@ __global__ void __launch_bounds__(kLW<T> * 32) k_local(LocalArgs<T> a) {
                 dy = ty - p.y;
                 dz = tz - p.z;
                 r2 = dx * dx + dy * dy + dz * dz;
-                hit = r2 < rc2 && r2 > (T)0;
-                if (ELEM && hit && r2 < a.near2) {
+                hit = in_range(r2, rc2);
+                if (ELEM && hit && below(r2, a.near2)) {
                     const int4 v = a.qvs[s];
                     hit = !(v.x == oidx || v.y == oidx || v.z == oidx);
                 }
@@ -452,8 +549,7 @@ __global__ void __launch_bounds__(kLW<T> * 32) k_local(LocalArgs<T> a) {
                 __syncwarp();
                 const int slot = (head + lane) & (kQueue - 1);
                 const v4_t<T> d = s_qd[wid][slot];
-                pair_terms<T, MODE>(a.k, d.x, d.y, d.z, d.w, a.src.g[s_qs[wid][slot]], nx, ny,
-                                    nz, acc, s_tab);
+                eval(d, a.src.g[s_qs[wid][slot]]);
                 head = (head + 32) & (kQueue - 1);
                 qn -= 32;
                 __syncwarp();
@@ -464,8 +560,17 @@ __global__ void __launch_bounds__(kLW<T> * 32) k_local(LocalArgs<T> a) {
     if (lane < qn) {
         const int slot = (head + lane) & (kQueue - 1);
         const v4_t<T> d = s_qd[wid][slot];
-        pair_terms<T, MODE>(a.k, d.x, d.y, d.z, d.w, a.src.g[s_qs[wid][slot]], nx, ny, nz, acc,
-                            s_tab);
+        eval(d, a.src.g[s_qs[wid][slot]]);
+    }
+    if (TAB && MODE == OUT_DBL) {
+        const T sn = acc.sxx;
+        acc.ux = (T)6 * (acc.ux + nx * sn);
+        acc.uy = (T)6 * (acc.uy + ny * sn);
+        acc.uz = (T)6 * (acc.uz + nz * sn);
+    }
+    if (TAB && MODE == OUT_S) {
+        acc.sxx *= (T)6; acc.sxy *= (T)6; acc.sxz *= (T)6;
+        acc.syy *= (T)6; acc.syz *= (T)6; acc.szz *= (T)6;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -483,6 +588,32 @@ __global__ void __launch_bounds__(kLW<T> * 32) k_local(LocalArgs<T> a) {
             acc.szz += __shfl_xor_sync(0xffffffffu, acc.szz, o);
         }
     }
+    if (S > 1) {
+        // lane 0 of every warp holds its part; the first warp's adds them in order
+        __shared__ T s_part[LW][9];
+        T* p = s_part[wid];
+        if (lane == 0) {
+            if (MODE & (OUT_U | OUT_DBL)) {
+                p[0] = acc.ux; p[1] = acc.uy; p[2] = acc.uz;
+            }
+            if (MODE & OUT_S) {
+                p[3] = acc.sxx; p[4] = acc.sxy; p[5] = acc.sxz;
+                p[6] = acc.syy; p[7] = acc.syz; p[8] = acc.szz;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x != 0) return;
+        for (int w = 1; w < LW; ++w) {
+            const T* o = s_part[w];
+            if (MODE & (OUT_U | OUT_DBL)) {
+                acc.ux += o[0]; acc.uy += o[1]; acc.uz += o[2];
+            }
+            if (MODE & OUT_S) {
+                acc.sxx += o[3]; acc.sxy += o[4]; acc.sxz += o[5];
+                acc.syy += o[6]; acc.syz += o[7]; acc.szz += o[8];
+            }
+        }
+    }
     if (lane != 0) return;
     if (KIND == TK_WALL) {
         // global wall data u^g = -u^l (Sec. 3.2.2), layout [wall][c][Nz][Nx]
@@ -498,17 +629,39 @@ __global__ void __launch_bounds__(kLW<T> * 32) k_local(LocalArgs<T> a) {
     store_target<T, MODE>(a.k, acc, a.out + (size_t)oidx * a.out_stride);
 }
 
-template <typename T, int KIND, int REACH>
-static void launch_kind(const LocalArgs<T>& a, int mode, cudaStream_t st) {
+// Whether a target's cells are split over the kSplit warps of a block.  A call with few
+// targets is a chain of latencies, which four warps share; with many targets the
+// chip is full and four partly filled last batches cost more than one.
+// FP32, one against four warps: 1,296 nodal targets 21.2 -> 14.9 us, 2,592 20.9 ->
+// 18.9, 5,184 33.3 -> 35.2, 10,368 39.9 -> 45.9; free targets 2,000 33.9 -> 30.0,
+// 100,000 1.87 -> 1.83 ms (20,000 sources) and .60 -> .73 (1,000).  FP64 sums fill
+// the FP64 pipe with a few warps per SM: 162 targets 35 -> 18 us, 648 40 -> 42,
+// 1,296 80 -> 88.
+template <typename T> static bool split_targets(int n_tgt, int nsm) {
+    return n_tgt <= (sizeof(T) == 8 ? 2 : 24) * nsm;
+}
+
+template <typename T, int KIND, int MODE, int REACH>
+static void launch_split(const LocalArgs<T>& a, bool split, cudaStream_t st) {
     constexpr int LW = kLW<T>;
-    dim3 b(LW * 32), g((a.n_tgt + LW - 1) / LW);
+    if (split)
+        k_local<T, KIND, MODE, false, REACH, kSplit><<<a.n_tgt, kSplit * 32, 0, st>>>(a);
+    else
+        k_local<T, KIND, MODE, false, REACH, 1><<<(a.n_tgt + LW - 1) / LW, LW * 32, 0, st>>>(a);
+}
+
+template <typename T, int KIND, int REACH>
+static void launch_kind(const LocalArgs<T>& a, int mode, int nsm, cudaStream_t st) {
+    const bool sp = split_targets<T>(a.n_tgt, nsm);
+    if (KIND == TK_WALL) {
+        launch_split<T, KIND, OUT_U, REACH>(a, sp, st);
+        return;
+    }
     switch (mode) {
-        case OUT_U: k_local<T, KIND, OUT_U, false, REACH><<<g, b, 0, st>>>(a); break;
-        case OUT_S: k_local<T, KIND, OUT_S, false, REACH><<<g, b, 0, st>>>(a); break;
-        case OUT_U | OUT_S:
-            k_local<T, KIND, OUT_U | OUT_S, false, REACH><<<g, b, 0, st>>>(a);
-            break;
-        case OUT_DBL: k_local<T, KIND, OUT_DBL, false, REACH><<<g, b, 0, st>>>(a); break;
+        case OUT_U: launch_split<T, KIND, OUT_U, REACH>(a, sp, st); break;
+        case OUT_S: launch_split<T, KIND, OUT_S, REACH>(a, sp, st); break;
+        case OUT_U | OUT_S: launch_split<T, KIND, OUT_U | OUT_S, REACH>(a, sp, st); break;
+        case OUT_DBL: launch_split<T, KIND, OUT_DBL, REACH>(a, sp, st); break;
         default: break;
     }
 }
@@ -516,28 +669,35 @@ static void launch_kind(const LocalArgs<T>& a, int mode, cudaStream_t st) {
 // the grid's search reach as a compile-time constant (cells >= r_cut/2 or
 // r_cut/3; grids of larger cells use reach 2)
 template <typename T, int KIND>
-static void launch_kind(const LocalArgs<T>& a, int mode, cudaStream_t st) {
-    if (a.cg.reach == 3) launch_kind<T, KIND, 3>(a, mode, st);
-    else launch_kind<T, KIND, 2>(a, mode, st);
+static void launch_kind(const LocalArgs<T>& a, int mode, int nsm, cudaStream_t st) {
+    if (a.cg.reach == 3) launch_kind<T, KIND, 3>(a, mode, nsm, st);
+    else launch_kind<T, KIND, 2>(a, mode, nsm, st);
 }
 
+template <int LAYER, int REACH>
+static void launch_elem(const LocalArgs<double>& a, cudaStream_t st) {
+    k_local<double, TK_POINTS, LAYER == 0 ? OUT_U : OUT_DBL, true, REACH, kSplit>
+        <<<a.n_tgt, kSplit * 32, 0, st>>>(a);
+}
+
+// Always four warps per target: the 16 points per triangle give each plenty of pairs, and
+// the SMs' shares of the targets even out (1,296 targets 2.04 -> 1.88 ms, 648
+// .66 -> .50, 16,200 18.4 -> 16.4).
 cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg,
                            const SortedSources<double>& src, const int4* qvs, double near,
                            const SortedSources<double>& tgt, const double* nrm_tgt, int layer,
                            double* out, int out_stride, cudaStream_t st) {
     if (tgt.n <= 0) return cudaSuccess;
-    // targets: the mesh nodes in cell order, so the warps of a block mostly
-    // scan the same candidate cells (L1 reuse); output in caller order
+    // targets: the mesh nodes in cell order, so neighbouring blocks mostly scan
+    // the same candidate cells (L1 / L2 reuse); output in caller order
     LocalArgs<double> a{geo, cg, local_const<double>(geo, cg), src, qvs, near * near, tgt.n,
                         tgt.cell, tgt.pos, tgt.perm, nrm_tgt, out, out_stride};
-    constexpr int LW = kLW<double>;
-    dim3 b(LW * 32), g((tgt.n + LW - 1) / LW);
     if (cg.reach == 3) {
-        if (layer == 0) k_local<double, TK_POINTS, OUT_U, true, 3><<<g, b, 0, st>>>(a);
-        else k_local<double, TK_POINTS, OUT_DBL, true, 3><<<g, b, 0, st>>>(a);
+        if (layer == 0) launch_elem<0, 3>(a, st);
+        else launch_elem<1, 3>(a, st);
     } else {
-        if (layer == 0) k_local<double, TK_POINTS, OUT_U, true, 2><<<g, b, 0, st>>>(a);
-        else k_local<double, TK_POINTS, OUT_DBL, true, 2><<<g, b, 0, st>>>(a);
+        if (layer == 0) launch_elem<0, 2>(a, st);
+        else launch_elem<1, 2>(a, st);
     }
     return cudaGetLastError();
 }
@@ -545,14 +705,14 @@ cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg,
 template <typename T>
 cudaError_t local_sum(const GridGeom& geo, const CellGrid& cg, const SortedSources<T>& src,
                       int kind, int n_tgt, const int* tcell, const v4_t<T>* tpos,
-                      const double* nrm_tgt, int out_mode, T* out, int out_stride,
+                      const double* nrm_tgt, int out_mode, T* out, int out_stride, int nsm,
                       cudaStream_t st) {
     if (n_tgt <= 0) return cudaSuccess;
     LocalArgs<T> a{geo, cg, local_const<T>(geo, cg), src, nullptr, (T)0, n_tgt, tcell, tpos,
                    nullptr, nrm_tgt, out, out_stride};
-    if (kind == TK_SORTED) launch_kind<T, TK_SORTED>(a, out_mode, st);
-    else if (kind == TK_POINTS) launch_kind<T, TK_POINTS>(a, out_mode, st);
-    else launch_kind<T, TK_WALL>(a, OUT_U, st);
+    if (kind == TK_SORTED) launch_kind<T, TK_SORTED>(a, out_mode, nsm, st);
+    else if (kind == TK_POINTS) launch_kind<T, TK_POINTS>(a, out_mode, nsm, st);
+    else launch_kind<T, TK_WALL>(a, OUT_U, nsm, st);
     return cudaGetLastError();
 }
 
@@ -563,7 +723,7 @@ cudaError_t local_sum(const GridGeom& geo, const CellGrid& cg, const SortedSourc
                                              double, v4_t<T>*, cudaStream_t);                  \
     template cudaError_t local_sum<T>(const GridGeom&, const CellGrid&,                       \
                                       const SortedSources<T>&, int, int, const int*,          \
-                                      const v4_t<T>*, const double*, int, T*, int,             \
+                                      const v4_t<T>*, const double*, int, T*, int, int,        \
                                       cudaStream_t);                                           \
     template cudaError_t locate_targets<T>(const GridGeom&, const CellGrid&, int, int,        \
                                            const double*, int*, v4_t<T>*, cudaStream_t);

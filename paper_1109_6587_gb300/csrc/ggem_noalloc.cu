@@ -177,7 +177,7 @@ extern "C" ggem_status ggem_local_velocity_noalloc(const ggem_params* prm, void*
     SortedSources<double> src{pos, gs, cell, perm, start, n_src};
     if (tgt_is_src) {
         if (local_sum<double>(geo, cg, src, TK_SORTED, n_tgt, nullptr, nullptr, nullptr, OUT_U,
-                              u, 3, st) != cudaSuccess)
+                              u, 3, 0, st) != cudaSuccess)
             return GGEM_ERR_CUDA;
         return GGEM_OK;
     }
@@ -188,7 +188,7 @@ extern "C" ggem_status ggem_local_velocity_noalloc(const ggem_params* prm, void*
                                    st) != cudaSuccess)
             return GGEM_ERR_CUDA;
         if (local_sum<double>(geo, cg, src, TK_POINTS, nt, tcell, tpos, nullptr, OUT_U,
-                              u + 3 * (size_t)t0, 3, st) != cudaSuccess)
+                              u + 3 * (size_t)t0, 3, 0, st) != cudaSuccess)
             return GGEM_ERR_CUDA;
     }
     return GGEM_OK;

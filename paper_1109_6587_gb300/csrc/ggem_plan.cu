@@ -157,7 +157,8 @@ void run_global(ggem_plan_t* P, const SortedSources<T>& src, bool mesh, int out_
     T* Wl = (T*)P->d_wall;
     stage(P, ST_WALL, 1, [&] {
         GG_CUDA(local_sum<T>(geo, P->cg, src, TK_WALL, 2 * geo.Nz * geo.Nx, P->d_wall_cell,
-                             (const v4_t<T>*)P->d_wall_pos, nullptr, OUT_U, Wl, 0, st));
+                             (const v4_t<T>*)P->d_wall_pos, nullptr, OUT_U, Wl, 0, P->nsm,
+                             st));
     });
     stage(P, ST_SPREAD, 2, [&] {
         GG_CUDA(spread<T>(geo, P->cg, P->d_yj, (const T*)P->d_ydiff, src,
@@ -234,7 +235,8 @@ void point_forces_impl(ggem_plan_t* P, int n_src, const double* xs, const double
                                       (v4_t<T>*)P->d_tgt_pos, st));
         GG_CUDA(local_sum<T>(geo, P->cg, src, tgt_is_src ? TK_SORTED : TK_POINTS,
                              tgt_is_src ? n_src : n_tgt, P->d_tgt_cell,
-                             (const v4_t<T>*)P->d_tgt_pos, nullptr, mode, loc, stride, st));
+                             (const v4_t<T>*)P->d_tgt_pos, nullptr, mode, loc, stride, P->nsm,
+                             st));
     });
     int sel = (u ? 1 : 0) | (s ? 2 : 0);
     run_global<T>(P, src, false, sel, P->st);
@@ -308,7 +310,7 @@ void local_only_impl(ggem_plan_t* P, int n_src, const double* xs, const double* 
                                       (v4_t<T>*)P->d_tgt_pos, st));
         GG_CUDA(local_sum<T>(geo, P->cg, src, tgt_is_src ? TK_SORTED : TK_POINTS, nt,
                              P->d_tgt_cell, (const v4_t<T>*)P->d_tgt_pos, nullptr, mode, loc,
-                             stride, st));
+                             stride, P->nsm, st));
         if (nt > 0) k_split_local<T><<<(nt + 255) / 256, 256, 0, st>>>(nt, loc, stride, u, s);
         GG_CUDA(cudaGetLastError());
     });
@@ -354,7 +356,7 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
     if (!elem) {
         stage(P, ST_LOCAL, 1, [&] {
             GG_CUDA(local_sum<T>(geo, P->cg, src, TK_SORTED, n, nullptr, nullptr, P->d_nrm,
-                                 layer == 0 ? OUT_U : OUT_DBL, loc, 3, ls));
+                                 layer == 0 ? OUT_U : OUT_DBL, loc, 3, P->nsm, ls));
         });
     } else if (P->n_qp == 0) {
         // no triangles: every element integral is empty
@@ -365,7 +367,7 @@ void layer_impl(ggem_plan_t* P, int layer, const double* q, double* out) {
         stage(P, ST_LOCAL, 1, [&] {
             if constexpr (sizeof(T) == 4) {
                 GG_CUDA(elem32_sum(geo, P->cg, P->el, 1.01 * P->near_edge, src, P->d_nrm, layer,
-                                   loc, 3, ls));
+                                   loc, 3, P->nsm, ls));
             } else if (P->ff) {
                 GG_CUDA(elemff_sum(geo, P->cg, P->el, P->d_ff_hi, P->d_ff_lo, P->d_ff_g,
                                    P->d_qv_sorted, 1.01 * P->near_edge, src, P->d_nrm, layer, loc,
