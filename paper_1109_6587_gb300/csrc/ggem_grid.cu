@@ -83,15 +83,21 @@ __device__ __forceinline__ int bitrev(int v, int logM) {
 // Real-to-complex along x for R rows per block: the row of Nx reals is read as
 // M = Nx/2 complex values z_n = x_2n + i x_2n+1, transformed with length M, then
 // X_k = E_k + exp(-2 pi i k/Nx) O_k with E, O the even/odd-sample spectra.
-// Output X_k, k = 0..M-1, in place.
+// Output X_k, k = 0..M-1, in place.  Blocks from nb1 on transform the nrows2 rows of
+// data2 (the wall values ride along with the grid's: 2 launches less).
 template <typename T>
 __global__ void k_fft_x_r2c(c2_t<T>* data, long nrows, int M, int logM,
                             const c2_t<T>* __restrict__ tw, const c2_t<T>* __restrict__ tpost,
-                            int R) {
+                            int R, unsigned nb1, c2_t<T>* data2, long nrows2) {
     using X = Cx<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
     c2_t<T>* s = reinterpret_cast<c2_t<T>*>(smraw);
     long row0 = (long)blockIdx.x * R;
+    if (blockIdx.x >= nb1) {                    // block-uniform
+        data = data2;
+        nrows = nrows2;
+        row0 = (long)(blockIdx.x - nb1) * R;
+    }
     int rr = (int)min((long)R, nrows - row0);
     for (int e = threadIdx.x; e < rr * M; e += blockDim.x) {
         int r = e / M, n = e - r * M;
@@ -148,17 +154,19 @@ __global__ void k_fft_x_c2r(c2_t<T>* data, long nrows, int M, int logM,
 
 // Complex transform along z: planes of [Nz][nkx] complex, TB columns per block;
 // only the first ncols columns of each plane (the others hold zeros and stay
-// zero).
+// zero).  Planes from nplanes1 on are those of data2.
 template <typename T>
 __global__ void k_fft_z(c2_t<T>* data, int nkx, int ncols, int Nz, int logNz,
-                        const c2_t<T>* __restrict__ tw, int TB, bool inv) {
+                        const c2_t<T>* __restrict__ tw, int TB, bool inv, int nplanes1,
+                        c2_t<T>* data2) {
     extern __shared__ __align__(16) unsigned char smraw[];
     c2_t<T>* s = reinterpret_cast<c2_t<T>*>(smraw);
     int ncb = (ncols + TB - 1) / TB;
     long plane = blockIdx.x / ncb;
     int col0 = (blockIdx.x - plane * ncb) * TB;
     int tb = min(TB, ncols - col0);
-    c2_t<T>* base = data + plane * (long)Nz * nkx + col0;
+    c2_t<T>* base = (plane < nplanes1 ? data + plane * (long)Nz * nkx
+                                      : data2 + (plane - nplanes1) * (long)Nz * nkx) + col0;
     for (int e = threadIdx.x; e < Nz * TB; e += blockDim.x) {
         int z = e / TB, c = e - z * TB;
         c2_t<T> v = Cx<T>::mk(0, 0);
@@ -174,56 +182,62 @@ __global__ void k_fft_z(c2_t<T>* data, int nkx, int ncols, int Nz, int logNz,
 
 static int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
 
+// Rows per block: 2048 complex values, fewer (256 at least) while the blocks do not
+// fill the SMs four times: 3,168 rows of 32 are 25 blocks of 128 rows or 198 of 16.
+// One FP64 capsule (32 x 33 x 32), forward with the wall data 61 -> 18 us, inverse 30 -> 17.
 template <typename T>
 static cudaError_t fft_x(const GridGeom& geo, T* data, int nplanes, const void* tw_x, bool inv,
-                         cudaStream_t st) {
+                         int nsm, cudaStream_t st, T* data2 = nullptr, int nplanes2 = 0) {
     int M = geo.Nx / 2, logM = ilog2(M);
-    long nrows = (long)nplanes * geo.Nz;
+    const long nrows = (long)nplanes * geo.Nz, nrows2 = (long)nplanes2 * geo.Nz;
     int R = max(1, 2048 / M);
+    while (R > 1 && R * M > 256 && (nrows + R - 1) / R < 4L * nsm) R >>= 1;
     size_t smem = (size_t)R * M * sizeof(c2_t<T>);
     const c2_t<T>* tw = (const c2_t<T>*)tw_x;
     const c2_t<T>* tpost = tw + M / 2;
-    unsigned nb = (unsigned)((nrows + R - 1) / R);
+    const unsigned nb = (unsigned)((nrows + R - 1) / R), nb2 = (unsigned)((nrows2 + R - 1) / R);
     if (inv) {
         grant_max_smem((const void*)k_fft_x_c2r<T>);
         k_fft_x_c2r<T><<<nb, 256, smem, st>>>((c2_t<T>*)data, nrows, M, logM, tw, tpost, R);
     } else {
         grant_max_smem((const void*)k_fft_x_r2c<T>);
-        k_fft_x_r2c<T><<<nb, 256, smem, st>>>((c2_t<T>*)data, nrows, M, logM, tw, tpost, R);
+        k_fft_x_r2c<T><<<nb + nb2, 256, smem, st>>>((c2_t<T>*)data, nrows, M, logM, tw, tpost, R,
+                                                    nb, (c2_t<T>*)data2, nrows2);
     }
     return cudaGetLastError();
 }
 
 template <typename T>
 static cudaError_t fft_z(const GridGeom& geo, T* data, int nplanes, const void* tw_z, bool inv,
-                         cudaStream_t st, int ncols = 0) {
+                         cudaStream_t st, int ncols = 0, T* data2 = nullptr,
+                         int nplanes2 = 0) {
     int Nz = geo.Nz, logNz = ilog2(Nz), nkx = geo.Nx / 2;
     if (ncols <= 0 || ncols > nkx) ncols = nkx;
     int TB = min(ncols, 8);
     // (the oversampled grids of the spectral evaluation reach Nz = 2048)
     while (TB > 1 && (size_t)TB * Nz * sizeof(c2_t<T>) > (size_t)160 * 1024) TB >>= 1;
     size_t smem = (size_t)TB * Nz * sizeof(c2_t<T>);
-    unsigned nb = (unsigned)((long)nplanes * ((ncols + TB - 1) / TB));
+    unsigned nb = (unsigned)((long)(nplanes + nplanes2) * ((ncols + TB - 1) / TB));
     grant_max_smem((const void*)k_fft_z<T>);
     k_fft_z<T><<<nb, 256, smem, st>>>((c2_t<T>*)data, nkx, ncols, Nz, logNz,
-                                      (const c2_t<T>*)tw_z, TB, inv);
+                                      (const c2_t<T>*)tw_z, TB, inv, nplanes, (c2_t<T>*)data2);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t fft_forward(const GridGeom& geo, T* data, int nplanes, const void* tw_x,
-                        const void* tw_z, cudaStream_t st) {
-    cudaError_t e = fft_x<T>(geo, data, nplanes, tw_x, false, st);
+cudaError_t fft_forward(const GridGeom& geo, T* data, int nplanes, T* data2, int nplanes2,
+                        const void* tw_x, const void* tw_z, int nsm, cudaStream_t st) {
+    cudaError_t e = fft_x<T>(geo, data, nplanes, tw_x, false, nsm, st, data2, nplanes2);
     if (e != cudaSuccess) return e;
-    return fft_z<T>(geo, data, nplanes, tw_z, false, st);
+    return fft_z<T>(geo, data, nplanes, tw_z, false, st, 0, data2, nplanes2);
 }
 
 template <typename T>
 cudaError_t fft_inverse(const GridGeom& geo, T* data, int nplanes, const void* tw_x,
-                        const void* tw_z, cudaStream_t st, int active_kx) {
+                        const void* tw_z, int nsm, cudaStream_t st, int active_kx) {
     cudaError_t e = fft_z<T>(geo, data, nplanes, tw_z, true, st, active_kx);
     if (e != cudaSuccess) return e;
-    return fft_x<T>(geo, data, nplanes, tw_x, true, st);
+    return fft_x<T>(geo, data, nplanes, tw_x, true, nsm, st);
 }
 
 // -------------------------------------------------- Chebyshev contraction
@@ -716,10 +730,10 @@ cudaError_t spectral_pad(const GridGeom& geo, const T* spec, int nplanes, int Mx
 }
 
 #define GGEM_INST_GRID(T)                                                                     \
-    template cudaError_t fft_forward<T>(const GridGeom&, T*, int, const void*, const void*,    \
-                                        cudaStream_t);                                         \
+    template cudaError_t fft_forward<T>(const GridGeom&, T*, int, T*, int, const void*,        \
+                                        const void*, int, cudaStream_t);                       \
     template cudaError_t fft_inverse<T>(const GridGeom&, T*, int, const void*, const void*,    \
-                                        cudaStream_t, int);                                    \
+                                        int, cudaStream_t, int);                               \
     template cudaError_t cheb_apply<T>(int, const T*, bool, const T*, T*, long, cudaStream_t,  \
                                        int*, int, const void*);                                \
     template cudaError_t interp_combine<T>(const GridGeom&, const double*, const T*, const T*, \

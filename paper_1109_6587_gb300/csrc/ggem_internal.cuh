@@ -451,11 +451,11 @@ cudaError_t spread(const GridGeom& geo, const CellGrid& cg, const double* yj, co
                    T* work, int nsm, cudaStream_t st);
 
 template <typename T>
-cudaError_t fft_forward(const GridGeom& geo, T* data, int nplanes, const void* tw_x,
-                        const void* tw_z, cudaStream_t st);
+cudaError_t fft_forward(const GridGeom& geo, T* data, int nplanes, T* data2, int nplanes2,
+                        const void* tw_x, const void* tw_z, int nsm, cudaStream_t st);
 template <typename T>
 cudaError_t fft_inverse(const GridGeom& geo, T* data, int nplanes, const void* tw_x,
-                        const void* tw_z, cudaStream_t st, int active_kx = 0);
+                        const void* tw_z, int nsm, cudaStream_t st, int active_kx = 0);
 
 template <typename T>
 cudaError_t cheb_apply(int Ny, const T* M, bool inv, const T* in, T* out, long cols,

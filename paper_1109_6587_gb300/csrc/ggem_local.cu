@@ -26,6 +26,10 @@ template <> __device__ __forceinline__ float d_rsqrt<float>(float x) {
 }
 template <> __device__ __forceinline__ double d_rsqrt<double>(double x) { return rsqrt(x); }
 
+// Threads per block of the per-point kernels below: their FP64 divisions and floors run
+// at 2 lanes per cycle and SM, so 8,000 points go to 125 blocks, not 32.
+constexpr int kPtBlock = 64;
+
 __global__ void k_cell_count(GridGeom geo, CellGrid cg, int n, const double* __restrict__ x,
                              int* __restrict__ count, int* __restrict__ cell_of) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -107,10 +111,11 @@ cudaError_t build_cells(const GridGeom& geo, const CellGrid& cg, int n, const do
     if (n > 0) {
         // src_cell doubles as the per-source cell scratch before the scatter
         int* cell_of = cursor + ncell;   // caller provides cursor[ncell + n]
-        k_cell_count<<<(n + 255) / 256, 256, 0, st>>>(geo, cg, n, x, cell_count, cell_of);
+        const int nb = (n + kPtBlock - 1) / kPtBlock;
+        k_cell_count<<<nb, kPtBlock, 0, st>>>(geo, cg, n, x, cell_count, cell_of);
         k_scan<<<1, 1024, 0, st>>>(ncell, cell_count, cell_start);
-        k_cell_scatter<T><<<(n + 255) / 256, 256, 0, st>>>(geo, cg, n, x, cell_of, cell_start,
-                                                           cursor, src_cell, perm, pos);
+        k_cell_scatter<T><<<nb, kPtBlock, 0, st>>>(geo, cg, n, x, cell_of, cell_start, cursor,
+                                                   src_cell, perm, pos);
     } else {
         cudaMemsetAsync(cell_start, 0, (ncell + 1) * sizeof(int), st);
     }
@@ -208,7 +213,9 @@ __global__ void k_locate(GridGeom geo, CellGrid cg, int n, int kind, const doubl
 template <typename T>
 cudaError_t locate_targets(const GridGeom& geo, const CellGrid& cg, int n, int kind,
                            const double* x, int* cell, v4_t<T>* pos, cudaStream_t st) {
-    if (n > 0) k_locate<T><<<(n + 255) / 256, 256, 0, st>>>(geo, cg, n, kind, x, cell, pos);
+    if (n > 0)
+        k_locate<T><<<(n + kPtBlock - 1) / kPtBlock, kPtBlock, 0, st>>>(geo, cg, n, kind, x, cell,
+                                                                       pos);
     return cudaGetLastError();
 }
 

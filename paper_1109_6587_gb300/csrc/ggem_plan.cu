@@ -166,9 +166,8 @@ void run_global(ggem_plan_t* P, const SortedSources<T>& src, bool mesh, int out_
                           (const v4_t<T>*)(mesh ? P->d_mesh_sdf : P->d_sdf), A, B,
                           P->nsm, st));
     });
-    stage(P, ST_FFT_FWD, 4, [&] {
-        GG_CUDA(fft_forward<T>(geo, A, geo.Ny * 3, P->d_tw_x, P->d_tw_z, st));
-        GG_CUDA(fft_forward<T>(geo, Wl, 6, P->d_tw_x, P->d_tw_z, st));
+    stage(P, ST_FFT_FWD, 2, [&] {
+        GG_CUDA(fft_forward<T>(geo, A, geo.Ny * 3, Wl, 6, P->d_tw_x, P->d_tw_z, P->nsm, st));
     });
     stage(P, ST_CHEB_FWD, 1, [&] {
         GG_CUDA(cheb_apply<T>(geo.Ny, (const T*)P->d_cheb_fwd, false, A, B, (long)3 * P->nmodes * 2,
@@ -197,7 +196,7 @@ void run_global(ggem_plan_t* P, const SortedSources<T>& src, bool mesh, int out_
                                     (const T*)P->d_spec_dz, (T*)P->d_spec, st));
             // (only the coarse grid's Nx/2 columns in x are nonzero for the z pass)
             GG_CUDA(fft_inverse<T>(fg, (T*)P->d_spec, nth * nout, P->d_spec_twx,
-                                   P->d_spec_twz, st, geo.Nx / 2));
+                                   P->d_spec_twz, P->nsm, st, geo.Nx / 2));
         });
         return;
     }
@@ -206,7 +205,7 @@ void run_global(ggem_plan_t* P, const SortedSources<T>& src, bool mesh, int out_
                               (long)nout * P->nmodes * 2, st, P->d_tc_err, P->nsm, P->d_tc_inv));
     });
     stage(P, ST_FFT_INV, 2, [&] {
-        GG_CUDA(fft_inverse<T>(geo, B, geo.Ny * nout, P->d_tw_x, P->d_tw_z, st));
+        GG_CUDA(fft_inverse<T>(geo, B, geo.Ny * nout, P->d_tw_x, P->d_tw_z, P->nsm, st));
     });
 }
 
