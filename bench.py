@@ -173,14 +173,14 @@ def _peaks():
 
 # Algorithmic flops of one (target, source) pair of the local sum (see roofline)
 FLOPS_PAIR_SINGLE = 52
-FLOPS_PAIR_DOUBLE = 72
+FLOPS_PAIR_DOUBLE = 68
 # DRAM bytes (read + write) of one local-sum launch, the single- and the
 # double-layer launch averaged as the stage is, from ncu captures of the
 # kernels as they stand (dram__bytes_read.sum + dram__bytes_write.sum; the
 # summaries are kept with the profiles), per (workload, precision, quadrature);
 # none for other configurations
 LOCAL_TRAFFIC = {
-    ("rbc4000", "mixed", "element"): (4687680000 + 41640448 + 5192181248 + 67060480) / 2,
+    ("rbc4000", "mixed", "element"): (3852601088 + 62584832 + 4337458176 + 108844800) / 2,
 }
 
 SAMPLE_ABOVE = 100_000      # larger workloads count pairs on a sample of targets
@@ -230,21 +230,43 @@ def _elem_pair_count(susp, rcut):
     from scipy.spatial import cKDTree
     b = susp.box
     qx, qt = _quad_points(susp)
-
-    def wrap(a):
-        a = a.copy()
-        a[:, 0] %= b.Lx
-        a[:, 2] %= b.Lz
-        a[:, 1] -= b.y0
-        return a
     box = [b.Lx, 4 * b.W + 4 * rcut, b.Lz]
     idx, scale = _target_sample(len(susp.x))
-    tq = cKDTree(wrap(qx), boxsize=box)
-    tn = cKDTree(wrap(susp.x[idx]), boxsize=box)
+    tq = cKDTree(_wrapped(qx, b), boxsize=box)
+    tn = cKDTree(_wrapped(susp.x[idx], b), boxsize=box)
     total = int(tn.count_neighbors(tq, rcut))
     # the 16 points of each triangle containing a (sampled) node are the polar rule's
     own = np.bincount(susp.tri.ravel(), minlength=len(susp.x))[idx].sum()
     return int(scale * (total - 16 * own))
+
+
+def _wrapped(a, b):
+    a = a.copy()
+    a[:, 0] %= b.Lx
+    a[:, 2] %= b.Lz
+    a[:, 1] -= b.y0
+    return a
+
+
+def _list_pair_count(susp, alpha, rcut):
+    """The pairs of the FP32 element rule's point lists: 16 points per triangle whose
+    centroid is nearer than 4 longest edges, 7 beyond, 3 from 3 / alpha where alpha
+    times the longest edge is at most 0.33 (each list only if it starts below 0.85
+    r_cut).  The kernel decides by a cell's nearest point, so it evaluates more."""
+    from scipy.spatial import cKDTree
+    b, x, tri = susp.box, susp.x, susp.tri
+    h = max(float(np.linalg.norm(x[tri[:, i]] - x[tri[:, (i + 1) % 3]], axis=1).max())
+            for i in range(3))
+    r7 = 4.0 * h
+    r3 = max(r7, 3.0 / alpha) if alpha * h <= 0.33 else rcut
+    r7, r3 = (r if r < 0.85 * rcut else rcut for r in (r7, r3))
+    box = [b.Lx, 4 * b.W + 4 * rcut, b.Lz]
+    idx, scale = _target_sample(len(x))
+    tc = cKDTree(_wrapped(x[tri].mean(1), b), boxsize=box)
+    tn = cKDTree(_wrapped(x[idx], b), boxsize=box)
+    n7, n3, n = (int(v) for v in tn.count_neighbors(tc, [r7, r3, rcut]))
+    own = int(np.bincount(tri.ravel(), minlength=len(x))[idx].sum())
+    return int(scale * (16 * (n7 - own) + 7 * (n3 - n7) + 3 * (n - n3)))
 
 
 def aggregate(t_ms, steps, n_points, world, device):
@@ -345,7 +367,9 @@ def roofline(res, args):
     esz = 4 if args.precision == "mixed" else 8
     plane = b.Nz * b.Nx
     if name == "local_sum":
-        pairs = _elem_pair_count(susp, rc) if args.quadrature == "element" else _pair_count(susp, rc)
+        pairs = (_list_pair_count(susp, a, rc) if args.precision == "mixed" else
+                 _elem_pair_count(susp, rc)) if args.quadrature == "element" else \
+            _pair_count(susp, rc)
         # algorithmic flops per (target, source) pair within r_cut, counting
         # add, sub, mul and rsqrt / exp2 as 1 and a fused multiply-add as 2
         # (the peak below counts an FMA as 2): displacement, r^2, 1/r, r,
@@ -355,8 +379,9 @@ def roofline(res, args):
         # single layer's A = erfc/r - c1 e, B = (erfc/r^3 + c1 e/r^2) x.g and
         # u += A g + B x (19: 52 in all) or the double layer's D, E, x.n, g.n
         # and v += x (D x.g x.n + E g.n) + g E x.n + n E x.g with the last
-        # term summed as a scalar (39: 72 in all); the stage averages one
-        # launch of each
+        # term summed as a scalar and E's constant taken out (68 in all); the
+        # stage averages one launch of each.  Mixed element plans take fewer
+        # points of far triangles: the pairs are those of their lists
         flops = pairs * (FLOPS_PAIR_SINGLE + FLOPS_PAIR_DOUBLE) / 2.0
         peak = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
         ach = flops / avg_s / 1e12
