@@ -22,6 +22,8 @@
 // the sums differ by 6e-10 to 2.3e-8 (2.8: up to 5.2e-8; alpha h = 0.5: 2.2e-7,
 // where the list is not used).  In candidates per target the lists halve the work of
 // dense suspensions and take a third off dilute ones.
+// Triangles large against r_cut keep list 0 only, each point in the cell that holds it
+// (kBinRadius).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -37,12 +39,33 @@ namespace {
 constexpr int kPts[kElemLists] = {16, 7, 3};
 constexpr double kFarEdges = 4.0, kDimRadius = 3.0, kDimEdge = 0.33;
 
+// A point can lie two thirds of a triangle's longest edge h nearer to a target than
+// the centroid it is binned by, so a cell dropped for lying beyond r_cut holds
+// points within it, down to r_cut - 2 h / 3, whose terms carry up to
+// exp(-alpha^2 (r_cut - 2 h / 3)^2); and whole steps are summed unmasked, with points
+// beyond r_cut, whose terms carry up to exp(-alpha^2 r_cut^2).  Where
+// alpha (r_cut - 2 h / 3) < kBinRadius or alpha r_cut < kBinCut every point is
+// therefore binned by itself, its terms masked at r_cut, and list 0 is the only one.
+// On these lines (FP64, spheres r_cut apart and less) the terms left out and added are
+// up to 8e-7 of the largest double-layer sum, nearly all of it added ones (1.2e-6 at
+// r_cut = 3.95 / alpha, 3e-6 at 3.75); by centroid, h = 1.2 r_cut was off by
+// 3.7e-4 of the whole double layer and r_cut = 2 / alpha by 2.0e-3.  With r_cut =
+// 4 / alpha the line is at h = 0.225 r_cut, beyond the last edge with a list 1
+// (0.2125).  The price, double layer of 100 spheres: .55 -> .58 ms at h = 0.62 r_cut,
+// .73 -> .75 at 0.33; 2.87 -> 4.23 at r_cut = 3.9 / alpha, h = 0.07, which loses lists
+// 1 and 2.
+constexpr double kBinRadius = 3.4, kBinCut = 3.999;
+
 // search reach in cells and its neighbour offsets
 constexpr int R32 = kElemReach, kSide = 2 * R32 + 1, kOffsets = kSide * kSide * kSide;
 
 // phi_v w of point a of a rule on the unit triangle of area 1/2 (FP64)
 struct RuleTab {
     double phi[16][3], w[16];
+};
+
+struct ListTab {
+    double phi[16][3];
 };
 
 RuleTab rule_tab(int list, const QuadRule& g) {
@@ -144,6 +167,19 @@ __global__ void k_tri_sorted(GridGeom geo, CellGrid cg, int m, const int* __rest
     for (int i = 0; i < 3; ++i) shift[3 * (size_t)s + i] = o[i] - c[i];
 }
 
+// The 16 points of every triangle, for binning them one by one.
+__global__ void k_points(int m, const double* __restrict__ x, const int* __restrict__ tri,
+                         ListTab tab, double* __restrict__ xq) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= 16 * m) return;
+    const int k = e >> 4, a = e & 15;
+    const double* xa = x + 3 * (size_t)tri[3 * (size_t)k];
+    const double* xb = x + 3 * (size_t)tri[3 * (size_t)k + 1];
+    const double* xc = x + 3 * (size_t)tri[3 * (size_t)k + 2];
+    for (int i = 0; i < 3; ++i)
+        xq[3 * (size_t)e + i] = tab.phi[a][0] * xa[i] + tab.phi[a][1] * xb[i] + tab.phi[a][2] * xc[i];
+}
+
 // 64-point steps of list `pts` points per triangle in each cell
 __global__ void k_step_counts(int ncell, int pts, const int* __restrict__ start,
                               int* __restrict__ cnt) {
@@ -229,10 +265,6 @@ __global__ void k_neighbours(CellGrid cg, float hx, float hy, float hz, float re
     if (!FILL && lane == 0) cnt[c0] = n;
 }
 
-struct ListTab {
-    double phi[16][3];
-};
-
 // positions of one list, a warp per step, a lane per slot pair: offsets from
 // the cell corner in units of 1/(alpha sqrt(log2 e)); slots past the cell's
 // last point get the dummy offset 1e4 (terms exactly zero) and zero strength
@@ -268,6 +300,46 @@ __global__ void k_list_positions(int nsteps, const int4* __restrict__ map,
         // vertices of every 16-slot group (list 0: one triangle each)
         if (PTS == 16 && k == 0 && (lane & 7) == 0)
             vert[(size_t)step * 4 + (lane >> 3)] = in ? tv[s] : make_int4(-1, -1, -1, 0);
+    }
+    float4* o = pack + (size_t)step * 96 + lane;
+    o[0] = make_float4(p[0][0], p[1][0], p[0][1], p[1][1]);
+    o[32] = make_float4(p[0][2], p[1][2], 0.f, 0.f);
+    o[64] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// The same for points binned one by one: a slot's point from the cell order perm
+// (point = 16 triangle + rule index), with its triangle's vertices and twice the
+// area (float bits) and its rule index.
+__global__ void k_point_positions(GridGeom geo, CellGrid cg, int nsteps,
+                                  const int4* __restrict__ map, const int* __restrict__ perm,
+                                  const double* __restrict__ xq, const int* __restrict__ tri,
+                                  const double* __restrict__ tri_area, double sc,
+                                  float4* __restrict__ pack, int4* __restrict__ vert,
+                                  unsigned char* __restrict__ rule) {
+    const int step = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (step >= nsteps) return;                  // warp-uniform
+    const int4 mp = map[step];
+    float p[2][3];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int s = mp.x + mp.z + 2 * lane + k;
+        const size_t slot = (size_t)step * 64 + 2 * lane + k;
+        p[k][0] = p[k][1] = p[k][2] = 1e4f;
+        int4 v = make_int4(-1, -1, -1, 0);
+        int a = 0;
+        if (s < mp.y) {
+            const int id = perm[s], t = id >> 4;
+            const double* c = xq + 3 * (size_t)id;
+            int cx, cy, cz;
+            double o[3];
+            locate(geo, cg, c[0], c[1], c[2], cx, cy, cz, o[0], o[1], o[2]);
+            for (int i = 0; i < 3; ++i) p[k][i] = (float)(o[i] * sc);
+            v = make_int4(tri[3 * (size_t)t], tri[3 * (size_t)t + 1], tri[3 * (size_t)t + 2],
+                          __float_as_int((float)(2.0 * tri_area[t])));
+            a = id & 15;
+        }
+        vert[slot] = v;
+        rule[slot] = (unsigned char)a;
     }
     float4* o = pack + (size_t)step * 96 + lane;
     o[0] = make_float4(p[0][0], p[1][0], p[0][1], p[1][1]);
@@ -331,6 +403,37 @@ __global__ void k_list_strengths(int n0, int n1, int n2, const int4* __restrict_
     else step_strengths<kPts[2]>(lane, map2[step - n0 - n1], tv, q, scale, c[2], o);
 }
 
+// strengths of points binned one by one
+__global__ void k_point_strengths(int nsteps, const int4* __restrict__ vert,
+                                  const unsigned char* __restrict__ rule,
+                                  const float* __restrict__ q, float scale, StrengthTab tab,
+                                  float4* __restrict__ pack) {
+    __shared__ float c[16][3];
+    for (int e = threadIdx.x; e < 48; e += blockDim.x) (&c[0][0])[e] = (&tab.c[0][0][0])[e];
+    __syncthreads();
+    const int step = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (step >= nsteps) return;                  // warp-uniform
+    float g[2][3];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const size_t slot = (size_t)step * 64 + 2 * lane + k;
+        const int4 v = vert[slot];
+        const int a = rule[slot];
+        g[k][0] = g[k][1] = g[k][2] = 0.f;
+        if (v.x >= 0) {
+            const float f = scale * __int_as_float(v.w);
+            const float ca = f * c[a][0], cb = f * c[a][1], cc = f * c[a][2];
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                g[k][i] = ca * q[3 * (size_t)v.x + i] + cb * q[3 * (size_t)v.y + i] +
+                          cc * q[3 * (size_t)v.z + i];
+        }
+    }
+    float4* o = pack + (size_t)step * 96 + lane;
+    *reinterpret_cast<float2*>(&o[32].z) = make_float2(g[0][0], g[1][0]);
+    o[64] = make_float4(g[0][1], g[1][1], g[0][2], g[1][2]);
+}
+
 // --------------------------------------------------------------- the sum
 // Two candidate pairs at once (add/mul/fma .f32x2: one issued instruction
 // serves two pairs); rsqrt, exp2 and the reciprocal stay scalar.  Every
@@ -345,8 +448,9 @@ __device__ __forceinline__ float rcp_ftz(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// the hardware approximations (about 2 ulp); r^2 lies in (0, (1.7 r_cut)^2) but
-// for the dummies, far from denormal inputs and results
+// the hardware approximations (about 2 ulp); r is at most r_cut, a cell's diagonal
+// (up to 0.9 r_cut where one cell spans the slit) and two thirds of an edge, but for
+// the dummies: far from denormal inputs and results
 __device__ __forceinline__ float rsqrt_ftz(float x) {
     float r;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -419,7 +523,7 @@ struct Elem32Args {
     const int4* nbr;
     const unsigned short* noff;
     float lim1, lim2;                // squared distances from which a cell uses lists 1, 2
-    const int4* vert;                // list 0: vertices of each 16-slot group
+    const int4* vert;                // list 0: vertices of each 16-slot group (POINTS: slot)
     const double* nrm;               // [n][3] target normals (caller order)
     float* out;
     int out_stride;
@@ -435,6 +539,7 @@ constexpr int kCap = 128;     // culled cells per batch (a target may need sever
 // target (slightly widened, so that rounding can only keep more).  Entries:
 // first step, step count and offset index; bit 15 marks the cells that can
 // hold triangles around the target.
+template <bool POINTS>
 __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, float ox, float oy,
                                                 float oz, int& i, int end, int* s_st, int* s_cnt,
                                                 unsigned short* s_off) {
@@ -462,7 +567,7 @@ __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, f
             const int l = d2 >= a.lim2 ? 2 : (d2 >= a.lim1 ? 1 : 0);
             st = l == 2 ? e.z : (l == 1 ? e.y : e.x);
             constexpr int p0 = kPts[0], p1 = kPts[1], p2 = kPts[2];
-            cnt = (e.w * (l == 2 ? p2 : (l == 1 ? p1 : p0)) + 63) >> 6;
+            cnt = (e.w * (POINTS ? 1 : (l == 2 ? p2 : (l == 1 ? p1 : p0))) + 63) >> 6;
         }
         const unsigned m = __ballot_sync(0xffffffffu, keep);
         if (keep) {
@@ -487,12 +592,10 @@ __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, f
 // every coordinate already paired, each load of a warp covering 512 contiguous
 // bytes.  Each cell fills whole steps with dummies, so a step needs no bounds
 // test.
-// Candidates beyond r_cut are evaluated unmasked: their terms carry
-// exp(-alpha^2 r^2) <= e^-16 (and erfc(alpha r) <= 1.6e-8), below the FP32
-// rounding of the sum, and a step with no candidate within r_cut is skipped; in
-// the same way a triangle counts with the cell of its centroid (the sums with
-// points within r_cut left out or beyond it counted differ from the strictly
-// truncated ones by the same 3e-8 to 4e-7 as when every point had its own cell).
+// Candidates beyond r_cut are evaluated unmasked, and a step with no candidate within
+// r_cut is skipped; in the same way a triangle counts with the cell of its
+// centroid.  POINTS: the points were binned one by one, and each counts within r_cut only
+// (kBinRadius says when).
 // Points of the triangles around the target (left to the singular correction)
 // can only lie in the cells the culling marks near; only there is each
 // candidate within near2 checked and, if excluded, given zero strength.
@@ -508,8 +611,8 @@ __device__ __forceinline__ int cull_cells_batch(const Elem32Args& a, int lane, f
 // 12.4 ms without list 2, 11.3 ms with it.  Cells of
 // r_cut / 4 or / 5 have fewer candidates and more cells: 145.7 and 148.1 against
 // 145.5 ms per two launches (list 1 from 5 edges).
-template <int LAYER, int S>
-__global__ void __launch_bounds__(LWE * 32, 12) k_local_elem32(Elem32Args a,
+template <int LAYER, int S, bool POINTS>
+__global__ void __launch_bounds__(LWE * 32, POINTS ? 10 : 12) k_local_elem32(Elem32Args a,
                                                           const float4* __restrict__ pk) {
     __shared__ int s_st[LWE][kCap];
     __shared__ int s_cnt[LWE][kCap];
@@ -532,8 +635,8 @@ __global__ void __launch_bounds__(LWE * 32, 12) k_local_elem32(Elem32Args a,
     const float rc2 = a.k.rc2;
     PairAcc2 acc;
     for (int i = a.nstart[c]; i < nend;) {
-        const int nc = cull_cells_batch(a, lane, ox, oy, oz, i, nend, s_st[wid], s_cnt[wid],
-                                        s_off[wid]);
+        const int nc = cull_cells_batch<POINTS>(a, lane, ox, oy, oz, i, nend, s_st[wid],
+                                                s_cnt[wid], s_off[wid]);
         for (int ci = S > 1 ? wid : 0; ci < nc; ci += S) {
             const int st = s_st[wid][ci], end = st + s_cnt[wid][ci];
             const int oi = s_off[wid][ci] & 0x7fff;
@@ -557,7 +660,16 @@ __global__ void __launch_bounds__(LWE * 32, 12) k_local_elem32(Elem32Args a,
                        wz = make_float2(pc.z, pc.w);
                 f2_split(r2, r0, r1);
                 if (!__any_sync(0xffffffffu, r0 < rc2 || r1 < rc2)) return;
-                if (NEAR) {
+                if (POINTS) {
+                    if (NEAR) {
+                        const int4* v = a.vert + (size_t)s * 64 + 2 * lane;
+                        const int4 v0 = v[0], v1 = v[1];
+                        if (v0.x == oidx || v0.y == oidx || v0.z == oidx) r0 = rc2;
+                        if (v1.x == oidx || v1.y == oidx || v1.z == oidx) r1 = rc2;
+                    }
+                    if (!(r0 < rc2)) wx.x = wy.x = wz.x = 0.f;
+                    if (!(r1 < rc2)) wx.y = wy.y = wz.y = 0.f;
+                } else if (NEAR) {
                     if (r0 < a.k.near2 || r1 < a.k.near2) {
                         // both candidates are points of one triangle (list 0)
                         const int4 v = a.vert[(size_t)s * 4 + (lane >> 3)];
@@ -617,6 +729,10 @@ float coord_scale(double alpha) { return (float)(alpha * 1.2011224087864498); }
 
 }  // namespace
 
+bool elem32_by_point(double near_edge, double alpha, double rcut) {
+    return alpha * (rcut - near_edge * (2.0 / 3.0)) < kBinRadius || alpha * rcut < kBinCut;
+}
+
 // A point of a triangle around the target can be farther from it than the
 // triangle's longest edge only by rounding; `near` carries that margin.  A far
 // cell never is a near one (kFarEdges > 1).
@@ -630,7 +746,8 @@ void elem32_far_distances(double near_edge, double alpha, double rcut, double* f
 
 cudaError_t elem32_steps(const ElemLists32& L, int ncell, int* scratch, cudaStream_t st) {
     for (int l = 0; l < kElemLists; ++l) {
-        k_step_counts<<<(ncell + 255) / 256, 256, 0, st>>>(ncell, kPts[l], L.tri_start, scratch);
+        const int pts = L.points ? (l == 0 ? 1 : 0) : kPts[l];
+        k_step_counts<<<(ncell + 255) / 256, 256, 0, st>>>(ncell, pts, L.tri_start, scratch);
         cudaError_t e = scan_counts(ncell, scratch, L.sstart[l], st);
         if (e != cudaSuccess) return e;
     }
@@ -664,6 +781,36 @@ cudaError_t elem32_neighbours(const GridGeom& geo, const CellGrid& cg, const Ele
 cudaError_t elem32_centroids(int m, const double* x, const int* tri, double* cen,
                              cudaStream_t st) {
     if (m > 0) k_centroids<<<(m + 255) / 256, 256, 0, st>>>(m, x, tri, cen);
+    return cudaGetLastError();
+}
+
+cudaError_t elem32_points(int m, const double* x, const int* tri, const QuadRule& rule, double* xq,
+                          cudaStream_t st) {
+    const RuleTab r = rule_tab(0, rule);
+    ListTab tab;
+    for (int a = 0; a < 16; ++a)
+        for (int v = 0; v < 3; ++v) tab.phi[a][v] = r.phi[a][v];
+    if (m > 0) k_points<<<(m * 16 + 255) / 256, 256, 0, st>>>(m, x, tri, tab, xq);
+    return cudaGetLastError();
+}
+
+cudaError_t elem32_point_order(const CellGrid& cg, const ElemLists32& L, const float4* pos,
+                               const int* perm, int* perm_out, cudaStream_t st) {
+    k_cell_subsort<<<cg.ncx * cg.ncy * cg.ncz, 64, 0, st>>>(
+        L.tri_start, pos, perm, (float)(4.0 / cg.hx), (float)(4.0 / cg.hy), (float)(4.0 / cg.hz),
+        perm_out);
+    return cudaGetLastError();
+}
+
+cudaError_t elem32_point_fill(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
+                              const int* perm, const double* xq, const int* tri,
+                              const double* tri_area, cudaStream_t st) {
+    const int ncell = cg.ncx * cg.ncy * cg.ncz, ns = L.nsteps[0];
+    if (ns == 0) return cudaSuccess;
+    k_step_map<<<(ncell + 255) / 256, 256, 0, st>>>(ncell, L.tri_start, L.sstart[0], L.map[0]);
+    k_point_positions<<<(ns + 7) / 8, 256, 0, st>>>(geo, cg, ns, L.map[0], perm, xq, tri, tri_area,
+                                                    (double)coord_scale(geo.alpha), L.pack, L.vert,
+                                                    L.prule);
     return cudaGetLastError();
 }
 
@@ -718,7 +865,10 @@ cudaError_t elem32_strengths(const ElemLists32& L, const QuadRule& rule, int nno
             for (int v = 0; v < 3; ++v) tab.c[l][a][v] = (float)(r.phi[a][v] * r.w[a]);
     }
     const int ns = L.nsteps[0] + L.nsteps[1] + L.nsteps[2];
-    if (ns > 0)
+    if (ns > 0 && L.points)
+        k_point_strengths<<<(ns + 7) / 8, 256, 0, st>>>(ns, L.vert, L.prule, q32, (float)scale, tab,
+                                                        L.pack);
+    else if (ns > 0)
         k_list_strengths<<<(ns + 7) / 8, 256, 0, st>>>(L.nsteps[0], L.nsteps[1], L.nsteps[2],
                                                        L.map[0], L.map[1], L.map[2], L.tv, q32,
                                                        (float)scale, tab, L.pack);
@@ -771,9 +921,12 @@ cudaError_t elem32_sum(const GridGeom& geo, const CellGrid& cg, const ElemLists3
     // -> 246, 24,300 466 -> 436 / 397 -> 410, 64,200 on finer spheres 2.63 -> 2.66 / 2.18
     // -> 2.57 ms: every warp culls the whole neighbour list, which a full chip feels.
     const bool split = tgt.n <= 96 * nsm;
-    void (*kf)(Elem32Args, const float4*) =
-        split ? (layer == 0 ? k_local_elem32<0, LWE> : k_local_elem32<1, LWE>)
-              : (layer == 0 ? k_local_elem32<0, 1> : k_local_elem32<1, 1>);
+    void (*const kfs[2][2][2])(Elem32Args, const float4*) = {
+        {{k_local_elem32<0, 1, false>, k_local_elem32<0, 1, true>},
+         {k_local_elem32<0, LWE, false>, k_local_elem32<0, LWE, true>}},
+        {{k_local_elem32<1, 1, false>, k_local_elem32<1, 1, true>},
+         {k_local_elem32<1, LWE, false>, k_local_elem32<1, LWE, true>}}};
+    const auto kf = kfs[layer == 0 ? 0 : 1][split][L.points];
     cudaFuncSetAttribute((const void*)kf, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
     kf<<<split ? tgt.n : (tgt.n + LWE - 1) / LWE, LWE * 32, 0, st>>>(a, L.pack);
     return cudaGetLastError();

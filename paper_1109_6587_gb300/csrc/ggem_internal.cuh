@@ -91,10 +91,12 @@ __device__ __forceinline__ void locate(const GridGeom& geo, const CellGrid& cg, 
 }
 
 // FP32 element rule: point lists per quadrature rule of the triangles, binned
-// by centroid (ggem_elem32.cu).  Cells at least r_cut / kElemReach wide.
+// by centroid, or (points) the 16-point list alone, every point binned by itself
+// (ggem_elem32.cu).  Cells at least r_cut / kElemReach wide.
 constexpr int kElemLists = 3, kElemReach = 3;
 struct ElemLists32 {
-    int* tri_start = nullptr;             // [ncell + 1] sorted triangles of each cell
+    bool points = false;                  // every point binned by itself
+    int* tri_start = nullptr;             // [ncell + 1] sorted triangles (points) of each cell
     int4* tv = nullptr;                   // [m] sorted triangles: vertices, 2A (float bits)
     double* shift = nullptr;              // [m][3] point position -> offset from the cell corner
     int* sstart[kElemLists] = {};         // [ncell + 1] first 64-point step of each cell
@@ -102,6 +104,8 @@ struct ElemLists32 {
     int nsteps[kElemLists] = {};
     float4* pack = nullptr;               // [steps][3][32]: the lists one after the other
     int4* vert = nullptr;                 // [4 steps of list 0] vertices of each 16-slot group
+                                          //   (points: [64 steps], of each slot, 2A)
+    unsigned char* prule = nullptr;       // points: [64 steps] rule index of each slot
     int* nstart = nullptr;                // [ncell + 1] neighbour list of each target cell
     int4* nbr = nullptr;                  // its entries: first step per list, triangles
     unsigned short* noff = nullptr;       //   and offset index
@@ -271,8 +275,15 @@ struct ggem_plan {
     // FP32 element rule: point lists of the triangles
     ggem::ElemLists32 el;
     size_t nbr_cap = 0;                // entries that el.nbr holds
-    size_t step_cap = 0;               // steps that el.pack holds,
-    size_t step_cap_l[ggem::kElemLists] = {};  // and el.map (el.vert: list 0)
+    size_t pack_cap = 0;               // entries that el.pack holds,
+    size_t step_cap_l[ggem::kElemLists] = {};  // el.map,
+    size_t vert_cap = 0, prule_cap = 0;        // el.vert and el.prule,
+    size_t point_cap[5] = {};          // and of the five arrays below
+    double* d_ep_x = nullptr;          // points binned singly: positions, cell / perm (unordered,
+    int* d_ep_cell = nullptr;          //   ordered) / offsets
+    int* d_ep_perm = nullptr;
+    int* d_ep_perm2 = nullptr;
+    float4* d_ep_pos = nullptr;
     double* d_et_cen = nullptr;        // triangles: centroids, cell / perm (unordered, ordered) / offsets
     int* d_et_cell = nullptr;
     int* d_et_perm = nullptr;
@@ -388,6 +399,17 @@ cudaError_t elem32_order(const GridGeom& geo, const CellGrid& cg, int m, const E
                          const float4* pos, const int* perm, int* perm_out, const double* cen,
                          const int* tri, const double* tri_area, cudaStream_t st);
 cudaError_t elem32_steps(const ElemLists32& L, int ncell, int* scratch, cudaStream_t st);
+// Points binned one by one (L.points, tri_start then counts points): positions xq of
+// all 16 m points (binned by build_cells), their order within the cells, and with
+// the list allocated its slots.
+bool elem32_by_point(double near_edge, double alpha, double rcut);
+cudaError_t elem32_points(int m, const double* x, const int* tri, const QuadRule& rule, double* xq,
+                          cudaStream_t st);
+cudaError_t elem32_point_order(const CellGrid& cg, const ElemLists32& L, const float4* pos,
+                               const int* perm, int* perm_out, cudaStream_t st);
+cudaError_t elem32_point_fill(const GridGeom& geo, const CellGrid& cg, const ElemLists32& L,
+                              const int* perm, const double* xq, const int* tri,
+                              const double* tri_area, cudaStream_t st);
 // neighbour lists of the cells with targets (tgt_start), of L's steps or, with
 // src_start, of the points sorted there (entries: first point, 0, 0, points):
 // counts (scratch: ncell ints; fills nstart), or with `fill` the entries

@@ -822,7 +822,8 @@ void plan_free(ggem_plan_t* P) {
                     P->d_et_perm, P->d_et_perm2, P->d_et_pos, P->el.tri_start, P->el.tv,
                     P->el.shift, P->el.sstart[0], P->el.sstart[1], P->el.sstart[2], P->el.map[0],
                     P->el.map[1], P->el.map[2], P->el.pack, P->el.vert, P->el.nstart,
-                    P->el.nbr, P->el.noff};
+                    P->el.nbr, P->el.noff, P->el.prule, P->d_ep_x, P->d_ep_cell, P->d_ep_perm,
+                    P->d_ep_perm2, P->d_ep_pos};
     for (void* p : ptrs) dfree(p);
     precond_free(P);
     dfree(P->d_pc_Zb);
@@ -853,19 +854,46 @@ void neighbour_lists(ggem_plan_t* P, const int* src_start) {
     GG_CUDA(elem32_neighbours(P->geo, P->cg, L, P->d_mesh_start, src_start, nullptr, true, st));
 }
 
-// FP32 element rule: the triangles (by centroid) into the cells, then the
-// neighbour lists of the mesh nodes' cells and the point lists, grown where the
-// mesh needs more steps than they hold.  A list is built where cells beyond its distance are common: at 0.85
-// r_cut and more the few percent of points it would save cost as much again in
-// strengths.
+// `want` entries of *p, freed and allocated anew with an eighth to spare where it
+// holds fewer (the capacity counts nothing in between, should that fail).
+template <typename X>
+void grow(ggem_plan_t* P, X** p, size_t* cap, size_t want) {
+    if (want <= *cap) return;
+    dfree(*p);
+    *p = nullptr;
+    *cap = 0;
+    dalloc(P, p, want + want / 8);
+    *cap = want + want / 8;
+}
+
+// FP32 element rule: the triangles by centroid (or, where they are large against
+// r_cut, their points one by one) into the cells, then the neighbour lists of
+// the mesh nodes' cells and the point lists, grown where the mesh needs more
+// steps than they hold.  A list is built where cells beyond its distance are common:
+// at 0.85 r_cut and more the few percent of points it would save cost as much
+// again in strengths.
 void elem32_mesh(ggem_plan_t* P, int m) {
     cudaStream_t st = P->st;
     ElemLists32& L = P->el;
-    GG_CUDA(elem32_centroids(m, P->d_x, P->d_tri, P->d_et_cen, st));
-    GG_CUDA(build_cells<float>(P->geo, P->cg, m, P->d_et_cen, P->d_cell_count, L.tri_start,
-                               P->d_cursor, P->d_et_cell, P->d_et_perm, P->d_et_pos, st));
-    GG_CUDA(elem32_order(P->geo, P->cg, m, L, P->d_et_pos, P->d_et_perm, P->d_et_perm2,
-                         P->d_et_cen, P->d_tri, P->d_tri_area, st));
+    L.points = elem32_by_point(P->near_edge, P->geo.alpha, P->geo.rcut);
+    if (L.points) {
+        const size_t np = 16 * (size_t)m;
+        grow(P, &P->d_ep_x, &P->point_cap[0], 3 * np);
+        grow(P, &P->d_ep_cell, &P->point_cap[1], np);
+        grow(P, &P->d_ep_perm, &P->point_cap[2], np);
+        grow(P, &P->d_ep_perm2, &P->point_cap[3], np);
+        grow(P, &P->d_ep_pos, &P->point_cap[4], np);
+        GG_CUDA(elem32_points(m, P->d_x, P->d_tri, P->rule, P->d_ep_x, st));
+        GG_CUDA(build_cells<float>(P->geo, P->cg, (int)np, P->d_ep_x, P->d_cell_count, L.tri_start,
+                                   P->d_cursor, P->d_ep_cell, P->d_ep_perm, P->d_ep_pos, st));
+        GG_CUDA(elem32_point_order(P->cg, L, P->d_ep_pos, P->d_ep_perm, P->d_ep_perm2, st));
+    } else {
+        GG_CUDA(elem32_centroids(m, P->d_x, P->d_tri, P->d_et_cen, st));
+        GG_CUDA(build_cells<float>(P->geo, P->cg, m, P->d_et_cen, P->d_cell_count, L.tri_start,
+                                   P->d_cursor, P->d_et_cell, P->d_et_perm, P->d_et_pos, st));
+        GG_CUDA(elem32_order(P->geo, P->cg, m, L, P->d_et_pos, P->d_et_perm, P->d_et_perm2,
+                             P->d_et_cen, P->d_tri, P->d_tri_area, st));
+    }
     GG_CUDA(elem32_steps(L, P->ncell, P->d_cell_count, st));
     for (int l = 0; l < kElemLists; ++l)
         GG_CUDA(cudaMemcpyAsync(&L.nsteps[l], L.sstart[l] + P->ncell, sizeof(int),
@@ -876,30 +904,18 @@ void elem32_mesh(ggem_plan_t* P, int m) {
         if (!std::isfinite(L.far[l])) L.nsteps[l] = 0;
     size_t total = 0;
     for (int l = 0; l < kElemLists; ++l) {
-        const size_t ns = L.nsteps[l];
-        total += ns;
-        if (ns > P->step_cap_l[l]) {
-            dfree(L.map[l]);
-            L.map[l] = nullptr;
-            if (l == 0) {
-                dfree(L.vert);
-                L.vert = nullptr;
-            }
-            P->step_cap_l[l] = 0;
-            dalloc(P, &L.map[l], ns + ns / 8);
-            if (l == 0) dalloc(P, &L.vert, 4 * (ns + ns / 8));
-            P->step_cap_l[l] = ns + ns / 8;
-        }
+        total += L.nsteps[l];
+        grow(P, &L.map[l], &P->step_cap_l[l], L.nsteps[l]);
     }
-    if (total > P->step_cap) {
-        dfree(L.pack);
-        L.pack = nullptr;
-        P->step_cap = 0;
-        dalloc(P, &L.pack, 96 * (total + total / 8));
-        P->step_cap = total + total / 8;
-    }
+    grow(P, &L.vert, &P->vert_cap, (L.points ? 64 : 4) * (size_t)L.nsteps[0]);
+    if (L.points) grow(P, &L.prule, &P->prule_cap, 64 * (size_t)L.nsteps[0]);
+    grow(P, &L.pack, &P->pack_cap, 96 * total);
     neighbour_lists(P, nullptr);
-    GG_CUDA(elem32_fill(P->geo, P->cg, L, P->rule, P->d_x, st));
+    if (L.points)
+        GG_CUDA(elem32_point_fill(P->geo, P->cg, L, P->d_ep_perm2, P->d_ep_x, P->d_tri,
+                                  P->d_tri_area, st));
+    else
+        GG_CUDA(elem32_fill(P->geo, P->cg, L, P->rule, P->d_x, st));
 }
 
 }  // namespace
