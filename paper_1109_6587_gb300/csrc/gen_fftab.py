@@ -17,7 +17,13 @@ degrees 0..6 as float pairs, 7..9 as floats (their terms are below 2e-8).
 Run: python gen_fftab.py > ggem_fftab.cuh
 
 The FP64 sums take the same functions in doubles, of degree 10 (truncation below
-2e-17 of each function's largest value).
+2e-17 of each function's largest value), near the target.  Farther out 1/rho - A_g
+and the like are differences of nearly equal numbers (the local kernels fall as
+exp(-s/2)), so from s = 3.5 on they take the local kernels themselves, scaled,
+  1 - rho A_g, 1 - rho^3 B_g, 1 - rho^5 D_g = erfc(x) - w, erfc(x) + w,
+  erfc(x) + w (1 + 2 x^2 / 3),  x = rho / sqrt 2,  w = 2 x exp(-x^2) / sqrt(pi),
+in the same degree and intervals (relative truncation below 1e-15 where they are
+used: A and B from interval 6, D from interval 4).
 Run: python gen_fftab.py fp64 > ggem_smooth64.cuh
 """
 import sys
@@ -26,7 +32,7 @@ import mpmath as mp
 import numpy as np
 
 mp.mp.dps = 50
-NINT, DEG, PAIRS, DEG64 = 73, 9, 7, 10
+NINT, DEG, PAIRS, DEG64, FAR0 = 73, 9, 7, 10, 4
 
 
 def smooth(m, s):
@@ -36,6 +42,7 @@ def smooth(m, s):
 C = mp.sqrt(2 / mp.pi)
 FUNCS = [lambda s: C * (smooth(0, s) + mp.exp(-s / 2)), lambda s: C * smooth(2, s),
          lambda s: C * smooth(4, s) / 3, lambda s: C * mp.exp(-s / 2) / 6]
+FAR = [lambda s, k=k: 1 - mp.sqrt(s) ** (2 * k + 1) * FUNCS[k](s) for k in range(3)]
 
 
 def interpolant(f, i, deg=DEG):
@@ -94,22 +101,33 @@ def main():
     print("};")
 
 
-def main64():
-    print("// Generated by gen_fftab.py fp64 (mpmath, 50 digits): A_g, B_g, D_g, E_g on |s - i| <= 1/2,")
-    print("// degree %d in u = s - i.  kSmooth64[function][degree][interval]." % DEG64)
-    print("#pragma once")
-    print("#define GGEM_SMOOTH64_NINT %d" % NINT)
-    print("#define GGEM_SMOOTH64_DEG %d" % DEG64)
-    print("__device__ const double kSmooth64[4][%d][%d] = {" % (DEG64 + 1, NINT))
-    for f in FUNCS:
-        tab = [interpolant(f, i, DEG64) for i in range(NINT)]
+def table64(name, rows):
+    """rows[function][degree][interval]"""
+    print("__device__ const double %s[%d][%d][%d] = {" % (name, len(rows), DEG64 + 1, NINT))
+    for tab in rows:
         print("    {")
-        for k in range(DEG64 + 1):
-            row = [float(tab[i][k]).hex() for i in range(NINT)]
+        for row in tab:
             print("        {" + ",\n         ".join(", ".join(row[j:j + 4])
                                                     for j in range(0, NINT, 4)) + "},")
         print("    },")
     print("};")
+
+
+def main64():
+    print("// Generated by gen_fftab.py fp64 (mpmath, 50 digits), degree %d in u = s - i on" % DEG64)
+    print("// |s - i| <= 1/2, as [function][degree][interval]: kFar64 the scaled local kernels")
+    print("// 1 - rho A_g, 1 - rho^3 B_g, 1 - rho^5 D_g (zero below interval %d, where they are" % FAR0)
+    print("// not used), kSmooth64 A_g, B_g, D_g, E_g.")
+    print("#pragma once")
+    print("#define GGEM_SMOOTH64_NINT %d" % NINT)
+    print("#define GGEM_SMOOTH64_DEG %d" % DEG64)
+
+    def rows(f, i0):
+        tab = [interpolant(f, i, DEG64) if i >= i0 else [mp.mpf(0)] * (DEG64 + 1)
+               for i in range(NINT)]
+        return [[float(tab[i][k]).hex() for i in range(NINT)] for k in range(DEG64 + 1)]
+    table64("kFar64", [rows(f, FAR0) for f in FAR])
+    table64("kSmooth64", [rows(f, 0) for f in FUNCS])
 
 
 if __name__ == "__main__":

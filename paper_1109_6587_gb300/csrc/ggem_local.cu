@@ -163,7 +163,7 @@ template <typename T> LocalConst<T> local_const(const GridGeom& geo, const CellG
     k.ke = (T)(-a * a * 1.4426950408889634074);
     const double s2 = 2.0 * a * a, lam = a * 1.4142135623730950488;
     k.s2 = (T)s2; k.lam = (T)lam; k.lam3 = (T)(s2 * lam); k.lam5 = (T)(s2 * s2 * lam);
-    // the tables end at s = 72.5, where the kernels are below 2e-17 of 1/r
+    // the tables end at s = 72.5, exp(-36) of the near field
     if (sizeof(T) == 8) k.rc2 = (T)std::min((double)k.rc2, (GGEM_SMOOTH64_NINT - 0.6) / s2);
     return k;
 }
@@ -287,16 +287,18 @@ __device__ __forceinline__ void pair_terms(const LocalConst<T>& k, T dx, T dy, T
     }
 }
 
-// Two of the smooth parts A_g, B_g (F = 0) or D_g, E_g (F = 2) at s = 2 alpha^2 r^2.
-// The coefficients come through L1 (12 KB for the two; 20 loads of at most five
-// lines per 32 pairs, against some 900 cycles of FP64 arithmetic).
-template <int F>
-__device__ __forceinline__ void smooth64(double s2, double r2, double& p, double& q) {
-    const double m = fma(r2, s2, 6755399441055744.0);     // nearest integer in the low bits
-    const int i = __double2loint(m) & 127;
-    const double u = fma(r2, s2, -(m - 6755399441055744.0));
-    const double* a = &kSmooth64[F][0][0] + i;
-    const double* b = &kSmooth64[F + 1][0][0] + i;
+// Interval of s = 2 alpha^2 r^2 and the remainder in it.
+__device__ __forceinline__ int interval64(const LocalConst<double>& k, double r2, double& u) {
+    const double m = fma(r2, k.s2, 6755399441055744.0);   // nearest integer in the low bits
+    u = fma(r2, k.s2, -(m - 6755399441055744.0));
+    return __double2loint(m);
+}
+
+// Two polynomials of the tables.  The coefficients come through L1 (12 KB for the
+// two; 20 loads of at most five lines per 32 pairs, against some 900 cycles of FP64
+// arithmetic).
+__device__ __forceinline__ void poly64(const double* a, const double* b, double u, double& p,
+                                       double& q) {
     constexpr int N = GGEM_SMOOTH64_NINT;
     p = __ldg(a + GGEM_SMOOTH64_DEG * N);
     q = __ldg(b + GGEM_SMOOTH64_DEG * N);
@@ -307,27 +309,39 @@ __device__ __forceinline__ void smooth64(double s2, double r2, double& p, double
     }
 }
 
-// The same terms in FP64, one output kind at a time: the singular parts 1/r, 1/r^3,
-// 1/r^5 and the smooth ones from tables, no exponential and no erfc.  The double
-// layer is summed over 6 (the caller multiplies), its last term's scalar E x.g in
-// a.sxx.  About 55 FP64 instructions per pair where exp and erfcx took about 95:
-// element rule, 1,296 targets, 40,960 points 3.2 -> 2.0 ms.
+// The same terms in FP64, one output kind at a time.  Near the target the singular
+// parts 1/r, 1/r^3, 1/r^5 less the smooth ones from tables, no exponential and no
+// erfc.  That difference loses digits as the kernels decay (3e-15 of them at s = 5,
+// 1e-14 at 8, 2e-10 at 32, r_cut = 4 / alpha), so A and B from interval 6 and D from
+// interval 4 on come from tables of the scaled kernels, times 1/r, 1/r^3, 1/r^5: below
+// 3e-15 everywhere but near the zero of A.  The two differ by selects only: the whole
+// double layer of the case below 1.831 -> 1.838 ms.  The double layer is summed over 6 (the caller
+// multiplies), its last term's scalar E x.g in a.sxx.  About 55 FP64 instructions
+// per pair where exp and erfcx took about 95: element rule, 1,296 targets,
+// 40,960 points 3.2 -> 2.0 ms.
 template <int MODE>
 __device__ __forceinline__ void pair_terms64(const LocalConst<double>& k, double dx, double dy,
                                              double dz, double r2, const double4_32a& g,
                                              double nx, double ny, double nz, PairAcc<double>& a) {
+    constexpr int F = MODE == OUT_U ? 0 : 2;
     const double ir = rsqrt(r2), ir2 = ir * ir;
     const double xg = fma(dz, g.z, fma(dy, g.y, dx * g.x));
-    double p, q;
+    double u, p, q;
+    const int i = interval64(k, r2, u);
+    const bool far = i >= (F == 0 ? 6 : 4);
+    const double* ta = (far ? &kFar64[F][0][0] : &kSmooth64[F][0][0]) + i;
+    const double* tb = (F == 0 && far ? &kFar64[1][0][0] : &kSmooth64[F + 1][0][0]) + i;
+    poly64(ta, tb, u, p, q);
     if (MODE == OUT_U) {
-        smooth64<0>(k.s2, r2, p, q);
-        const double A = fma(-k.lam, p, ir), B = fma(-k.lam3, q, ir2 * ir) * xg;
+        const double ir3 = ir2 * ir;
+        const double A = fma(far ? ir : -k.lam, p, far ? 0.0 : ir);
+        const double B = fma(far ? ir3 : -k.lam3, q, far ? 0.0 : ir3) * xg;
         a.ux = fma(B, dx, fma(A, g.x, a.ux));
         a.uy = fma(B, dy, fma(A, g.y, a.uy));
         a.uz = fma(B, dz, fma(A, g.z, a.uz));
     } else {
-        smooth64<2>(k.s2, r2, p, q);
-        const double D = fma(k.lam5, p, -(ir2 * ir2 * ir)), E = k.lam3 * q;      // over 6
+        const double ir5 = -(ir2 * ir2 * ir);
+        const double D = fma(far ? ir5 : k.lam5, p, far ? 0.0 : ir5), E = k.lam3 * q;   // over 6
         if (MODE == OUT_S) {
             // d_i (D xg d_k + E g_k) + E g_i d_k, and E xg on the diagonal
             const double Dx = D * xg, Ex = E * xg;
