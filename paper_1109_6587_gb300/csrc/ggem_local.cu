@@ -149,6 +149,7 @@ template <typename T> struct LocalConst {
     T al, al2, rc2, c1, c2, c3, c4, fU, fS, hx, hy, hz;
     T ke;   // -alpha^2 log2(e): exp(-alpha^2 r^2) = 2^(ke r^2)
     T s2, lam, lam3, lam5;   // FP64 tables: 2 alpha^2, powers of sqrt(2) alpha
+    bool beyond;             // r_cut reaches beyond the tables
 };
 
 template <typename T> LocalConst<T> local_const(const GridGeom& geo, const CellGrid& cg) {
@@ -163,8 +164,7 @@ template <typename T> LocalConst<T> local_const(const GridGeom& geo, const CellG
     k.ke = (T)(-a * a * 1.4426950408889634074);
     const double s2 = 2.0 * a * a, lam = a * 1.4142135623730950488;
     k.s2 = (T)s2; k.lam = (T)lam; k.lam3 = (T)(s2 * lam); k.lam5 = (T)(s2 * s2 * lam);
-    // the tables end at s = 72.5, exp(-36) of the near field
-    if (sizeof(T) == 8) k.rc2 = (T)std::min((double)k.rc2, (GGEM_SMOOTH64_NINT - 0.6) / s2);
+    k.beyond = s2 * geo.rcut * geo.rcut > GGEM_SMOOTH64_NINT - 0.6;
     return k;
 }
 
@@ -309,6 +309,14 @@ __device__ __forceinline__ void poly64(const double* a, const double* b, double 
     }
 }
 
+// The same beyond the tables (s > 72.5, exp(-36) of the near field): 1 - rho A_g and
+// 1 - rho^3 B_g (F = 0), or 1 - rho^5 D_g and E_g, at x = alpha r.
+template <int F> __device__ __noinline__ double2 beyond64(double x) {
+    const double ec = erfc(x), ex = exp(-x * x), w = 1.1283791670955125739 * x * ex;
+    if (F == 0) return make_double2(ec - w, ec + w);
+    return make_double2(fma(w, fma(x * x, 2.0 / 3.0, 1.0), ec), 0.13298076013381091 * ex);
+}
+
 // The same terms in FP64, one output kind at a time.  Near the target the singular
 // parts 1/r, 1/r^3, 1/r^5 less the smooth ones from tables, no exponential and no
 // erfc.  That difference loses digits as the kernels decay (3e-15 of them at s = 5,
@@ -323,15 +331,21 @@ template <int MODE>
 __device__ __forceinline__ void pair_terms64(const LocalConst<double>& k, double dx, double dy,
                                              double dz, double r2, const double4_32a& g,
                                              double nx, double ny, double nz, PairAcc<double>& a) {
-    constexpr int F = MODE == OUT_U ? 0 : 2;
+    constexpr int F = MODE == OUT_U ? 0 : 2, N = GGEM_SMOOTH64_NINT;
     const double ir = rsqrt(r2), ir2 = ir * ir;
     const double xg = fma(dz, g.z, fma(dy, g.y, dx * g.x));
     double u, p, q;
     const int i = interval64(k, r2, u);
     const bool far = i >= (F == 0 ? 6 : 4);
-    const double* ta = (far ? &kFar64[F][0][0] : &kSmooth64[F][0][0]) + i;
-    const double* tb = (F == 0 && far ? &kFar64[1][0][0] : &kSmooth64[F + 1][0][0]) + i;
-    poly64(ta, tb, u, p, q);
+    if (k.beyond && i >= N) {
+        const double2 e = beyond64<F>(k.al * (r2 * ir));
+        p = e.x;
+        q = e.y;
+    } else {
+        const double* ta = (far ? &kFar64[F][0][0] : &kSmooth64[F][0][0]) + i;
+        const double* tb = (F == 0 && far ? &kFar64[1][0][0] : &kSmooth64[F + 1][0][0]) + i;
+        poly64(ta, tb, u, p, q);
+    }
     if (MODE == OUT_U) {
         const double ir3 = ir2 * ir;
         const double A = fma(far ? ir : -k.lam, p, far ? 0.0 : ir);

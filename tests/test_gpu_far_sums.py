@@ -1,5 +1,6 @@
 """FP64 local sums at targets whose sources are all far away: the returned values have
-their digits.  Relative to the largest component: the kernels fall by
+their digits, also for a cutoff beyond the tables' end (6.02 / alpha), and no term
+within r_cut is left out.  Relative to the largest component: the kernels fall by
 2 alpha r per unit of alpha r, so positions good to a few 1e-15 of the box give 4e-14
 at most; bar 1e-13.  (Velocity and stress in one call take erfc's own route, 1e-13 up
 to 4 / alpha.)"""
@@ -37,7 +38,8 @@ def _pair(alpha, d, g):
 
 @pytest.mark.parametrize("quadrature", ["nodal", "element"])     # both search reaches
 @pytest.mark.parametrize("rf,ar", [(4.0, 1.3), (4.0, 1.6), (4.0, 1.7), (4.0, 2.9), (4.0, 3.95),
-                                   (6.5, 5.0), (6.5, 5.95), (6.5, 6.01)])
+                                   (6.5, 5.0), (6.5, 5.95), (6.5, 6.01), (6.5, 6.03),
+                                   (6.5, 6.45), (7.9, 7.8)])
 def test_far_pair(ggem, quadrature, rf, ar):
     box = W.Box(16.0, 16.0, 6.0, -3.0, 32, 33, 32)
     rng = np.random.default_rng(int(100 * ar))
