@@ -11,3 +11,13 @@ if ROOT not in sys.path:
 def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: needs a CUDA GPU (runs the sm_103a library)")
     config.addinivalue_line("markers", "slow: larger CPU oracle cases")
+
+
+@pytest.fixture(scope="session")
+def ggem():
+    """The binding, its library built."""
+    from paper_1109_6587_gb300 import _build
+
+    _build.build()
+    from paper_1109_6587_gb300 import ggem as G
+    return G

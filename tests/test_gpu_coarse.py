@@ -13,15 +13,6 @@ pytestmark = pytest.mark.gpu
 TOL_MIXED = 1e-5
 
 
-@pytest.fixture(scope="module")
-def ggem():
-    from paper_1109_6587_gb300 import _build
-
-    _build.build()
-    from paper_1109_6587_gb300 import ggem as G
-    return G
-
-
 def _layers(ggem, s, q, tg, quadrature, **kw):
     import torch
     P = ggem.Plan.for_box(s.box, precision="mixed", quadrature=quadrature, max_points=len(s.x),

@@ -15,15 +15,6 @@ pytestmark = pytest.mark.gpu
 TOL = 1e-13
 
 
-@pytest.fixture(scope="module")
-def ggem():
-    from paper_1109_6587_gb300 import _build
-
-    _build.build()
-    from paper_1109_6587_gb300 import ggem as G
-    return G
-
-
 def _pair(alpha, d, g):
     r = math.sqrt(float(d @ d))
     x, sp, xg = alpha * r, math.sqrt(math.pi), float(d @ g)
