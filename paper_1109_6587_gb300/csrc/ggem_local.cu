@@ -701,18 +701,12 @@ static void launch_kind(const LocalArgs<T>& a, int mode, int nsm, cudaStream_t s
     }
 }
 
-// the grid's search reach as a compile-time constant (cells >= r_cut/2 or
-// r_cut/3; grids of larger cells use reach 2)
+// the grid's search reach as a compile-time constant: 2 (cells >= r_cut/2, nodal
+// plans) or 3 (cells >= r_cut/3, element plans)
 template <typename T, int KIND>
 static void launch_kind(const LocalArgs<T>& a, int mode, int nsm, cudaStream_t st) {
     if (a.cg.reach == 3) launch_kind<T, KIND, 3>(a, mode, nsm, st);
     else launch_kind<T, KIND, 2>(a, mode, nsm, st);
-}
-
-template <int LAYER, int REACH>
-static void launch_elem(const LocalArgs<double>& a, cudaStream_t st) {
-    k_local<double, TK_POINTS, LAYER == 0 ? OUT_U : OUT_DBL, true, REACH, kSplit>
-        <<<a.n_tgt, kSplit * 32, 0, st>>>(a);
 }
 
 // Always four warps per target: the 16 points per triangle give each plenty of pairs, and
@@ -727,13 +721,9 @@ cudaError_t local_sum_elem(const GridGeom& geo, const CellGrid& cg,
     // the same candidate cells (L1 / L2 reuse); output in caller order
     LocalArgs<double> a{geo, cg, local_const<double>(geo, cg), src, qvs, near * near, tgt.n,
                         tgt.cell, tgt.pos, tgt.perm, nrm_tgt, out, out_stride};
-    if (cg.reach == 3) {
-        if (layer == 0) launch_elem<0, 3>(a, st);
-        else launch_elem<1, 3>(a, st);
-    } else {
-        if (layer == 0) launch_elem<0, 2>(a, st);
-        else launch_elem<1, 2>(a, st);
-    }
+    auto* kf = layer == 0 ? k_local<double, TK_POINTS, OUT_U, true, kElemReach, kSplit>
+                          : k_local<double, TK_POINTS, OUT_DBL, true, kElemReach, kSplit>;
+    kf<<<tgt.n, kSplit * 32, 0, st>>>(a);
     return cudaGetLastError();
 }
 
