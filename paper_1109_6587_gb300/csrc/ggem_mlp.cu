@@ -793,7 +793,7 @@ ggem_status ggem_mlp_train(ggem_plan_t* P, int n, const double* feat, const doub
             std::mt19937_64 rng(seed);
             if (init) {
                 GG_CUDA(cudaMemsetAsync(mom, 0, NSTAT * sizeof(double), st));
-                k_mlp_moments<<<2 * 152, 128, 0, st>>>(n, f, t, mom);
+                k_mlp_moments<<<2 * P->nsm, 128, 0, st>>>(n, f, t, mom);
                 std::vector<double> hm(NSTAT);
                 GG_CUDA(cudaMemcpyAsync(hm.data(), mom, NSTAT * sizeof(double),
                                         cudaMemcpyDeviceToHost, st));
