@@ -10,17 +10,17 @@
 // and each (target, cell) pair uses one of the lists: list 1 where the whole
 // cell is at least kFarEdges = 4 longest edges from the target, list 2 where it
 // also is at least kDimRadius / alpha away, list 0 elsewhere.  The rules
-// integrate the same product of the linear density and the kernel; over one triangle of edge h at distance d they differ by the
-// kernel's Taylor terms beyond degree 4, of order (0.6 h / d)^5, and the kernel
+// integrate the same product of the linear density and the kernel; over one
+// triangle of edge h at distance d they differ by the kernel's Taylor terms beyond degree 4, of order (0.6 h / d)^5, and the kernel
 // falls off as exp(-alpha^2 d^2) besides.  Measured in FP64 with N(0,1)
 // densities on suspensions of 642- and 162-node spheres and biconcave cells, h / r_cut
 // from 0.02 to 0.16, the whole double-layer sums differ by (rms, over the rms
 // sum) 0.3e-8 to 1.1e-8 at 5 edges, 1.0e-8 to 5.5e-8 at 4 and 2.7e-8 to 1.3e-7 at
-// 3.5: at 4 the difference stays below the unit rounding of FP32 (6e-8), while
-// two orders of summation differ by 2e-7 to 7e-7.  List 2 lives on the kernel's
+// 3.5, while two orders of summation differ by 2e-7 to 7e-7.  List 2 lives on the kernel's
 // decay: beyond kDimRadius = 3 the terms carry exp(-9), and with alpha h <= 0.33
 // the sums differ by 6e-10 to 2.3e-8 (2.8: up to 5.2e-8; alpha h = 0.5: 2.2e-7,
-// where the list is not used).  In candidates per target the lists halve the work of
+// where the list is not used).  Both as dispatched, by cells: 2e-8 to 8e-8 (rms),
+// single targets up to 2e-7 of the largest sum.  In candidates per target the lists halve the work of
 // dense suspensions and take a third off dilute ones.
 // Triangles large against r_cut keep list 0 only, each point in the cell that holds it
 // (kBinRadius).

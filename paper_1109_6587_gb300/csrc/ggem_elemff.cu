@@ -168,6 +168,8 @@ __global__ void __launch_bounds__(FW * 32, 6) k_local_elem_ff(FFArgs a) {
                          grid_diff(tz, ph.z, pl.z)};
         ff r2 = ff_norm(ff_sum3(ff_sqr(d[0]), ff_sqr(d[1]), ff_sqr(d[2])));
         ff g[3] = {{ph.w, pl.w}, {pg.x, pg.y}, {pg.z, pg.w}};
+        // (the tables end at s = 72.5, r = 6.02 / alpha: a longer r_cut is cut there,
+        // where the terms are exp(-36) of the near field that every sum holds too)
         const bool ok = (r2.hi < a.rc2.hi || (r2.hi == a.rc2.hi && r2.lo < a.rc2.lo)) &&
                         r2.hi > 0.f && r2.hi < (float)GGEM_FF_NINT - 0.5f;
         if (!ok) {
