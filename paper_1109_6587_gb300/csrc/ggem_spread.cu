@@ -319,7 +319,7 @@ cudaError_t spread(const GridGeom& geo, const CellGrid& cg, const double* yj, co
         // few pairs: share their planes between up to 4 warps, to 16 warps per SM.  The
         // stage with at most 1, 2, 4, 8, 16 parts (us): 162 sources in FP64 177, 111, 76, 64,
         // 75, in FP32 46, 31, 26, 22, 19; 648 sources 261, 169, 138, 142, 139 and 66, 44,
-        // 34, 28, 29; from 1,296 sources (four parts by the second bound) no difference
+        // 34, 28, 29; from 1,296 sources on the second bound decides
         const int parts = std::max(1, std::min(4, 16 * nsm / npairs));
         const dim3 g((unsigned)((npairs + WPB - 1) / WPB), (unsigned)parts);
         const size_t smem = WPB * pair_smem<T>(geo.Ny);
